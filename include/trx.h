@@ -27,7 +27,8 @@
  *   'T' for real data), diag in {'N','U'}; case-insensitive.
  * - The call is asynchronous on `stream` (a cudaStream_t; NULL is the legacy
  *   default stream) and returns once the work is enqueued. It allocates no
- *   device memory: the tensor-core FP32 path uses the handle's workspace.
+ *   device memory: the tensor-core paths use the handle's workspace (FP32
+ *   needs it, FP64 runs without it on the CUDA cores).
  * - Return codes: 0 on success; -i if the i-th BLAS argument is illegal
  *   (side=1, uplo=2, transa=3, diag=4, m=5, n=6, alpha=7, A=8, lda=9, B=10,
  *   ldb=11), checked before anything else and before the handle is used;
@@ -96,7 +97,13 @@ enum {
     TRX_OPT_GEMM = 2,      /* FP32 GEMM-update engine: 0 automatic, 1 CUDA
                               cores (FP32 FMA), 2 tensor cores (tcgen05,
                               split BF16 products of TRX_OPT_SPLIT terms,
-                              FP32 accumulation)                            */
+                              FP32 accumulation). FP64 updates: 1 keeps all
+                              of them on the CUDA cores (DFMA); 0 and 2 take
+                              the larger ones to the tensor cores where the
+                              workspace allows (64-bit fixed-point rows in
+                              eight BF16 digits, exact integer sums: error
+                              below 4 u |op(A)||B| per element, elements
+                              that cannot hold it computed by DFMA)        */
     TRX_OPT_GRAPH = 3,     /* 1 (default): replay the launch chain as a
                               cached CUDA graph; 0: launch directly         */
     TRX_OPT_PROFILE = 4,   /* 1: time every launch with CUDA events and
@@ -296,9 +303,10 @@ int trx_set_workspace(trx_handle_t handle, void* ptr, size_t bytes);
  * op is 'S' (TRSM) or 'M' (TRMM), for which side/m/n are the call's; 'Y' for
  * a call on a prepared factor (TRSM or TRMM, same side/m/n); or 'G' for a
  * tensor-core trx_sgemm_update, with m = M + K and n = N (side 'L').
- * Depends on the handle's options (the CUDA-core and FP64 paths need none,
- * except FP64 TRSM on the mixed engine, TRX_OPT_FP64_TRSM, which needs the
- * FP32 solve's).
+ * Depends on the handle's options (the CUDA-core path needs none; FP64 TRSM
+ * on the mixed engine, TRX_OPT_FP64_TRSM, needs the FP32 solve's). For the
+ * recursive FP64 calls it is what their updates on the tensor cores use; with
+ * less the call runs all its updates on the CUDA cores instead.
  * Returns 0 and sets *bytes, or an argument code as for the compute calls. */
 int trx_workspace_size(trx_handle_t handle, char op, char side, int64_t m,
                        int64_t n, int elem_bytes, size_t* bytes);

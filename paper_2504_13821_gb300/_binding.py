@@ -237,6 +237,19 @@ class Handle:
                "trx_set_workspace")
         self._ws, self._ws_bytes = ws, nbytes
 
+    def offer_workspace(self, nbytes: int):
+        """Grow the workspace to nbytes where that is possible: an FP64 call
+        uses it for its tensor-core updates and runs without it on the CUDA
+        cores (no growth under a stream capture, which cannot synchronise,
+        nor past the device's memory)."""
+        import torch
+        if nbytes <= self._ws_bytes or torch.cuda.is_current_stream_capturing():
+            return
+        try:
+            self.ensure_workspace(nbytes)
+        except torch.cuda.OutOfMemoryError:
+            pass
+
     def profile(self, reset: bool = False) -> dict:
         p = _Profile()
         _check(load_library().trx_get_profile(self._h, ctypes.byref(p), int(reset)),
@@ -301,7 +314,11 @@ def _call(op: str, side, uplo, trans, diag, alpha, A, B, handle=None, stream=Non
     b_ptr, ldb = _colmajor(B, "B")
     h = handle if handle is not None else default_handle(B.device)
     elem = B.element_size()
-    h.ensure_workspace(h.workspace_size("S" if op == "trsm" else "M", side, m, n, elem))
+    need = h.workspace_size("S" if op == "trsm" else "M", side, m, n, elem)
+    if elem == 4 or h.get_option(OPT_FP64_TRSM) > 0 and op == "trsm":
+        h.ensure_workspace(need)
+    else:
+        h.offer_workspace(need)
     if stream is None:
         stream = torch.cuda.current_stream(B.device)
     s_ptr = stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)

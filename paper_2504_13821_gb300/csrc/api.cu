@@ -267,6 +267,13 @@ bool use_tc(trx_handle_t h, int64_t k, bool trsm, int64_t nrhs) {
                        leaf_for(h->opt_leaf, k, trsm, (int)sizeof(T), nrhs));
 }
 
+// The FP64 tensor-core update folds gamma into a power-of-two scaling: it
+// takes a gamma of ordinary size (NaN and Inf: the DFMA update).
+bool oz_gamma_ok(double gamma) {
+    const double a = std::fabs(gamma);
+    return a >= 0x1p-200 && a <= 0x1p200;
+}
+
 template <typename T>
 struct Exec {
     trx_handle_t h;
@@ -281,6 +288,7 @@ struct Exec {
     __nv_bfloat16* w_lo2 = nullptr;
     int* dag_flags = nullptr;      // device-scheduled TRSM: block flags + task counter
     int* thin_scratch = nullptr;   // thin TRSM: task counter, stop word, block flags
+    void* oz_ws = nullptr;         // FP64 updates on the tensor cores: operand images
     cudaStream_t s;
     bool profile;
 
@@ -347,13 +355,23 @@ struct Exec {
                                            st.y1 > st.y0 ? &yo : nullptr);
                         cls = st.inv ? TRX_KERNEL_LEAF_TRSM : TRX_KERNEL_GEMM_TC;
                     } else {
+                        cls = TRX_KERNEL_GEMM_SIMT;
                         for (const TcGemm& g : st.gemms) {
+                            if constexpr (std::is_same<T, double>::value) {
+                                if (oz_ws && oz_gamma_ok(st.gamma) &&
+                                    oz_applies(h->opt_gemm, g.mlen, c.nrhs, g.klen)) {
+                                    e = launch_oz_update(c, g, st.beta, st.gamma, oz_ws, h->d_err,
+                                                         h->wait_ns, h->num_sms, s);
+                                    cls = TRX_KERNEL_GEMM_TC;
+                                    if (e != cudaSuccess) break;
+                                    continue;
+                                }
+                            }
                             e = launch_gemm_simt<T>(c, c.C, c.c_rs, c.c_cs, g.rc, g.mlen, g.rk,
                                                     g.klen, (T)st.beta, (T)st.gamma, s,
                                                     h->num_sms);
                             if (e != cudaSuccess) break;
                         }
-                        cls = TRX_KERNEL_GEMM_SIMT;
                     }
                     for (const TcGemm& g : st.gemms) {
                         if (st.dense) {      // rows of a triangular block: (i+1) 2n each
@@ -444,7 +462,7 @@ struct Exec {
 };
 
 struct GraphKey {
-    int op, elem, tc, b, slices, dag, thin;
+    int op, elem, tc, b, slices, dag, thin, oz;
     int64_t k, nrhs, a_rs, a_cs, c_rs, c_cs, unit;
     const void* A;
     const void* C;
@@ -671,6 +689,13 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
             }
         }
     }
+    // FP64: the larger updates on the tensor cores, where the handle's workspace
+    // holds their operand images (else the DFMA updates, which need none) and
+    // the call is one chain (column-panel branches would share the images)
+    if (std::is_same<T, double>::value && P == 1) {
+        const size_t need = oz_workspace(h->opt_gemm, k, ex.c.nrhs, b);
+        if (need > 0 && h->ws != nullptr && h->ws_bytes >= need) parts[0].oz_ws = h->ws;
+    }
     const int dense = trsm ? 0 : trmm_dense_mode(h->opt_trmm_dense, h->opt_leaf, plan.tc, k);
     Plan pre, body;
     pre.tc = body.tc = plan.tc;
@@ -757,7 +782,8 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
     key.unit = ex.c.unit;
     key.A = ex.c.A;
     key.C = ex.c.C;
-    key.ws = plan.tc ? h->ws : nullptr;
+    key.oz = parts[0].oz_ws != nullptr;
+    key.ws = plan.tc || key.oz ? h->ws : nullptr;
     key.planes = factor_planes ? f->m_hi : nullptr;
     key.alpha = (double)alpha;
     key.wait_ns = h->wait_ns;
@@ -1379,7 +1405,10 @@ int trx_workspace_size(trx_handle_t h, char op, char side, int64_t m, int64_t n,
         tc = true;
     }
     *bytes = (tc && k > 0 && nrhs > 0) ? ws_layout(k, nrhs, slices_for(h)).total : 0;
-    if (*bytes && o == 'S' && use_dag_mode(h->opt_trsm_dag, true, true, 4, k, nrhs))
+    const bool pair64 = o == 'M' && h->opt_fp64_trmm > 0 && k >= kPairMinK;
+    if (elem_bytes == 8 && (o == 'S' || o == 'M') && !mixed64 && !pair64 && k > 0 && nrhs > 0)
+        *bytes = oz_workspace(h->opt_gemm, k, nrhs, leaf_for(h->opt_leaf, k, o == 'S', 8, nrhs));
+    if (*bytes && (elem_bytes == 4 || mixed64) && o == 'S' && use_dag_mode(h->opt_trsm_dag, true, true, 4, k, nrhs))
         *bytes += dag_extra_bytes(k, nrhs, slices_for(h));
     return TRX_SUCCESS;
 }

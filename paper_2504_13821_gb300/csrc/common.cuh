@@ -22,6 +22,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <utility>
 #include <vector>
 
@@ -147,6 +148,26 @@ template <typename T>
 cudaError_t launch_gemm_simt(const Canon<T>& p, const T* Y, int64_t y_rs, int64_t y_cs,
                              int64_t rc, int64_t mlen, int64_t rk, int64_t klen, T beta,
                              T gamma, cudaStream_t s, int num_sms = 152);
+
+// FP64 updates on the tensor cores (gemm_oz.cu): the scratch of one update
+// of mlen x klen times klen x nrhs, and the update itself (rows
+// [g.rc, g.rc + g.mlen) from rows [g.rk, g.rk + g.klen) of C).
+size_t oz_update_bytes(int64_t mlen, int64_t nrhs, int64_t klen);
+struct TcGemm;
+cudaError_t launch_oz_update(const Canon<double>& p, const TcGemm& g, double beta, double gamma,
+                             void* ws, int* err, long long wait_ns, int num_sms, cudaStream_t s);
+// The pieces of an update that gemm_oz.cu left to the DFMA kernel: flag
+// (i / 32) * per_row + j / cols of row i and right-hand side j (swap: of
+// right-hand side i and row j) is non-zero.
+struct OzPieces {
+    const int* flags = nullptr;
+    int64_t per_row = 0;
+    int cols = 1;
+    bool swap = false;
+};
+cudaError_t launch_gemm_simt_pieces(const Canon<double>& p, int64_t rc, int64_t mlen, int64_t rk,
+                                    int64_t klen, double beta, double gamma,
+                                    const OzPieces& pieces, cudaStream_t s, int num_sms);
 
 // B := 0 over an m x n column-major block (alpha == 0 quick return).
 template <typename T>

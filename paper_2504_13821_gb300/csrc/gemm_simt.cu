@@ -32,7 +32,14 @@ struct GemmArgs {
     int64_t y_rs, y_cs;
     int64_t rc, mlen, rk, klen;
     T beta, gamma;
+    OzPieces pc;           // pc.flags: only the flagged pieces (null: everything)
 };
+
+// Whether output (i, j) belongs to a piece the tensor-core update left out.
+__device__ __forceinline__ bool flagged(const OzPieces& pc, int64_t i, int64_t j) {
+    const int64_t r = pc.swap ? j : i, c = pc.swap ? i : j;
+    return pc.flags[(r >> 5) * pc.per_row + c / pc.cols] != 0;
+}
 
 // TM x TM outputs per thread; tile BM = BN = 16 TM.
 template <typename T, int TM>
@@ -47,6 +54,15 @@ __global__ void __launch_bounds__(NT) gemm_simt_kernel(GemmArgs<T> g) {
     const int tx = tid % 16, ty = tid / 16;
     const int64_t i0 = (int64_t)blockIdx.y * BM;
     const int64_t j0 = (int64_t)blockIdx.x * BN;
+    if (g.pc.flags) {
+        // the tile's flags at the granularity of the smallest piece (8)
+        int any = 0;
+        for (int e = tid; e < (BM / 8) * (BN / 8); e += NT) {
+            const int64_t i = i0 + e / (BN / 8) * 8, j = j0 + e % (BN / 8) * 8;
+            if (i < g.mlen && j < p.nrhs) any |= flagged(g.pc, i, j);
+        }
+        if (!__syncthreads_or(any)) return;
+    }
     const bool a_row_fast = (p.a_rs == 1 || p.a_rs == -1);
     const bool y_row_fast = (g.y_rs == 1 || g.y_rs == -1);
 
@@ -116,7 +132,7 @@ __global__ void __launch_bounds__(NT) gemm_simt_kernel(GemmArgs<T> g) {
 #pragma unroll
         for (int v = 0; v < TM; ++v) {
             const int64_t gj = j0 + ty + 16 * v;
-            if (gj >= p.nrhs) continue;
+            if (gj >= p.nrhs || (g.pc.flags && !flagged(g.pc, gi, gj))) continue;
             T* c = p.C + (g.rc + gi) * p.c_rs + gj * p.c_cs;
             *c = g.beta * *c + g.gamma * acc[u][v];
         }
@@ -126,11 +142,12 @@ __global__ void __launch_bounds__(NT) gemm_simt_kernel(GemmArgs<T> g) {
 }  // namespace
 
 template <typename T>
-cudaError_t launch_gemm_simt(const Canon<T>& p, const T* Y, int64_t y_rs, int64_t y_cs,
-                             int64_t rc, int64_t mlen, int64_t rk, int64_t klen, T beta,
-                             T gamma, cudaStream_t s, int num_sms) {
+static cudaError_t launch_simt(const Canon<T>& p, const T* Y, int64_t y_rs, int64_t y_cs,
+                               int64_t rc, int64_t mlen, int64_t rk, int64_t klen, T beta,
+                               T gamma, const OzPieces& pieces, cudaStream_t s, int num_sms) {
     if (mlen <= 0 || p.nrhs <= 0) return cudaSuccess;
     GemmArgs<T> g;
+    g.pc = pieces;
     g.p = p;
     g.Y = Y;
     g.y_rs = y_rs;
@@ -153,6 +170,21 @@ cudaError_t launch_gemm_simt(const Canon<T>& p, const T* Y, int64_t y_rs, int64_
     if (tm == 1) return launch_kernel(gemm_simt_kernel<T, 1>, grid, dim3(NT), 0, s, g);
     if (tm == 2) return launch_kernel(gemm_simt_kernel<T, 2>, grid, dim3(NT), 0, s, g);
     return launch_kernel(gemm_simt_kernel<T, 4>, grid, dim3(NT), 0, s, g);
+}
+
+template <typename T>
+cudaError_t launch_gemm_simt(const Canon<T>& p, const T* Y, int64_t y_rs, int64_t y_cs,
+                             int64_t rc, int64_t mlen, int64_t rk, int64_t klen, T beta,
+                             T gamma, cudaStream_t s, int num_sms) {
+    return launch_simt<T>(p, Y, y_rs, y_cs, rc, mlen, rk, klen, beta, gamma, OzPieces{}, s,
+                          num_sms);
+}
+
+cudaError_t launch_gemm_simt_pieces(const Canon<double>& p, int64_t rc, int64_t mlen, int64_t rk,
+                                    int64_t klen, double beta, double gamma,
+                                    const OzPieces& pieces, cudaStream_t s, int num_sms) {
+    return launch_simt<double>(p, p.C, p.c_rs, p.c_cs, rc, mlen, rk, klen, beta, gamma, pieces, s,
+                               num_sms);
 }
 
 template cudaError_t launch_gemm_simt<float>(const Canon<float>&, const float*, int64_t, int64_t,

@@ -50,6 +50,7 @@ cudaError_t convert_configure();
 cudaError_t refine_configure();
 cudaError_t dag_configure();
 cudaError_t thin_configure();
+cudaError_t oz_configure();
 
 // Kernel attributes (dynamic shared-memory limits) for the current device:
 // run once per device by every handle's and the allocation-free entry's
@@ -69,6 +70,7 @@ cudaError_t leaf_configure_all() {
     if ((e = refine_configure()) != cudaSuccess) return e;
     if ((e = dag_configure()) != cudaSuccess) return e;
     if ((e = thin_configure()) != cudaSuccess) return e;
+    if ((e = oz_configure()) != cudaSuccess) return e;
     return tc_configure();
 }
 

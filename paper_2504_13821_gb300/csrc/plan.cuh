@@ -399,6 +399,32 @@ inline int thin_leaf_rows(int64_t opt, bool tc, bool trsm, int elem, int64_t k, 
     return nrhs <= kThinWideNrhs ? 2048 : 1024;
 }
 
+// FP64 updates on the tensor cores (gemm_oz.cu) in place of DFMA, when the
+// handle's workspace holds their operand images and TRX_OPT_GEMM is not 1 (CUDA
+// cores). The DFMA update takes its multiply-adds at 1.1 TFLOP/s, the
+// tensor-core one about 18 us of launches and fill plus its K steps one after
+// the other (0.065 us per element of K where few tiles run), so the line is
+// where the first exceeds the second. Measured (rows x right-hand sides x K,
+// us, DFMA / tensor cores): 256x200x256 39 / 35, 512x64x512 44 / 52,
+// 512x200x512 107 / 52, 512x1024x512 547 / 78, 2048x16x2048 152 / 150,
+// 1024x1024x1024 1804 / 143, 2048x4096x2048 28519 / 1002, 4096^3 109994 / 3380.
+constexpr int64_t kOzMaxK = 65024;       // its two-digit FP32 sums are exact up to here
+inline bool oz_applies(int64_t gemm_mode, int64_t mlen, int64_t nrhs, int64_t klen) {
+    if (gemm_mode == 1 || klen < 64 || klen > kOzMaxK) return false;
+    return 2.0 * (double)mlen * (double)nrhs * (double)klen >= 2e7 + 7.2e4 * (double)klen;
+}
+// Workspace of a call's tensor-core FP64 updates: the first one down the
+// recursion's left edge that applies is the largest (every other has fewer rows
+// and a shorter K). 0: none applies.
+inline size_t oz_workspace(int64_t gemm_mode, int64_t k, int64_t nrhs, int b) {
+    for (int64_t s = k; s > b;) {
+        const int64_t s1 = split_point(s, b);
+        if (oz_applies(gemm_mode, s - s1, nrhs, s1)) return oz_update_bytes(s - s1, nrhs, s1);
+        s = s1;
+    }
+    return 0;
+}
+
 inline bool use_tc_mode(int elem, int64_t gemm_mode, int64_t k, int b) {
     if (elem != 4 || gemm_mode == 1 || k <= b) return false;   // k <= b: one leaf, no update
     if (gemm_mode == 2) return k > b;

@@ -149,9 +149,16 @@ bool is_small(const trx_server_s* s, const Req& r) {
     return f.elem == 4 || (double)f.k * (double)f.k * nrhs <= kSmallFp64Work;
 }
 
+// Whether a request runs the recursive FP64 path (not an FP32-based engine).
+bool plain_fp64(const trx_server_s* s, const Req& r) {
+    return s->facs[r.fid].elem == 8 &&
+           !(upc(r.op) == 'S' ? s->cfg.fp64_corrections > 0 : s->cfg.fp64_trmm > 0);
+}
+
 // Device bytes a request holds while in flight: its right-hand side (and
 // result), plus the operand planes of a tensor-core FP32 call (three BF16
-// slices of the k x k triangle and of the k x nrhs right-hand side).
+// slices of the k x k triangle and of the k x nrhs right-hand side) or the
+// operand images of the recursive FP64 path's updates.
 size_t cost_bytes(const trx_server_s* s, const Req& r) {
     const Fac& f = s->facs[r.fid];
     const int64_t nrhs = upc(r.side) == 'L' ? r.n : r.m;
@@ -159,6 +166,10 @@ size_t cost_bytes(const trx_server_s* s, const Req& r) {
     if (r.op == 'R') b += (size_t)r.m * (size_t)r.n * 8;
     const bool tc_call = !is_small(s, r);
     const bool fp32_solve = f.elem == 4 || (upc(r.op) == 'S' && s->cfg.fp64_corrections > 0);
+    size_t images = 0;
+    if (tc_call && plain_fp64(s, r) &&
+        trx_workspace_size(s->handles[0], r.op, r.side, r.m, r.n, 8, &images) == TRX_SUCCESS)
+        b += images;
     if (tc_call && fp32_solve) b += 6 * (size_t)f.k * (size_t)(f.k + nrhs);
     return b;
 }
@@ -218,6 +229,10 @@ int launch_large(trx_server_t s, Req& r) {
     const char wop = r.op == 'R' ? 'S' : r.op;
     int rc = trx_workspace_size(s->handles[i], wop, r.side, r.m, r.n, f.elem, &need);
     if (rc == TRX_SUCCESS) rc = ensure_ws(s, i, need);
+    if (rc == TRX_ERR_ALLOC && plain_fp64(s, r)) {
+        cudaGetLastError();              // FP64 runs without: its updates stay on the DFMA kernel
+        rc = TRX_SUCCESS;
+    }
     if (rc != TRX_SUCCESS) return rc;
     cudaError_t e = cudaStreamWaitEvent(st, r.ready, 0);
     if (e != cudaSuccess) return fail(e, "wait");
