@@ -129,9 +129,11 @@ enum {
                               the diagonal term in FP32 in the epilogue),
                               replacing the leaf kernel and the recursion
                               levels below that size;
-                              -1 off; 0 = automatic (default: 1024 rows when
-                              the order is at least 1024 and TRX_OPT_LEAF
-                              is automatic, else off)                     */
+                              -1 off; 0 = automatic (default: with
+                              TRX_OPT_LEAF automatic and the 6-term split
+                              the whole recursion gathered by row into one
+                              launch; else 1024 rows from order 1024 on when
+                              TRX_OPT_LEAF is automatic, else off)        */
     TRX_OPT_RESIDUAL = 9,  /* residual of trx_strsm_refined: 0 (automatic)
                               or 2: float-float on the FP32 pipes (pairs of
                               floats, exact product split and two-sum,
@@ -645,7 +647,8 @@ const char* trx_last_error_detail(void);
  * 4 or 8, leaf as TRX_OPT_LEAF, gemm_mode as TRX_OPT_GEMM, trmm_dense as
  * TRX_OPT_TRMM_DENSE, trsm_tc_leaf as TRX_OPT_TRSM_TC_LEAF, thin_leaf as
  * TRX_OPT_THIN_LEAF (the recursion's plan: the whole-call thin solve of
- * TRX_OPT_THIN is not shown), op 'S' (TRSM) or 'M' (TRMM). Returns an
+ * TRX_OPT_THIN is not shown, nor that an automatic FP32 TRMM on the tensor
+ * cores runs its leaves and updates in one launch), op 'S' (TRSM) or 'M' (TRMM). Returns an
  * argument code, TRX_ERR_INVALID_VALUE if buf is too small, or 0. */
 int trx_debug_plan(char op, char side, char uplo, char transa, char diag, int64_t m, int64_t n,
                    int elem_bytes, int leaf, int gemm_mode, int trmm_dense, int trsm_tc_leaf,

@@ -696,7 +696,14 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
         const size_t need = oz_workspace(h->opt_gemm, k, ex.c.nrhs, b);
         if (need > 0 && h->ws != nullptr && h->ws_bytes >= need) parts[0].oz_ws = h->ws;
     }
-    const int dense = trsm ? 0 : trmm_dense_mode(h->opt_trmm_dense, h->opt_leaf, plan.tc, k);
+    // TRMM on the tensor cores with both sizes left automatic: the recursion's
+    // updates gathered by row into one launch (six-term split: its long K ranges
+    // are summed in FP32 by chunks; with fewer terms they would add up in TMEM)
+    const bool rows = !trsm && plan.tc && slices == 3 && h->opt_trmm_dense == 0 &&
+                      h->opt_leaf == 0;
+    const int dense = trsm   ? 0
+                      : rows ? kTrmmRowsDiag
+                             : trmm_dense_mode(h->opt_trmm_dense, h->opt_leaf, plan.tc, k);
     Plan pre, body;
     pre.tc = body.tc = plan.tc;
     body.tc_leaf = plan.tc_leaf;
@@ -725,6 +732,8 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
         th.trsm = trsm;
         th.alpha = (double)alpha;
         body.steps.push_back(th);
+    } else if (rows) {
+        plan_trmm_rows(body, k, (double)alpha);
     } else {
         make_plan(body, trsm, k, b, (double)alpha, /*conv_m=*/false, dense);
     }
@@ -790,7 +799,7 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
     key.pdl = (int)h->opt_pdl;
     key.tc_leaf = (int)plan.tc_leaf;
     key.panels = P;
-    key.dense = dense;
+    key.dense = rows ? -1 : dense;
     const std::string ks(reinterpret_cast<const char*>(&key), sizeof(key));
     ++h->tick;
     for (auto& g : h->graphs) {

@@ -184,6 +184,30 @@ inline void plan_trmm_levels(Plan& pl, int64_t k, int b, double alpha, bool dens
     }
 }
 
+// The same product with the recursion's updates gathered by row: a 128-row
+// tile's update from every block to its left is one K range from 0 to its own
+// last row, so the whole TRMM is one launch, longest rows first, C is read and
+// written once, and no level waits for the one before it. The sum of a row
+// runs over the same terms in 256-term chunks added in FP32, as inside one
+// update. Measured against the leaves and levels (us, order x right-hand
+// sides): 500 x 300 50 -> 33, 1000 x 100 57 -> 34, 1024 x 1024 equal, 4096 x 4096
+// 467 -> 353, 8192 x 40 239 -> 216, 16384 x 16384 17037 -> 16314; side R
+// 5000 x 3000 1059 -> 608; the error is 0.27-0.99 of theirs.
+inline void plan_trmm_rows(Plan& pl, int64_t k, double alpha) {
+    pl.steps.push_back(Step{kConvY});
+    Step d{kGemm};
+    d.tc = true;
+    d.dense = true;
+    d.beta = alpha;
+    d.gamma = alpha;
+    for (int64_t t = (k - 1) / 128 * 128; t >= 0; t -= 128) {
+        const int64_t mlen = std::min<int64_t>(128, k - t);
+        d.gemms.push_back(TcGemm{t, mlen, 0, round_up(t + mlen, 32)});
+    }
+    pl.steps.push_back(d);
+}
+constexpr int kTrmmRowsDiag = 128;   // diagonal blocks its operand planes carry densely
+
 // The whole launch sequence of one call: operand planes (tensor-core path),
 // then the recursion of Section 3.1.
 // dense > 0 (TRMM on the tensor-core path only): leaves of that many rows as
