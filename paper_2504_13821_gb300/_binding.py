@@ -243,7 +243,7 @@ class Handle:
         cores (no growth under a stream capture, which cannot synchronise,
         nor past the device's memory)."""
         import torch
-        if nbytes <= self._ws_bytes or torch.cuda.is_current_stream_capturing():
+        if torch.cuda.is_current_stream_capturing():
             return
         try:
             self.ensure_workspace(nbytes)
@@ -315,10 +315,11 @@ def _call(op: str, side, uplo, trans, diag, alpha, A, B, handle=None, stream=Non
     h = handle if handle is not None else default_handle(B.device)
     elem = B.element_size()
     need = h.workspace_size("S" if op == "trsm" else "M", side, m, n, elem)
-    if elem == 4 or h.get_option(OPT_FP64_TRSM) > 0 and op == "trsm":
-        h.ensure_workspace(need)
-    else:
-        h.offer_workspace(need)
+    if need > h._ws_bytes:
+        if elem == 4 or op == "trsm" and h.get_option(OPT_FP64_TRSM) > 0:
+            h.ensure_workspace(need)
+        else:
+            h.offer_workspace(need)
     if stream is None:
         stream = torch.cuda.current_stream(B.device)
     s_ptr = stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)

@@ -439,6 +439,14 @@ struct Exec {
                     bytes = 4.0 * ((double)tc.k * (tc.k + 1) / 2 + 2.0 * tc.k * tc.nrhs);
                     break;
                 }
+                case kOzTrmm:
+                    if constexpr (std::is_same<T, double>::value)
+                        e = launch_oz_trmm(c, st.alpha, oz_ws, h->d_err, h->wait_ns, h->num_sms,
+                                           s);
+                    cls = TRX_KERNEL_GEMM_TC;
+                    flops = (double)c.k * c.k * c.nrhs;
+                    bytes = 8.0 * ((double)c.k * (c.k + 1) / 2 + 2.0 * c.k * c.nrhs);
+                    break;
                 case kDag: {
                     __nv_bfloat16* const w3[3] = {w_hi, w_lo, w_lo2};
                     e = launch_trsm_dag(*reinterpret_cast<const Canon<float>*>(&c), pl, w3,
@@ -692,9 +700,15 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
     // FP64: the larger updates on the tensor cores, where the handle's workspace
     // holds their operand images (else the DFMA updates, which need none) and
     // the call is one chain (column-panel branches would share the images)
+    bool oz_trmm = false;
     if (std::is_same<T, double>::value && P == 1) {
-        const size_t need = oz_workspace(h->opt_gemm, k, ex.c.nrhs, b);
-        if (need > 0 && h->ws != nullptr && h->ws_bytes >= need) parts[0].oz_ws = h->ws;
+        const auto fits = [&](size_t need) {
+            return need > 0 && h->ws != nullptr && h->ws_bytes >= need;
+        };
+        oz_trmm = !trsm && h->opt_leaf == 0 && oz_gamma_ok((double)alpha) &&
+                  oz_trmm_applies(h->opt_gemm, k, ex.c.nrhs) &&
+                  fits(oz_trmm_bytes(k, ex.c.nrhs));
+        if (oz_trmm || fits(oz_workspace(h->opt_gemm, k, ex.c.nrhs, b))) parts[0].oz_ws = h->ws;
     }
     // TRMM on the tensor cores with both sizes left automatic: the recursion's
     // updates gathered by row into one launch (six-term split: its long K ranges
@@ -732,6 +746,10 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
         th.trsm = trsm;
         th.alpha = (double)alpha;
         body.steps.push_back(th);
+    } else if (oz_trmm) {
+        Step oz{kOzTrmm};
+        oz.alpha = (double)alpha;
+        body.steps.push_back(oz);
     } else if (rows) {
         plan_trmm_rows(body, k, (double)alpha);
     } else {
@@ -791,7 +809,7 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
     key.unit = ex.c.unit;
     key.A = ex.c.A;
     key.C = ex.c.C;
-    key.oz = parts[0].oz_ws != nullptr;
+    key.oz = parts[0].oz_ws == nullptr ? 0 : oz_trmm ? 2 : 1;
     key.ws = plan.tc || key.oz ? h->ws : nullptr;
     key.planes = factor_planes ? f->m_hi : nullptr;
     key.alpha = (double)alpha;
@@ -1416,7 +1434,10 @@ int trx_workspace_size(trx_handle_t h, char op, char side, int64_t m, int64_t n,
     *bytes = (tc && k > 0 && nrhs > 0) ? ws_layout(k, nrhs, slices_for(h)).total : 0;
     const bool pair64 = o == 'M' && h->opt_fp64_trmm > 0 && k >= kPairMinK;
     if (elem_bytes == 8 && (o == 'S' || o == 'M') && !mixed64 && !pair64 && k > 0 && nrhs > 0)
-        *bytes = oz_workspace(h->opt_gemm, k, nrhs, leaf_for(h->opt_leaf, k, o == 'S', 8, nrhs));
+        *bytes = o == 'M' && h->opt_leaf == 0 && oz_trmm_applies(h->opt_gemm, k, nrhs)
+                     ? oz_trmm_bytes(k, nrhs)
+                     : oz_workspace(h->opt_gemm, k, nrhs,
+                                    leaf_for(h->opt_leaf, k, o == 'S', 8, nrhs));
     if (*bytes && (elem_bytes == 4 || mixed64) && o == 'S' && use_dag_mode(h->opt_trsm_dag, true, true, 4, k, nrhs))
         *bytes += dag_extra_bytes(k, nrhs, slices_for(h));
     return TRX_SUCCESS;
@@ -1674,11 +1695,15 @@ int refine_fixed(trx_handle_t h, bool fp64_data, char side, char uplo, char tran
     const bool lowerI = lower != (transI == 'T');
     const size_t mn64 = align256((size_t)k * nr * 8), mn32 = align256((size_t)k * nr * 4);
     const size_t a32 = fp64_data ? align256((size_t)k * k * 4) : 0;
-    const size_t ap = align256(refine_pack_a_bytes(k, lowerI));
-    const size_t xp = align256(refine_pack_x_bytes(k, nr));
+    // the residual on the tensor cores (exact digit products, gemm_oz.cu), or in
+    // float-float on the FP32 pipes
+    const bool oz = oz_residual_applies(h->opt_gemm, k, nr);
+    const size_t ozb = oz ? align256(oz_residual_bytes(k, nr)) : 0;
+    const size_t ap = oz ? 0 : align256(refine_pack_a_bytes(k, lowerI));
+    const size_t xp = oz ? 0 : align256(refine_pack_x_bytes(k, nr));
     std::vector<int4> units, tiles;
     int64_t slots = 0;
-    refine_plan_units(k, lowerI, units, tiles, slots);     // counts (the table: on the device)
+    if (!oz) refine_plan_units(k, lowerI, units, tiles, slots);   // counts (the table: on the device)
     const size_t ub = align256((units.size() + tiles.size()) * sizeof(int4));
     const size_t pb = align256((size_t)slots * 64 * (size_t)nr * 8);
     // Orders up to the batched kernel's limit: every FP32 solve is one
@@ -1688,7 +1713,7 @@ int refine_fixed(trx_handle_t h, bool fp64_data, char side, char uplo, char tran
     const bool small = k <= kBatchMaxK;
     const int64_t npan = small ? (nr + 63) / 64 : 0;
     const size_t db = small ? align256((size_t)2 * npan * sizeof(BatchDesc)) + 256 : 0;
-    const size_t need = 3 * mn64 + mn32 + a32 + ap + xp + ub + pb + db;
+    const size_t need = 3 * mn64 + mn32 + a32 + ap + xp + ub + pb + db + ozb;
     int rc = refine_scratch(h, need, s);
     if (rc != TRX_SUCCESS) return rc;
     // The solves launch directly: their graph key would hold this call's
@@ -1713,6 +1738,7 @@ int refine_fixed(trx_handle_t h, bool fp64_data, char side, char uplo, char tran
     int4* Td = Ud + units.size();
     double* part = reinterpret_cast<double*>(tail + a32 + ap + xp + ub);
     BatchDesc* Dd = small ? reinterpret_cast<BatchDesc*>(tail + a32 + ap + xp + ub + pb) : nullptr;
+    void* Oz = tail + a32 + ap + xp + ub + pb + db;
     int* dcount = small ? reinterpret_cast<int*>(reinterpret_cast<char*>(Dd) + db - 256) : nullptr;
     const float* As = fp64_data ? A32 : static_cast<const float*>(A);
     const int64_t ldas = fp64_data ? k : lda;
@@ -1738,12 +1764,21 @@ int refine_fixed(trx_handle_t h, bool fp64_data, char side, char uplo, char tran
             e = left ? refine_cast_f32_f64(Bf, ldb, B64, k, k, nr, alpha, s)
                      : refine_transpose_f32_f64(Bf, ldb, B64, k, m, n, alpha, s);
     }
-    if (e == cudaSuccess)
+    // the residual's triangle in canonical order (an upper one reversed, X, B and
+    // R with it)
+    const Canon<float> c32 = canonicalize<float>('L', uplo, transI, diag, k, nr,
+                                                 static_cast<const float*>(A), lda, D32, k);
+    const Canon<double> c64 = canonicalize<double>('L', uplo, transI, diag, k, nr,
+                                                   static_cast<const double*>(A), lda, Xi, k);
+    const int64_t first_row = c64.c_rs < 0 ? k - 1 : 0;
+    if (e == cudaSuccess && oz)
+        e = fp64_data ? oz_residual_split_m(c64, Oz, s) : oz_residual_split_m(c32, Oz, s);
+    if (e == cudaSuccess && !oz)
         e = fp64_data ? refine_pack_a64(static_cast<const double*>(A), lda, k, lowerI,
                                         transI == 'T', unit, Ap, s)
                       : refine_pack_a(static_cast<const float*>(A), lda, k, lowerI, transI == 'T',
                                       unit, Ap, s);
-    if (e == cudaSuccess) e = refine_plan_units_device(k, lowerI, Ud, Td, s);
+    if (e == cudaSuccess && !oz) e = refine_plan_units_device(k, lowerI, Ud, Td, s);
     if (e == cudaSuccess && small) {
         std::vector<BatchDesc> dv((size_t)(2 * npan));
         for (int64_t q = 0; q < 2 * npan; ++q) {
@@ -1779,11 +1814,20 @@ int refine_fixed(trx_handle_t h, bool fp64_data, char side, char uplo, char tran
     if ((e = refine_cast_f32_f64(D32, k, Xi, k, k, nr, 1.0, s)) != cudaSuccess)
         return fail_cuda(e, "refine cast");
     for (int it = 0; it < corrections; ++it) {
-        e = refine_pack_x(Xi, nullptr, k, k, nr, Xp, s);
-        if (e == cudaSuccess)
-            e = refine_residual_packed(fp64_data ? 3 : 0, Ap, Xp, Ud, (int64_t)units.size(), Td,
-                                       (int64_t)tiles.size(), part, k, lowerI, B64, k, R64, k, nr,
-                                       h->d_err, h->wait_ns, s);
+        if (oz) {
+            const double *x = Xi + first_row, *b = B64 + first_row;
+            double* r = R64 + first_row;
+            e = fp64_data ? launch_oz_residual(c64, x, b, r, c64.c_rs, c64.c_cs, Oz, h->d_err,
+                                               h->wait_ns, h->num_sms, s)
+                          : launch_oz_residual(c32, x, b, r, c32.c_rs, c32.c_cs, Oz, h->d_err,
+                                               h->wait_ns, h->num_sms, s);
+        } else {
+            e = refine_pack_x(Xi, nullptr, k, k, nr, Xp, s);
+            if (e == cudaSuccess)
+                e = refine_residual_packed(fp64_data ? 3 : 0, Ap, Xp, Ud, (int64_t)units.size(),
+                                           Td, (int64_t)tiles.size(), part, k, lowerI, B64, k,
+                                           R64, k, nr, h->d_err, h->wait_ns, s);
+        }
         if (e == cudaSuccess) e = refine_cast_f64_f32(R64, k, D32, k, k, nr, s);
         if (e != cudaSuccess) return fail_cuda(e, "refine residual");
         if ((rc = solve32(false)) != TRX_SUCCESS) return rc;

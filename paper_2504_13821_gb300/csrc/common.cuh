@@ -149,25 +149,40 @@ cudaError_t launch_gemm_simt(const Canon<T>& p, const T* Y, int64_t y_rs, int64_
                              int64_t rc, int64_t mlen, int64_t rk, int64_t klen, T beta,
                              T gamma, cudaStream_t s, int num_sms = 152);
 
-// FP64 updates on the tensor cores (gemm_oz.cu): the scratch of one update
-// of mlen x klen times klen x nrhs, and the update itself (rows
-// [g.rc, g.rc + g.mlen) from rows [g.rk, g.rk + g.klen) of C).
-size_t oz_update_bytes(int64_t mlen, int64_t nrhs, int64_t klen);
+// FP64 on the tensor cores (gemm_oz.cu), each with its scratch: an update (rows
+// [g.rc, g.rc + g.mlen) of C from rows [g.rk, g.rk + g.klen)), the whole TRMM
+// C := alpha M C, and the residual R := B - M X with M (FP32 or FP64) split
+// once; X, B and R share their strides.
 struct TcGemm;
+size_t oz_update_bytes(int64_t mlen, int64_t nrhs, int64_t klen);
 cudaError_t launch_oz_update(const Canon<double>& p, const TcGemm& g, double beta, double gamma,
                              void* ws, int* err, long long wait_ns, int num_sms, cudaStream_t s);
-// The pieces of an update that gemm_oz.cu left to the DFMA kernel: flag
-// (i / 32) * per_row + j / cols of row i and right-hand side j (swap: of
-// right-hand side i and row j) is non-zero.
+size_t oz_trmm_bytes(int64_t k, int64_t nrhs);
+cudaError_t launch_oz_trmm(const Canon<double>& p, double alpha, void* ws, int* err,
+                           long long wait_ns, int num_sms, cudaStream_t s);
+size_t oz_residual_bytes(int64_t k, int64_t n);
+template <typename T>
+cudaError_t oz_residual_split_m(const Canon<T>& p, void* ws, cudaStream_t s);
+template <typename T>
+cudaError_t launch_oz_residual(const Canon<T>& p, const double* X, const double* B, double* R,
+                               int64_t c_rs, int64_t c_cs, void* ws, int* err, long long wait_ns,
+                               int num_sms, cudaStream_t s);
+// The pieces that these leave to the DFMA kernel, which adds gamma times their
+// sums to D: in segments of `seg` of K, flag (i / 32) * per_row + j / cols of row i
+// and right-hand side j (swap: of right-hand side i and row j) is non-zero.
+// tri: only M's strictly lower part counts.
 struct OzPieces {
     const int* flags = nullptr;
-    int64_t per_row = 0;
-    int cols = 1;
-    bool swap = false;
+    int64_t per_row = 0, per_seg = 0;
+    int cols = 1, seg = 0;
+    bool swap = false, tri = false;
 };
-cudaError_t launch_gemm_simt_pieces(const Canon<double>& p, int64_t rc, int64_t mlen, int64_t rk,
-                                    int64_t klen, double beta, double gamma,
-                                    const OzPieces& pieces, cudaStream_t s, int num_sms);
+template <typename TA>
+cudaError_t launch_gemm_simt_pieces(const TA* A, int64_t a_rs, int64_t a_cs, int64_t mlen,
+                                    int64_t klen, const double* Y, int64_t y_rs, int64_t y_cs,
+                                    int64_t nrhs, double gamma, double* D, int64_t d_rs,
+                                    int64_t d_cs, const OzPieces& pieces, cudaStream_t s,
+                                    int num_sms);
 
 // B := 0 over an m x n column-major block (alpha == 0 quick return).
 template <typename T>

@@ -36,7 +36,7 @@ inline int64_t split_point(int64_t s, int b) {
     return s1;
 }
 
-enum StepKind { kLeaf, kGemm, kConvM, kConvY, kConvYRows, kInvDiag, kInvCompact, kDag, kThin };
+enum StepKind { kLeaf, kGemm, kConvM, kConvY, kConvYRows, kInvDiag, kInvCompact, kDag, kThin, kOzTrmm };
 
 struct Step {
     StepKind kind;
@@ -425,17 +425,18 @@ inline int thin_leaf_rows(int64_t opt, bool tc, bool trsm, int elem, int64_t k, 
 
 // FP64 updates on the tensor cores (gemm_oz.cu) in place of DFMA, when the
 // handle's workspace holds their operand images and TRX_OPT_GEMM is not 1 (CUDA
-// cores). The DFMA update takes its multiply-adds at 1.1 TFLOP/s, the
-// tensor-core one about 18 us of launches and fill plus its K steps one after
-// the other (0.065 us per element of K where few tiles run), so the line is
-// where the first exceeds the second. Measured (rows x right-hand sides x K,
-// us, DFMA / tensor cores): 256x200x256 39 / 35, 512x64x512 44 / 52,
-// 512x200x512 107 / 52, 512x1024x512 547 / 78, 2048x16x2048 152 / 150,
-// 1024x1024x1024 1804 / 143, 2048x4096x2048 28519 / 1002, 4096^3 109994 / 3380.
-constexpr int64_t kOzMaxK = 65024;       // its two-digit FP32 sums are exact up to here
+// cores). The DFMA update takes about 0.75 TFLOP/s of its multiply-adds at these
+// sizes, and at least 0.075 us per element of K however narrow it is; the
+// tensor-core one 18 us of launches and fill plus 0.045 us per element of K. The
+// line is where the first exceeds the second. Measured (rows x right-hand sides
+// x K, us, DFMA / tensor cores): 128x200x128 13 / 23, 64x2048x64 21 / 21,
+// 256x200x256 37 / 27, 512x16x512 41 / 39, 512x64x512 41 / 39, 512x1024x512
+// 521 / 46, 1024x16x1024 78 / 58, 1024x1024x1024 1805 / 93, 2048x4096x2048 28567 /
+// 897, 4096^3 110049 / 3099.
 inline bool oz_applies(int64_t gemm_mode, int64_t mlen, int64_t nrhs, int64_t klen) {
-    if (gemm_mode == 1 || klen < 64 || klen > kOzMaxK) return false;
-    return 2.0 * (double)mlen * (double)nrhs * (double)klen >= 2e7 + 7.2e4 * (double)klen;
+    if (gemm_mode == 1 || klen < 64) return false;
+    return klen >= 600 ||
+           2.0 * (double)mlen * (double)nrhs * (double)klen >= 1.35e7 + 3.4e4 * (double)klen;
 }
 // Workspace of a call's tensor-core FP64 updates: the first one down the
 // recursion's left edge that applies is the largest (every other has fewer rows
@@ -447,6 +448,26 @@ inline size_t oz_workspace(int64_t gemm_mode, int64_t k, int64_t nrhs, int b) {
         s = s1;
     }
     return 0;
+}
+
+// The whole FP64 TRMM as one tensor-core product (launch_oz_trmm) in place of
+// the recursion's leaves and updates: from two leaves on (one leaf is one launch).
+// Measured (us, order x right-hand sides, recursion with DFMA / one product): 100 x
+// 100 43 / 43 (both the recursion), 128 x 16 42 / 31, 256 x 200 90 / 32, 1000 x 16
+// 396 / 69, 1000 x 200 495 / 79, 8192 x 100 10437 / 722, 4096 x 4096 59618 / 1985;
+// side R 1500 x 2500 6308 / 392.
+inline bool oz_trmm_applies(int64_t gemm_mode, int64_t k, int64_t nrhs) {
+    return gemm_mode != 1 && k >= 128 && nrhs >= 1;
+}
+
+// The residual of the refined solves (a fixed number of corrections) on the
+// tensor cores in place of the float-float one on the FP32 pipes: from order 128 on
+// (the smallest whose product has two tiles of K). Measured, the whole call with two
+// corrections (us, order x right-hand sides): 128 x 16 209 / 183, 300 x 64 735 / 644,
+// 700 x 16 498 / 279, 1000 x 100 698 / 365, 4096 x 16 1504 / 1041, 4096 x 256 3109 /
+// 1773; side R 200 x 2048 1390 / 710; the result's error 0.01-0.08 of the other's.
+inline bool oz_residual_applies(int64_t gemm_mode, int64_t k, int64_t nrhs) {
+    return gemm_mode != 1 && k >= 128 && nrhs >= 1;
 }
 
 inline bool use_tc_mode(int elem, int64_t gemm_mode, int64_t k, int b) {

@@ -151,3 +151,63 @@ def test_without_workspace_and_under_capture(trx):
     assert not np.array_equal(outs["fast"], outs["dfma"])
     for h in (dfma, fast, cap):
         h.close()
+
+
+@pytest.mark.parametrize("side,uplo,trans,diag", inputs.VARIANTS)
+def test_trmm_one_product(trx, side, uplo, trans, diag):
+    """The whole FP64 TRMM at tile, step and chunk edges (128 rows, 16, 192),
+    and across a scale segment (4096), against the oracle; repeatable."""
+    h = trx.Handle(0)
+    vi = inputs.VARIANTS.index((side, uplo, trans, diag))
+    sizes = [(128, 1), (129, 70), (191, 16), (257, 200), (640, 33)]
+    if vi in (0, 7, 10, 13):
+        sizes.append((4200, 9))
+    for k, nrhs in sizes:
+        m, n = (k, nrhs) if side == "L" else (nrhs, k)
+        out = [run_case("trmm", side, uplo, trans, diag, m, n, 1.5, np.float64,
+                        seed=inputs.variant_seed(k, vi), handle=h, lda_pad=1, ldb_pad=vi % 3)[2]
+               for _ in range(2)]
+        assert np.array_equal(*out)
+    assert h.check_device_error() == 0
+    h.close()
+
+
+def test_trmm_graded_columns(trx):
+    """Right-hand sides that grow over e^60 down the column: pieces the
+    fixed-point form cannot hold are computed from the kept original."""
+    k, n = 700, 96
+    A, B = inputs.problem("L", "L", k, n, seed=3, dtype=np.float64)
+    A = np.asfortranarray(np.where(np.isnan(A), 0.0, A) * k)
+    B = np.asfortranarray(B * np.exp(60.0 * np.arange(k) / k - 30.0)[:, None])
+    At, Bt = to_dev(A, "cuda:0"), to_dev(B, "cuda:0")
+    trx.trmm("L", "L", "N", "N", 1.0, At, Bt)
+    L, out = np.tril(A).astype(np.longdouble), Bt.cpu().numpy()
+    exact = L @ B.astype(np.longdouble)
+    mag = np.abs(L) @ np.abs(B).astype(np.longdouble)
+    assert np.all(np.abs(out - exact) <= k * U * mag)
+
+
+@pytest.mark.parametrize("side,uplo,trans,diag", inputs.VARIANTS)
+def test_refined_residual(trx, side, uplo, trans, diag):
+    """FP32 TRSM with fixed corrections: the backward error of the result is at
+    FP64 level (8 k u) with the tensor-core residual, and no larger than with the
+    float-float one (CUDA cores)."""
+    import oracle
+    k, nrhs = 300, 70
+    m, n = (k, nrhs) if side == "L" else (nrhs, k)
+    vi = inputs.VARIANTS.index((side, uplo, trans, diag))
+    A, B = inputs.problem(side, uplo, m, n, seed=inputs.variant_seed(k, vi), dtype=np.float32,
+                          poison_diag=(diag == "U"))
+    At, Bt = to_dev(A, "cuda:0"), to_dev(B, "cuda:0")
+    eta = []
+    for engine in (0, 1):
+        h = trx.Handle(0)
+        h.set_option(trx.OPT_GEMM, engine)
+        X = trx.trsm_refined_async(side, uplo, trans, diag, 1.5, At, Bt, corrections=2, handle=h)
+        torch.cuda.synchronize()
+        assert h.check_device_error() == 0
+        A64, B64 = np.asfortranarray(A.astype(np.float64)), np.asfortranarray(B.astype(np.float64))
+        eta.append(oracle.trsm_backward_error(side, uplo, trans, diag, 1.5, A64,
+                                              np.asfortranarray(X.cpu().numpy()), B64)["eta"])
+        h.close()
+    assert eta[0] <= 8 * k * U and eta[0] <= max(eta[1], 2 * U)
