@@ -364,20 +364,6 @@ __device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[W]) {
             : "r"(taddr));
     }
 }
-// All loads of the warp have landed; the registers pass through, so that no use
-// of them moves above the wait.
-__device__ __forceinline__ void tmem_wait_ld() {
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-template <int W>
-__device__ __forceinline__ void landed(float (&v)[W]) {
-#pragma unroll
-    for (int i = 0; i < W; i += 8)
-        asm volatile(""
-                     : "+f"(v[i]), "+f"(v[i + 1]), "+f"(v[i + 2]), "+f"(v[i + 3]), "+f"(v[i + 4]),
-                       "+f"(v[i + 5]), "+f"(v[i + 6]), "+f"(v[i + 7]));
-}
-
 template <int BN>
 struct Cfg {
     static constexpr int A_PLANE = BM * KS * 2, B_PLANE = BN * KS * 2;
@@ -646,7 +632,7 @@ __global__ void __launch_bounds__(NT, 1) oz_gemm_kernel(const __grid_constant__ 
                     float v[8];
                     tmem_ld(tq + c, v);
                     tmem_wait_ld();
-                    landed(v);
+                    tmem_landed(v);
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
                         if (col0 + c + u < p.cols && row_ok) {
@@ -682,10 +668,10 @@ __global__ void __launch_bounds__(NT, 1) oz_gemm_kernel(const __grid_constant__ 
                         tmem_ld(tq + 2 * BN + c, l4);
                         tmem_ld(tq + 3 * BN + c, l5);
                         tmem_wait_ld();
-                        landed(l2);
-                        landed(l3);
-                        landed(l4);
-                        landed(l5);
+                        tmem_landed(l2);
+                        tmem_landed(l3);
+                        tmem_landed(l4);
+                        tmem_landed(l5);
 #pragma unroll
                         for (int u = 0; u < W; ++u) {
                             long long x = T[c + u];
@@ -708,10 +694,10 @@ __global__ void __launch_bounds__(NT, 1) oz_gemm_kernel(const __grid_constant__ 
                         tmem_ld(tq + 6 * BN + c, l8);
                         tmem_ld(tq + 7 * BN + c, l9);
                         tmem_wait_ld();
-                        landed(l6);
-                        landed(l7);
-                        landed(l8);
-                        landed(l9);
+                        tmem_landed(l6);
+                        tmem_landed(l7);
+                        tmem_landed(l8);
+                        tmem_landed(l9);
 #pragma unroll
                         for (int u = 0; u < W; ++u) {
                             // carries of 256 from level 8 into 7 and from 7 into 6

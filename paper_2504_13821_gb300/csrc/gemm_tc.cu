@@ -81,7 +81,15 @@ struct Cfg {
     static constexpr int STAGE_BYTES = S * A_TILE + S * B_TILE;
     static constexpr int STAGES =
         (1024 + MAX_STAGES * STAGE_BYTES + 256 <= 227 * 1024) ? MAX_STAGES : 3;
-    static constexpr int TMEM_COLS = 2 * BN;
+    // The precise form's tiles below 256 columns: MMAs issued by the whole warp
+    // (umma_elected: one of 64 columns takes 48 clocks instead of the 128 that one
+    // lane needs to issue it) and the two accumulators of a chunk double buffered,
+    // for which tensor memory has room. At 256 columns an MMA takes 128 clocks
+    // either way and the kernel runs at the power limit; the denser issue measured
+    // 1-2 % slower there.
+    static constexpr bool WARP_ISSUE = S == 3 && BN < 256;
+    static constexpr int SETS = WARP_ISSUE ? 2 : 1;
+    static constexpr int TMEM_COLS = 2 * BN * SETS;
     static constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + 256;
     static_assert(SMEM_BYTES <= 227 * 1024, "ring does not fit in shared memory");
     static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) |
@@ -126,6 +134,7 @@ struct Params {
 constexpr int MAXG_SMALL = 4;
 template <int MG>
 struct ParamsT : Params {
+    static constexpr bool LONG = MG > MAXG_SMALL;
     int tile_start[MG + 1];
     TcGemm g[MG];
 };
@@ -158,18 +167,38 @@ __device__ bool wait_bounded(uint32_t bar, uint32_t parity, const Params& p, vol
     }
 }
 
+// The same for a whole warp (lane 0 waits where the phase is not there yet and the
+// others follow its verdict), with the fence that orders tensor-core work after it.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, const Params& p,
+                                          volatile int* abort, bool honour_abort = true) {
+    int w = mbar_try(bar, parity);
+    if (!__all_sync(0xffffffffu, w)) {
+        if ((threadIdx.x & 31) == 0) w = wait_bounded(bar, parity, p, abort, honour_abort);
+        w = __shfl_sync(0xffffffffu, w, 0);
+        if (!w) return false;
+    }
+    tc_fence_after();
+    return true;
+}
+
 struct Tile {
     int g, m, n;
 };
 
-// Round r of a CTA's tiles: the rounds run alternately forwards and backwards
-// over the CTAs, so where the tiles get shorter (a TRMM's rows, longest first)
-// a CTA that had a long one in one round has a short one in the next. 32 row
-// tiles x 16 column tiles on 152 CTAs: the busiest has 1.05 of the mean, in
-// plain order 1.29; rows of equal length are not affected.
-__device__ __forceinline__ int round_tile(int r) {
-    const int c = (r & 1) ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
-    return r * (int)gridDim.x + c;
+// The CTA's tile after tile t. A TRMM's rows (diag_beta, longest first) run in
+// rounds alternately forwards and backwards over the CTAs, so that a CTA that had
+// a long tile in one round has a short one in the next: 32 row tiles x 16 column
+// tiles on 152 CTAs, the busiest has 1.05 of the mean, in plain order 1.29. Only
+// launches with the long update list carry such rows; the short form's code is
+// kept free of it (in the 256-column kernel the registers it takes spill, which
+// measured 1.6 % on a TRSM at 16384).
+template <class PP>
+__device__ __forceinline__ int next_tile(const PP& p, int t) {
+    if (PP::LONG && p.diag_beta) {
+        const int g = (int)gridDim.x, r = t / g;
+        return (r + 1) * g + (g - 1 - (t - r * g));
+    }
+    return t + (int)gridDim.x;
 }
 
 // Tile t of the group: find its update (prefix sums), then raster the
@@ -177,13 +206,15 @@ __device__ __forceinline__ int round_tile(int r) {
 // time share operand rows and columns in L2.
 template <class PP>
 __device__ __forceinline__ Tile map_tile(const PP& p, int t) {
-    if (p.diag_beta) {
+    if (PP::LONG && p.diag_beta) {
         // one tile row per update, rows of similar length next to each other:
-        // bands of p.band of them, column by column
+        // bands of p.band of them, column by column. The bounds on g hold for any
+        // t: the update list lies in the constant bank, whose loads the compiler
+        // may move ahead of the test that t is a tile at all.
         const int band = t / (p.band * p.n_tiles_n), first = band * p.band;
-        const int gm = min(p.band, p.ngemms - first);
+        const int gm = max(1, min(p.band, p.ngemms - first));
         const int idx = t - band * p.band * p.n_tiles_n;
-        return Tile{first + idx % gm, 0, idx / gm};
+        return Tile{min(first + idx % gm, p.ngemms - 1), 0, idx / gm};
     }
     int lo = 0, hi = p.ngemms - 1;
     while (lo < hi) {
@@ -223,7 +254,9 @@ __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
     Smem* sm = reinterpret_cast<Smem*>(smem_raw + (ring - raw) + STAGES * STAGE_BYTES);
     volatile int* abort = &sm->abort;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = C::WARP_ISSUE ? __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0)
+                                   : (int)(threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(smem_u32(&sm->full[s]), 1);
@@ -258,7 +291,7 @@ __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
         // ---------------- TMA producer ----------------
         int stage = 0, issued = 0;
         uint32_t phase = 0;
-        for (int r = 0, t; (t = round_tile(r)) < p.total_tiles && !*abort; ++r) {
+        for (int t = blockIdx.x; t < p.total_tiles && !*abort; t = next_tile(p, t)) {
             const Tile ti = map_tile(p, t);
             const TcGemm& G = p.g[ti.g];
             const int nkb = (int)(G.klen / BK);
@@ -284,12 +317,54 @@ __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
             if (--stage < 0) { stage = STAGES - 1; phase ^= 1u; }
             wait_bounded(smem_u32(&sm->full[stage]), phase, p, abort, false);
         }
-    } else if (P && warp == 1 && lane == 0) {
+    } else if (C::WARP_ISSUE && warp == 1) {
+        // ---------------- MMA issuer, precise accumulation, whole warp ----------------
+        const uint32_t lead = elect_lane();
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+        int stage = 0, set = 0;
+        uint32_t phase = 0, acc_phase = 0;
+        const uint64_t a_ring = sdesc(ring), b_ring = sdesc(ring + S * A_TILE);
+        bool ok = true;
+        for (int t = blockIdx.x; ok && t < p.total_tiles && !*abort; t = next_tile(p, t)) {
+            const int nkb = (int)(p.g[map_tile(p, t).g].klen / BK);
+            for (int kb0 = 0; kb0 < nkb && ok; kb0 += CH) {
+                ok = warp_wait(smem_u32(&sm->acc_empty[set]), acc_phase ^ 1u, p, abort);
+                const uint32_t dbig = tm + (uint32_t)(set * 2 * BN), dsmall = dbig + BN;
+                const int kb1 = min(nkb, kb0 + CH);
+                for (int kb = kb0; kb < kb1 && ok; ++kb) {
+                    if (!(ok = warp_wait(smem_u32(&sm->full[stage]), phase, p, abort))) break;
+                    const uint64_t A = a_ring + (uint32_t)stage * (STAGE_BYTES >> 4);
+                    const uint64_t B = b_ring + (uint32_t)stage * (STAGE_BYTES >> 4);
+                    const uint32_t on = kb == kb0 ? 0u : 1u;
+#pragma unroll
+                    for (int kk = 0; kk < BK / 16; ++kk) {
+                        const uint64_t a0 = A + kk * 2, b0 = B + kk * 2;
+                        const uint64_t a1 = a0 + (A_TILE >> 4), b1 = b0 + (B_TILE >> 4);
+                        const uint64_t a2 = a1 + (A_TILE >> 4), b2 = b1 + (B_TILE >> 4);
+                        const uint32_t acc_on = kk == 0 ? on : 1u;
+                        umma_elected(dbig, a0, b0, C::IDESC, acc_on, lead);
+                        umma_elected(dsmall, a0, b1, C::IDESC, acc_on, lead);
+                        umma_elected(dsmall, a1, b0, C::IDESC, 1u, lead);
+                        umma_elected(dsmall, a0, b2, C::IDESC, 1u, lead);
+                        umma_elected(dsmall, a1, b1, C::IDESC, 1u, lead);
+                        umma_elected(dsmall, a2, b0, C::IDESC, 1u, lead);
+                    }
+                    umma_commit_elected(smem_u32(&sm->empty[stage]), lead);
+                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                }
+                if (!ok) break;
+                umma_commit_elected(smem_u32(&sm->acc_full[set]), lead);
+                if (++set == C::SETS) { set = 0; acc_phase ^= 1u; }
+            }
+        }
+        umma_commit_elected(smem_u32(&sm->drain), lead);
+        warp_wait(smem_u32(&sm->drain), 0, p, abort, false);
+    } else if (P && !C::WARP_ISSUE && warp == 1 && lane == 0) {
         // ---------------- MMA issuer, precise accumulation ----------------
         int stage = 0;
         uint32_t phase = 0, acc_phase = 0;
         const uint32_t dbig = tmem, dsmall = tmem + BN;
-        for (int r = 0, t; (t = round_tile(r)) < p.total_tiles && !*abort; ++r) {
+        for (int t = blockIdx.x; t < p.total_tiles && !*abort; t = next_tile(p, t)) {
             const Tile ti = map_tile(p, t);
             const int nkb = (int)(p.g[ti.g].klen / BK);
             bool ok = true;
@@ -344,8 +419,9 @@ __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
         // warp w: TMEM lanes 32 (w % 4) .., columns [half * HC, half * HC + HC)
         constexpr int HC = BN / 2;
         const int q = warp & 3, half = (warp - 2) >> 2;
+        int set = 0;
         uint32_t acc_phase = 0;
-        for (int r = 0, t; (t = round_tile(r)) < p.total_tiles; ++r) {
+        for (int t = blockIdx.x; t < p.total_tiles; t = next_tile(p, t)) {
             const Tile ti = map_tile(p, t);
             const TcGemm& G = p.g[ti.g];
             const int nkb = (int)(G.klen / BK);
@@ -363,14 +439,14 @@ __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
             bool ok = true;
             for (int kb0 = 0; kb0 < nkb; kb0 += CH) {
                 int w = 1;
-                if (lane == 0) w = wait_bounded(smem_u32(&sm->acc_full[0]), acc_phase, p, abort);
+                if (lane == 0) w = wait_bounded(smem_u32(&sm->acc_full[set]), acc_phase, p, abort);
                 w = __shfl_sync(0xffffffffu, w, 0);
                 if (!w) { ok = false; break; }
                 tc_fence_after();
 #pragma unroll
                 for (int cc = 0; cc < HC / 16; ++cc) {
                     float v[16];
-                    const uint32_t ta = tmem + (uint32_t)(half * HC + cc * 16) +
+                    const uint32_t ta = tmem + (uint32_t)(set * 2 * BN + half * HC + cc * 16) +
                                         ((uint32_t)(q * 32) << 16);
                     tmem_ld16(ta, v);
 #pragma unroll
@@ -383,8 +459,8 @@ __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&sm->acc_empty[0]));
-                acc_phase ^= 1u;
+                if (lane == 0) mbar_arrive(smem_u32(&sm->acc_empty[set]));
+                if (++set == C::SETS) { set = 0; acc_phase ^= 1u; }
             }
             if (!ok) break;
             // C := beta C + gamma sum over this thread's row and columns
@@ -420,7 +496,7 @@ __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
         // ---------------- MMA issuer ----------------
         int stage = 0, acc = 0;
         uint32_t phase = 0, acc_phase = 0;
-        for (int r = 0, t; (t = round_tile(r)) < p.total_tiles && !*abort; ++r) {
+        for (int t = blockIdx.x; t < p.total_tiles && !*abort; t = next_tile(p, t)) {
             const Tile ti = map_tile(p, t);
             const int nkb = (int)(p.g[ti.g].klen / BK);
             if (!wait_bounded(smem_u32(&sm->acc_empty[acc]), acc_phase ^ 1u, p, abort)) break;
@@ -466,7 +542,7 @@ __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
         const int q = warp & 3;                 // TMEM lanes 32q .. 32q+31
         int acc = 0;
         uint32_t acc_phase = 0;
-        for (int r = 0, t; (t = round_tile(r)) < p.total_tiles; ++r) {
+        for (int t = blockIdx.x; t < p.total_tiles; t = next_tile(p, t)) {
             const Tile ti = map_tile(p, t);
             const TcGemm& G = p.g[ti.g];
             const int64_t row = (int64_t)ti.m * BM + q * 32 + lane;
@@ -708,7 +784,7 @@ cudaError_t launch_gemm_tc(const Canon<float>& p, const void* maps, int slices,
         const int grid = (int)(tiles < num_sms ? tiles : num_sms);
         cudaError_t e;
         static thread_local ParamsT<MAXG_SMALL> prm_small;
-        const bool small = ng <= MAXG_SMALL;
+        const bool small = ng <= MAXG_SMALL && !diag_beta;
         if (small) {
             static_cast<Params&>(prm_small) = static_cast<const Params&>(prm);
             for (int i = 0; i <= ng; ++i) prm_small.tile_start[i] = prm.tile_start[i];
