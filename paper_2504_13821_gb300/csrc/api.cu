@@ -156,6 +156,12 @@ WsLayout ws_layout(int64_t k, int64_t nrhs, int slices) {
     return w;
 }
 
+// Leading dimension and bytes of B^T (side R turned, turn_applies), k rows.
+int64_t turn_ld(int64_t k) { return round_up(k, 4); }
+size_t turn_bytes(int64_t k, int64_t nrhs) {
+    return align256((size_t)nrhs * turn_ld(k) * 4);
+}
+
 // Extra workspace of the device-scheduled TRSM after the planes: the
 // diagonal blocks' inverses as `slices` compact k x 128 planes, then the
 // block flags and the task counter.
@@ -288,6 +294,10 @@ struct Exec {
     __nv_bfloat16* w_lo2 = nullptr;
     int* dag_flags = nullptr;      // device-scheduled TRSM: block flags + task counter
     int* thin_scratch = nullptr;   // thin TRSM: task counter, stop word, block flags
+    // side R solved on B^T: B and its transpose in the workspace
+    float *turn_b = nullptr, *turn_t = nullptr;
+    int64_t turn_ldb = 0, turn_ldt = 0;
+    bool turn_flip = false;
     void* oz_ws = nullptr;         // FP64 updates on the tensor cores: operand images
     cudaStream_t s;
     bool profile;
@@ -439,6 +449,18 @@ struct Exec {
                     bytes = 4.0 * ((double)tc.k * (tc.k + 1) / 2 + 2.0 * tc.k * tc.nrhs);
                     break;
                 }
+                case kTurnIn:
+                    e = launch_turn(turn_b, turn_ldb, turn_t, turn_ldt, c.nrhs, c.k, false,
+                                    turn_flip, s);
+                    cls = TRX_KERNEL_CONVERT;
+                    bytes = 8.0 * c.k * c.nrhs;
+                    break;
+                case kTurnOut:
+                    e = launch_turn(turn_t, turn_ldt, turn_b, turn_ldb, c.k, c.nrhs, turn_flip,
+                                    false, s);
+                    cls = TRX_KERNEL_CONVERT;
+                    bytes = 8.0 * c.k * c.nrhs;
+                    break;
                 case kOzTrmm:
                     if constexpr (std::is_same<T, double>::value)
                         e = launch_oz_trmm(c, st.alpha, oz_ws, h->d_err, h->wait_ns, h->num_sms,
@@ -478,7 +500,8 @@ struct GraphKey {
     const void* planes;
     double alpha;
     long long wait_ns;
-    int pdl, panels, dense, tc_leaf;
+    int pdl, panels, dense, tc_leaf, turn;
+    int64_t turn_ldb;
 };
 
 }  // namespace
@@ -624,6 +647,21 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
             return TRX_ERR_WORKSPACE;
         }
         char* base = static_cast<char*>(h->ws);
+        if constexpr (std::is_same<T, float>::value) {
+            if (upc(side) == 'R' && !dag && !plan.thin_leaf && h->opt_panels <= 1 &&
+                turn_applies(k, ex.c.nrhs) &&
+                h->ws_bytes >= need + turn_bytes(k, ex.c.nrhs)) {
+                ex.turn_b = B;
+                ex.turn_ldb = ldb;
+                ex.turn_t = reinterpret_cast<float*>(base + need);
+                ex.turn_ldt = turn_ld(k);
+                // the canonical problem's own C: rows contiguous and in its order
+                ex.turn_flip = ex.c.c_rs < 0;
+                ex.c.c_rs = 1;
+                ex.c.c_cs = ex.turn_ldt;
+                ex.c.C = ex.turn_t;
+            }
+        }
         ex.pl.ldm = w.ldm;
         ex.pl.ldy = w.ldy;
         ex.pl.slices = slices;
@@ -722,6 +760,7 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
     pre.tc = body.tc = plan.tc;
     body.tc_leaf = plan.tc_leaf;
     body.thin_leaf = plan.thin_leaf;
+    if (ex.turn_t) pre.steps.push_back(Step{kTurnIn});
     if (plan.tc && !factor_planes) {
         Step cm{kConvM};
         cm.b = dense;
@@ -755,6 +794,7 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
     } else {
         make_plan(body, trsm, k, b, (double)alpha, /*conv_m=*/false, dense);
     }
+    if (ex.turn_t) body.steps.push_back(Step{kTurnOut});
     if (h->opt_checked) {
         if (const char* why = validate_plan(body, k)) {
             snprintf(g_detail, sizeof(g_detail), "checked plan: %s", why);
@@ -808,7 +848,9 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
     key.c_cs = ex.c.c_cs;
     key.unit = ex.c.unit;
     key.A = ex.c.A;
-    key.C = ex.c.C;
+    key.C = ex.turn_t ? B : ex.c.C;      // the caller's array: replays write it
+    key.turn = ex.turn_t ? 1 + ex.turn_flip : 0;
+    key.turn_ldb = ex.turn_ldb;
     key.oz = parts[0].oz_ws == nullptr ? 0 : oz_trmm ? 2 : 1;
     key.ws = plan.tc || key.oz ? h->ws : nullptr;
     key.planes = factor_planes ? f->m_hi : nullptr;
@@ -1421,6 +1463,8 @@ int trx_workspace_size(trx_handle_t h, char op, char side, int64_t m, int64_t n,
         *bytes = (tc && k > 0 && nrhs > 0) ? (size_t)sl * ws_layout(k, nrhs, sl).y_bytes : 0;
         if (tc_s && k > 0 && nrhs > 0 && use_dag_mode(h->opt_trsm_dag, true, true, 4, k, nrhs))
             *bytes += dag_extra_bytes(k, nrhs, sl);
+        if (*bytes && upc(side) == 'R' && turn_applies(k, nrhs))
+            *bytes += turn_bytes(k, nrhs);
         return TRX_SUCCESS;
     }
     // FP64 TRSM on the mixed engine solves in FP32: that call's planes
@@ -1440,6 +1484,9 @@ int trx_workspace_size(trx_handle_t h, char op, char side, int64_t m, int64_t n,
                                     leaf_for(h->opt_leaf, k, o == 'S', 8, nrhs));
     if (*bytes && (elem_bytes == 4 || mixed64) && o == 'S' && use_dag_mode(h->opt_trsm_dag, true, true, 4, k, nrhs))
         *bytes += dag_extra_bytes(k, nrhs, slices_for(h));
+    if (*bytes && elem_bytes == 4 && (o == 'S' || o == 'M') && upc(side) == 'R' &&
+        turn_applies(k, nrhs))
+        *bytes += turn_bytes(k, nrhs);
     return TRX_SUCCESS;
 }
 

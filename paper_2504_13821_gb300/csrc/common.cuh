@@ -188,6 +188,11 @@ cudaError_t launch_gemm_simt_pieces(const TA* A, int64_t a_rs, int64_t a_cs, int
 template <typename T>
 cudaError_t launch_zero(T* B, int64_t m, int64_t n, int64_t ldb, cudaStream_t s);
 
+// dst := src^T, src rows x cols, column-major (at most 64 * 65535 columns), its
+// rows or columns in reverse order on request.
+cudaError_t launch_turn(const float* src, int64_t lds, float* dst, int64_t ldd, int64_t rows,
+                        int64_t cols, bool flip_rows, bool flip_cols, cudaStream_t s);
+
 // Split-BF16 planes of the strictly-lower part of M (rows/cols [0,k)).
 // diag_block > 0 (a multiple of 64): the planes also carry zeros on and
 // above the diagonal within each diag_block x diag_block diagonal block.

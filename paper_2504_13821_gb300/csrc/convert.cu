@@ -103,6 +103,36 @@ __global__ void __launch_bounds__(256) convert_m_kernel(Canon<float> p, Planes p
     }
 }
 
+// dst := src^T (src rows x cols, both column-major), its rows or columns in reverse
+// order: dst(j', i') = src(i, j), i' = rows-1-i with flip_rows, j' = cols-1-j with
+// flip_cols. 64x64 tiles through shared memory, all of a thread's sixteen loads
+// issued before its first shared store.
+__global__ void __launch_bounds__(256) turn_kernel(const float* src, int64_t lds, float* dst,
+                                                   int64_t ldd, int64_t rows, int64_t cols,
+                                                   int flip_rows, int flip_cols) {
+    pdl_trigger();
+    pdl_wait();
+    __shared__ float tile[64][65];
+    const int64_t i0 = (int64_t)blockIdx.x * 64, j0 = (int64_t)blockIdx.y * 64;
+    const int x = threadIdx.x & 63, y = threadIdx.x >> 6;
+    float v[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+        const int64_t i = i0 + x, j = j0 + y + 4 * u;
+        v[u] = i < rows && j < cols ? src[i + j * lds] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < 16; ++u) tile[x][y + 4 * u] = v[u];
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+        const int64_t i = i0 + y + 4 * u, j = j0 + x;
+        if (i < rows && j < cols)
+            dst[(flip_cols ? cols - 1 - j : j) + (flip_rows ? rows - 1 - i : i) * ldd] =
+                tile[y + 4 * u][x];
+    }
+}
+
 // Y planes when C's rows are contiguous (side L): no transpose, four
 // consecutive rows per thread, 8-byte stores.
 __global__ void __launch_bounds__(256) convert_y_contig_kernel(Canon<float> p, Planes pl) {
@@ -241,6 +271,14 @@ __global__ void zero_kernel(T* B, int64_t m, int64_t n, int64_t ldb) {
 }
 
 }  // namespace
+
+cudaError_t launch_turn(const float* src, int64_t lds, float* dst, int64_t ldd, int64_t rows,
+                        int64_t cols, bool flip_rows, bool flip_cols, cudaStream_t s) {
+    const int64_t gx = (rows + 63) / 64, gy = (cols + 63) / 64;
+    if (gy > 65535) return cudaErrorInvalidValue;
+    return launch_kernel(turn_kernel, dim3((unsigned)gx, (unsigned)gy), dim3(256), 0, s, src, lds,
+                         dst, ldd, rows, cols, (int)flip_rows, (int)flip_cols);
+}
 
 cudaError_t launch_convert_m(const Canon<float>& p, const Planes& pl, int diag_block,
                              cudaStream_t s) {

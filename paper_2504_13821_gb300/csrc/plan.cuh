@@ -36,7 +36,8 @@ inline int64_t split_point(int64_t s, int b) {
     return s1;
 }
 
-enum StepKind { kLeaf, kGemm, kConvM, kConvY, kConvYRows, kInvDiag, kInvCompact, kDag, kThin, kOzTrmm };
+enum StepKind { kLeaf, kGemm, kConvM, kConvY, kConvYRows, kInvDiag, kInvCompact, kDag, kThin, kOzTrmm,
+                kTurnIn, kTurnOut };
 
 struct Step {
     StepKind kind;
@@ -421,6 +422,20 @@ inline int thin_leaf_rows(int64_t opt, bool tc, bool trsm, int elem, int64_t k, 
     if (k < kThinLeafMinK || nrhs <= kThinMaxNrhs || nrhs > 1024) return 0;
     if (nrhs <= 128 && k < 2 * kThinLeafMinK) return 0;
     return nrhs <= kThinWideNrhs ? 2048 : 1024;
+}
+
+// Side R on the FP32 tensor-core chain: B^T in the workspace. The leaves' panels
+// and the updates' epilogues have a lane per row of C, which for side R lie ldb
+// apart in B: each lane's access is a line of its own. With room for k x nrhs floats
+// past the planes, B is turned into the workspace, solved there and turned back (in
+// the canonical order, so a reversed problem's rows run forwards too). The two
+// passes cost 16 bytes an element. Measured (us, nrhs x order, in place / turned):
+// TRSM 256 x 256 53 / 51, 600 x 300 58 / 52, 600 x 600 148 / 123, 2000 x 2000 628 /
+// 441, 4096 x 4096 1343 / 945, 8192 x 8192 5375 / 3813; TRMM 500 x 300 31 / 31,
+// 1000 x 1000 56 / 42, 3000 x 5000 609 / 432. Below 2^16 elements nothing is gained.
+constexpr int64_t kTurnMinElements = (int64_t)1 << 16;
+inline bool turn_applies(int64_t k, int64_t nrhs) {
+    return k * nrhs >= kTurnMinElements && k <= 64 * 65535ll && nrhs <= 64 * 65535ll;
 }
 
 // FP64 updates on the tensor cores (gemm_oz.cu) in place of DFMA, when the

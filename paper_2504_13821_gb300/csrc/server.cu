@@ -171,6 +171,8 @@ size_t cost_bytes(const trx_server_s* s, const Req& r) {
         trx_workspace_size(s->handles[0], r.op, r.side, r.m, r.n, 8, &images) == TRX_SUCCESS)
         b += images;
     if (tc_call && fp32_solve) b += 6 * (size_t)f.k * (size_t)(f.k + nrhs);
+    if (tc_call && f.elem == 4 && r.op != 'R' && upc(r.side) == 'R')
+        b += 4 * (size_t)f.k * (size_t)nrhs;           // B's transpose
     return b;
 }
 
