@@ -45,6 +45,13 @@ __device__ __forceinline__ void pdl_wait() {
 // TRX_OPT_PDL, set around each call).
 bool& pdl_enabled();
 
+// Launches with the attribute while it lives, whatever the option says.
+struct PdlScope {
+    bool saved;
+    PdlScope() : saved(pdl_enabled()) { pdl_enabled() = true; }
+    ~PdlScope() { pdl_enabled() = saved; }
+};
+
 template <typename... KArgs, typename... Args>
 cudaError_t launch_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
                           cudaStream_t s, Args&&... args) {

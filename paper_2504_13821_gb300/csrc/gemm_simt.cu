@@ -298,6 +298,10 @@ cudaError_t launch_gemm_simt_pieces(const TA* A, int64_t a_rs, int64_t a_cs, int
     const int64_t gy = (mlen + 16 * tm - 1) / (16 * tm), gx = (nrhs + 16 * tm - 1) / (16 * tm);
     if (gy > 65535) return cudaErrorInvalidValue;
     const dim3 grid((unsigned)gx, (unsigned)gy);
+    // its launch overlaps the tensor-core update's tail (it waits for that kernel
+    // before it reads a flag): 2 us less an update. The same on the update itself,
+    // over the operand split, gained 3 us alone and lost 1-2 % inside launch graphs.
+    const PdlScope overlap;
     if (tm == 1) return launch_kernel(gemm_pieces_kernel<TA, 1>, grid, dim3(NT), 0, s, g);
     if (tm == 2) return launch_kernel(gemm_pieces_kernel<TA, 2>, grid, dim3(NT), 0, s, g);
     return launch_kernel(gemm_pieces_kernel<TA, 4>, grid, dim3(NT), 0, s, g);

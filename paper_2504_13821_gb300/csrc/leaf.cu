@@ -46,6 +46,8 @@ extern template cudaError_t leaf_b256_launch<double>(const LeafArgs<double>&, cu
 
 cudaError_t leaf_wide_configure();
 cudaError_t leaf_wide_launch(const LeafArgs<float>& a, int num_sms, cudaStream_t s);
+cudaError_t leaf64_configure();
+cudaError_t leaf64_launch(const LeafArgs<double>& a, int num_sms, cudaStream_t s);
 cudaError_t convert_configure();
 cudaError_t refine_configure();
 cudaError_t dag_configure();
@@ -66,6 +68,7 @@ cudaError_t leaf_configure_all() {
     if ((e = leaf_b256_configure<float>()) != cudaSuccess) return e;
     if ((e = leaf_b256_configure<double>()) != cudaSuccess) return e;
     if ((e = leaf_wide_configure()) != cudaSuccess) return e;
+    if ((e = leaf64_configure()) != cudaSuccess) return e;
     if ((e = convert_configure()) != cudaSuccess) return e;
     if ((e = refine_configure()) != cudaSuccess) return e;
     if ((e = dag_configure()) != cudaSuccess) return e;
@@ -103,6 +106,11 @@ cudaError_t launch_leaf(bool trsm, const Canon<T>& p, int64_t r0, int b,
     if constexpr (std::is_same<T, float>::value) {
         if (blocked_on && trsm && nleaves == 1 && b > 64 && p.nrhs >= 1024)
             return leaf_wide_launch(a, num_sms, s);
+    }
+    // FP64, one leaf of 33..64 rows, many right-hand sides.
+    if constexpr (std::is_same<T, double>::value) {
+        if (blocked_on && trsm && nleaves == 1 && b > 32 && b <= 64 && p.nrhs >= 1024)
+            return leaf64_launch(a, num_sms, s);
     }
     if (blocked_on && trsm && nleaves == 1 && b > 32 && p.nrhs >= 1024)
         return leaf_blocked_launch<T>(a, (int64_t)(num_sms > 0 ? num_sms : 1) * 2, s);

@@ -1,0 +1,170 @@
+// FP64 TRSM leaf (Section 3.3 base kernel) of 33..64 rows with many right-hand
+// sides: blocked forward substitution in 16-row blocks, C columns per CTA of 128
+// threads.
+//
+// The FP64 pipe takes two FMAs per clock and SM: one FP64 instruction of a warp
+// holds it for 16 clocks, however few of its lanes count, and the substitution is
+// a chain of 64 multiply / FMA pairs. So L = 128 / C lanes share a column there (16 /
+// L rows each, x_j by shuffle), which keeps every lane's part of the chain short,
+// and in the rank-16 updates below the block every thread owns the same number of
+// rows x columns. Tiles are narrow (8 columns up to 8 an SM, 16 beyond) so that
+// every SM has one and two or three overlap one another's chains; the kernel of 64
+// columns per CTA and one lane per column that this one replaces kept 64 SMs busy
+// at 4096 right-hand sides.
+//
+// Measured, one 64-row leaf (us by right-hand sides, that kernel / this one, ncu):
+// 1024 47 / 17, 1500 48 / 21, 4096 54 / 29; four lanes per column took 20 (1024)
+// and 29 (4096), 32 columns per CTA 34 (4096). Below 1024 the lane-split leaf has as
+// short a chain and no barriers (16 us at 200 against 17).
+#include "common.cuh"
+#include "leaf_impl.cuh"
+
+namespace trx {
+namespace {
+
+template <int C>
+struct Leaf64 {
+    static constexpr int NT = 128, B = 64, SB = 16;
+    static constexpr int L = NT / C;                 // lanes per column in the substitution
+    static constexpr int RU = SB / L;                // rows per lane
+    static constexpr int CW = C / 8;   // columns per thread in the updates
+    static constexpr int CG = C / CW, RG = NT / CG;  // column and row groups
+    static constexpr int LDT = B + 1;                // column stride of the triangle
+    static constexpr int LDC = C + 2;                // row stride of the panel
+    static constexpr size_t smem = sizeof(double) * (size_t)(B * LDT + B + B * LDC);
+    static_assert(RG == SB, "a block's rows below divide evenly over the row groups");
+};
+
+template <int C>
+__global__ void __launch_bounds__(128) leaf64_kernel(LeafArgs<double> a) {
+    using S = Leaf64<C>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double* sT = reinterpret_cast<double*>(smem_raw);    // M(r0+i, r0+l) at l*LDT + i, i > l
+    double* sD = sT + S::B * S::LDT;                       // reciprocal diagonal
+    double* sC = sD + S::B;                                // C(r0+i, j0+c) at i*LDC + c
+    pdl_trigger();
+    pdl_wait();
+    const int tid = threadIdx.x;
+    const Canon<double>& p = a.p;
+    const int64_t r0 = a.r0, j0 = (int64_t)blockIdx.x * C;
+    const int bs = (int)min((int64_t)a.b, p.k - r0);
+    const int nc = (int)min((int64_t)C, p.nrhs - j0);
+
+    // panel and triangle along their contiguous index, every load of the panel
+    // in flight at once; rows past the leaf and columns past C are zero
+    constexpr int PL = S::B * C / S::NT;
+    const bool c_row_fast = p.c_rs == 1 || p.c_rs == -1;
+    double v[PL];
+#pragma unroll
+    for (int u = 0; u < PL; ++u) {
+        const int e = tid + u * S::NT;
+        const int i = c_row_fast ? e % S::B : e / C, c = c_row_fast ? e / S::B : e % C;
+        v[u] = i < bs && c < nc ? p.C[(r0 + i) * p.c_rs + (j0 + c) * p.c_cs] : 0.0;
+    }
+    const bool a_row_fast = p.a_rs == 1 || p.a_rs == -1;
+    const double* A = p.A + r0 * (p.a_rs + p.a_cs);
+    constexpr int TL = S::B * S::B / S::NT;
+    double d = 1.0;
+    if (tid < bs && !p.unit) d = A[tid * (p.a_rs + p.a_cs)];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        double t[TL / 2];
+#pragma unroll
+        for (int u = 0; u < TL / 2; ++u) {
+            const int e = tid + (h * (TL / 2) + u) * S::NT;
+            const int i = a_row_fast ? e % S::B : e / S::B, l = a_row_fast ? e / S::B : e % S::B;
+            t[u] = l < i && i < bs ? A[i * p.a_rs + l * p.a_cs] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < TL / 2; ++u) {
+            const int e = tid + (h * (TL / 2) + u) * S::NT;
+            const int i = a_row_fast ? e % S::B : e / S::B, l = a_row_fast ? e / S::B : e % S::B;
+            sT[l * S::LDT + i] = t[u];
+        }
+    }
+    if (tid < S::B) sD[tid] = 1.0 / d;
+#pragma unroll
+    for (int u = 0; u < PL; ++u) {
+        const int e = tid + u * S::NT;
+        const int i = c_row_fast ? e % S::B : e / C, c = c_row_fast ? e / S::B : e % C;
+        sC[i * S::LDC + c] = a.alpha * v[u];
+    }
+    __syncthreads();
+
+    const int sc = tid / S::L, sg = tid % S::L;            // substitution: column, lane of it
+    const int cg = tid % S::CG, rg = tid / S::CG;          // updates: columns, rows
+#pragma unroll
+    for (int s0 = 0; s0 < S::B; s0 += S::SB) {
+        // rows s0 .. s0+15 of column sc: lane sg holds rows sg + L u
+        double x[S::RU];
+#pragma unroll
+        for (int u = 0; u < S::RU; ++u) x[u] = sC[(s0 + sg + S::L * u) * S::LDC + sc];
+#pragma unroll
+        for (int j = 0; j < S::SB; ++j) {
+            const double xj = __shfl_sync(0xffffffffu, x[j / S::L], j % S::L, S::L) * sD[s0 + j];
+            if (sg == j % S::L) x[j / S::L] = xj;
+#pragma unroll
+            for (int u = j / S::L; u < S::RU; ++u) {
+                const int i = sg + S::L * u;
+                if (i > j) x[u] = fma(-sT[(s0 + j) * S::LDT + s0 + i], xj, x[u]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < S::RU; ++u) sC[(s0 + sg + S::L * u) * S::LDC + sc] = x[u];
+        __syncthreads();
+        // rank-16 update of the rows below
+        constexpr int UMAX = S::B / S::SB - 1;
+        const int nu = UMAX - s0 / S::SB;                  // compile-time after unrolling
+        double acc[UMAX][S::CW];
+#pragma unroll
+        for (int u = 0; u < UMAX; ++u)
+#pragma unroll
+            for (int w = 0; w < S::CW; ++w)
+                if (u < nu) acc[u][w] = sC[(s0 + S::SB * (u + 1) + rg) * S::LDC + cg * S::CW + w];
+#pragma unroll
+        for (int kk = 0; kk < S::SB; ++kk) {
+            double xv[S::CW];
+#pragma unroll
+            for (int w = 0; w < S::CW; ++w) xv[w] = sC[(s0 + kk) * S::LDC + cg * S::CW + w];
+#pragma unroll
+            for (int u = 0; u < UMAX; ++u) {
+                if (u >= nu) continue;
+                const double t = sT[(s0 + kk) * S::LDT + s0 + S::SB * (u + 1) + rg];
+#pragma unroll
+                for (int w = 0; w < S::CW; ++w) acc[u][w] = fma(-t, xv[w], acc[u][w]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < UMAX; ++u)
+#pragma unroll
+            for (int w = 0; w < S::CW; ++w)
+                if (u < nu) sC[(s0 + S::SB * (u + 1) + rg) * S::LDC + cg * S::CW + w] = acc[u][w];
+        __syncthreads();
+    }
+#pragma unroll
+    for (int u = 0; u < PL; ++u) {
+        const int e = tid + u * S::NT;
+        const int i = c_row_fast ? e % S::B : e / C, c = c_row_fast ? e / S::B : e % C;
+        if (i < bs && c < nc) p.C[(r0 + i) * p.c_rs + (j0 + c) * p.c_cs] = sC[i * S::LDC + c];
+    }
+}
+
+}  // namespace
+
+cudaError_t leaf64_configure() {
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(leaf64_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)Leaf64<8>::smem)) != cudaSuccess)
+        return e;
+    return cudaFuncSetAttribute(leaf64_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)Leaf64<16>::smem);
+}
+
+cudaError_t leaf64_launch(const LeafArgs<double>& a, int num_sms, cudaStream_t s) {
+    const int c = a.p.nrhs <= 8 * (int64_t)num_sms ? 8 : 16;
+    const dim3 grid((unsigned)((a.p.nrhs + c - 1) / c));
+    if (c == 8) return launch_kernel(leaf64_kernel<8>, grid, dim3(128), Leaf64<8>::smem, s, a);
+    return launch_kernel(leaf64_kernel<16>, grid, dim3(128), Leaf64<16>::smem, s, a);
+}
+
+}  // namespace trx
