@@ -516,7 +516,7 @@ int trx_batch_destroy(trx_batch_t batch);
 /* Tuning table of the batched kernel: the substitution block height (4, 8
  * or 16 rows) per order bucket (k <= 64, 128, 256, 512) and right-hand-side
  * bucket (nrhs <= 8, 24, more), for each element type; 8 everywhere on a new
- * handle. */
+ * handle. The FP32 kernel's height is 16 whatever its table says. */
 #define TRX_TUNE_K_BUCKETS 4
 #define TRX_TUNE_N_BUCKETS 3
 

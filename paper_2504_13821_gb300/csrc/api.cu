@@ -19,6 +19,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "batched.cuh"
 #include "common.cuh"
 #include "plan.cuh"
 #include "trx.h"
@@ -27,15 +28,6 @@ namespace trx {
 // Leaf kernels set their shared-memory limits once per device (leaf.cu).
 cudaError_t leaf_configure_all();
 
-struct BatchDesc {
-    int64_t k, nrhs;
-    const void* A;
-    int64_t a_rs, a_cs;
-    void* C;
-    int64_t c_rs, c_cs;
-    double alpha;
-    int unit, trsm, sb, pad;
-};
 cudaError_t batched_configure();
 cudaError_t launch_batched(int elem_bytes, const BatchDesc* descs, int64_t count, int* counter,
                            int grid_ctas, cudaStream_t s);
@@ -1015,10 +1007,30 @@ int batch_descs(trx_handle_t h, int elem_bytes, int64_t count, const trx_problem
         const int b = tune_index(d.k, d.nrhs);
         d.sb = sb_override ? sb_override[b]
                            : (&h->tune_sb[elem_bytes == 4 ? 0 : 1][0][0])[b];
-        out.push_back(d);
+        d.bucket = b;
+        d.problems = 1;
+        if (elem_bytes == 8 || d.trsm == 2) {
+            out.push_back(d);
+            continue;
+        }
+        // FP32: a descriptor per chunk of right-hand sides (the kernel's widest at this
+        // order; several chunks each beyond 256 of them), so that a large problem's
+        // chunks run on several CTAs at once
+        const int64_t w = batch_f32_chunk(d.k);
+        const int64_t step = ((d.nrhs + w - 1) / w + 255) / 256 * w;
+        const int64_t nrhs = d.nrhs;
+        for (int64_t c = 0; c < nrhs; c += step) {
+            BatchDesc piece = d;
+            piece.C = static_cast<float*>(d.C) + c * d.c_cs;
+            piece.nrhs = std::min(step, nrhs - c);
+            piece.problems = c == 0;
+            out.push_back(piece);
+        }
     }
-    std::stable_sort(out.begin(), out.end(), [](const BatchDesc& x, const BatchDesc& y) {
-        return (double)x.k * x.k * x.nrhs > (double)y.k * y.k * y.nrhs;
+    // largest first; FP32: a chunk's steps cost about as much as 16 columns more
+    const double extra = elem_bytes == 4 ? 16 : 0;
+    std::stable_sort(out.begin(), out.end(), [extra](const BatchDesc& x, const BatchDesc& y) {
+        return (double)x.k * x.k * (x.nrhs + extra) > (double)y.k * y.k * (y.nrhs + extra);
     });
     return TRX_SUCCESS;
 }
@@ -1275,9 +1287,10 @@ int trx_batched_autotune(trx_handle_t h, int elem_bytes, int64_t count,
             int rc = batch_descs(h, elem_bytes, count, problems, all, ov);
             if (rc != TRX_SUCCESS) return rc;
             for (auto& x : all)
-                if (tune_index(x.k, x.nrhs) == bkt) mine.push_back(x);
+                if (x.bucket == bkt) mine.push_back(x);
             all_ms[bkt][v] = 0.0;
-            count_b[bkt] = (int)mine.size();
+            count_b[bkt] = 0;
+            for (const auto& x : mine) count_b[bkt] += x.problems;
             if (mine.empty()) continue;
             double ms_sum = 0.0;
             for (int rep = 0; rep < 4; ++rep) {

@@ -1,5 +1,6 @@
 // Batched uneven TRSM / TRMM: thousands of small independent problems
-// (order k <= 512) in one persistent launch.
+// (order k <= 512) in one persistent launch: the launch, and the FP64 kernel
+// (batched_f32.cu has the FP32 one).
 //
 // Each problem is first mapped on the host to the canonical lower form of
 // common.cuh (any side/uplo/trans/diag, TRSM or TRMM). The descriptors are
@@ -22,35 +23,29 @@
 // recursive entry points.
 #include <algorithm>
 
+#include "batched.cuh"
 #include "common.cuh"
 
 namespace trx {
 
-struct BatchDesc {
-    int64_t k, nrhs;
-    const void* A;
-    int64_t a_rs, a_cs;
-    void* C;
-    int64_t c_rs, c_cs;
-    double alpha;
-    int unit, trsm, sb, pad;
-};
-
-constexpr int kBatchMaxK = 512;
+cudaError_t batched_f32_configure();
+int batched_f32_ctas_per_sm();
+cudaError_t launch_batched_f32(const BatchDesc* descs, int64_t count, int* counter, int grid,
+                               cudaStream_t s);
 
 namespace {
 
 template <typename T>
 struct BShape {
     static constexpr int NT = 256;
-    static constexpr int NC = sizeof(T) == 4 ? 32 : 16;    // columns per chunk
+    static constexpr int NC = 16;                          // columns per chunk
     static constexpr int LDC = NC + 1;                     // odd stride: three CTAs per SM
     static constexpr int CG = NC / 4;                      // column groups of 4
     static constexpr int RG = NT / CG;                     // row groups
     static constexpr int SBMAX = 16;                       // largest substitution block
     // panel, diagonal, two staged diagonal tiles of the substitution blocks
     static constexpr size_t smem =
-        sizeof(T) * ((size_t)kBatchMaxK * LDC + kBatchMaxK + 2 * SBMAX * SBMAX);
+        sizeof(T) * ((size_t)kBatchOrder * LDC + kBatchOrder + 2 * SBMAX * SBMAX);
 };
 
 template <typename T>
@@ -195,8 +190,8 @@ __global__ void __launch_bounds__(256, 3) batched_kernel(const BatchDesc* descs,
     using S = BShape<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* sC = reinterpret_cast<T*>(smem_raw);         // panel: row i, column c at i*LDC + c
-    T* sD = sC + (size_t)kBatchMaxK * S::LDC;         // reciprocal (TRSM) or plain (TRMM) diagonal
-    T* sTile = sD + kBatchMaxK;                        // two staged diagonal tiles
+    T* sD = sC + (size_t)kBatchOrder * S::LDC;         // reciprocal (TRSM) or plain (TRMM) diagonal
+    T* sTile = sD + kBatchOrder;                        // two staged diagonal tiles
     __shared__ int s_next;
     pdl_trigger();
     pdl_wait();
@@ -267,9 +262,7 @@ __global__ void __launch_bounds__(256, 3) batched_kernel(const BatchDesc* descs,
 }  // namespace
 
 cudaError_t batched_configure() {
-    cudaError_t e = cudaFuncSetAttribute(batched_kernel<float>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)BShape<float>::smem);
+    cudaError_t e = batched_f32_configure();
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(batched_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)BShape<double>::smem);
@@ -277,12 +270,10 @@ cudaError_t batched_configure() {
 
 // Resident CTAs per SM of the batched kernel (occupancy query, at least 1).
 int batched_ctas_per_sm(int elem_bytes) {
+    if (elem_bytes == 4) return batched_f32_ctas_per_sm();
     int n = 0;
-    const cudaError_t e = elem_bytes == 4
-        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batched_kernel<float>, BShape<float>::NT,
-                                                        BShape<float>::smem)
-        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batched_kernel<double>, BShape<double>::NT,
-                                                        BShape<double>::smem);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &n, batched_kernel<double>, BShape<double>::NT, BShape<double>::smem);
     return (e == cudaSuccess && n > 0) ? n : 1;
 }
 
@@ -295,8 +286,7 @@ cudaError_t launch_batched(int elem_bytes, const BatchDesc* descs, int64_t count
     if (e != cudaSuccess) return e;
     const int grid = (int)std::min<int64_t>(grid_ctas, count);
     if (elem_bytes == 4)
-        return launch_kernel(batched_kernel<float>, dim3(grid), dim3(256), BShape<float>::smem, s,
-                             descs, count, counter);
+        return launch_batched_f32(descs, count, counter, grid, s);
     return launch_kernel(batched_kernel<double>, dim3(grid), dim3(256), BShape<double>::smem, s,
                          descs, count, counter);
 }
