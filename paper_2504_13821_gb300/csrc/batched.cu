@@ -38,7 +38,7 @@ namespace {
 template <typename T>
 struct BShape {
     static constexpr int NT = 256;
-    static constexpr int NC = 16;                          // columns per chunk
+    static constexpr int NC = kBatchF64Chunk;              // columns per chunk
     static constexpr int LDC = NC + 1;                     // odd stride: three CTAs per SM
     static constexpr int CG = NC / 4;                      // column groups of 4
     static constexpr int RG = NT / CG;                     // row groups

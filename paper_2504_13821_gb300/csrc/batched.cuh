@@ -18,6 +18,7 @@ struct BatchDesc {
 
 constexpr int kBatchOrder = 512;   // largest order
 
+constexpr int kBatchF64Chunk = 16;   // right-hand sides of the FP64 kernel's chunk
 // Right-hand sides of the FP32 kernel's widest chunk at order k.
 __host__ __device__ constexpr int64_t batch_f32_chunk(int64_t k) { return k <= 256 ? 64 : 32; }
 

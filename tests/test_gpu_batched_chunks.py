@@ -1,4 +1,4 @@
-"""FP32 batched problems at the edges of the kernel's 16-row blocks, its 16-, 32- and
+"""Batched problems (FP32, and FP64 cut over several CTAs) at the edges of the kernel's 16-row blocks, its 16-, 32- and
 64-column chunks, the order where wide chunks end and the one where two blocks'
 columns no longer fit together; right-hand sides cut over several CTAs; every
 orientation; a batch larger than three rounds of the launch's CTAs (problems taken
@@ -18,12 +18,12 @@ pytestmark = pytest.mark.gpu
 WAYS = list(itertools.product("SM", "LR", "LU", "NT", "NU"))
 
 
-def run(shapes, seed):
+def run(shapes, seed, dtype=np.float32):
     import paper_2504_13821_gb300 as trx
     probs, host = [], []
     for i, (k, nrhs, (op, side, uplo, trans, diag), alpha) in enumerate(shapes):
         m, n = (k, nrhs) if side == "L" else (nrhs, k)
-        A, B = inputs.problem(side, uplo, m, n, seed=seed + i, dtype=np.float32,
+        A, B = inputs.problem(side, uplo, m, n, seed=seed + i, dtype=dtype,
                               poison_diag=(diag == "U"), lda=k + i % 4, ldb=m + i % 3)
         B[m:, :] = SENTINEL
         At, Bt = to_dev(A, "cuda:0"), to_dev(B, "cuda:0")
@@ -41,7 +41,7 @@ def run(shapes, seed):
         else:
             ref = oracle.trmm(side, uplo, trans, diag, alpha, Ak, B0)
             e = oracle.trmm_error(side, uplo, trans, diag, alpha, Ak, X, ref, B0)
-        assert np.isfinite(e) and e <= bound(k, np.float32), (op, side, uplo, trans, diag, k, nrhs)
+        assert np.isfinite(e) and e <= bound(k, dtype), (op, side, uplo, trans, diag, k, nrhs)
 
 
 @pytest.mark.parametrize("k", [1, 2, 15, 16, 17, 33, 64, 127, 129, 255, 256, 257, 300, 395, 411,
@@ -51,6 +51,14 @@ def test_edges(k):
     shapes = [(k, widths[(i + k) % len(widths)], way, (1.0, -0.5)[i % 2])
               for i, way in enumerate(WAYS)]
     run(shapes, 1000 * k)
+
+
+@pytest.mark.parametrize("k", [1, 17, 130, 512])
+def test_f64_cut_over_ctas(k):
+    widths = [1, 15, 16, 17, 64, 77, 300]
+    shapes = [(k, widths[i % 7], way, (1.0, -0.5)[i % 2]) for i, way in enumerate(WAYS)]
+    shapes.append((40, 9000, WAYS[k % 32], 1.0))
+    run(shapes, 1000 * k, np.float64)
 
 
 def test_many_problems_and_wide_right_hand_sides():
