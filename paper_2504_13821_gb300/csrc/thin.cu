@@ -27,15 +27,26 @@
 // right-hand sides (the thin leaves): on a leaf's rows, its columns of M
 // and its rows of C, with the tensor-core updates between leaves.
 //
-// A block is published as 1024 tagged 64-bit words (FP32 bits in the low
-// half, 1 in the high half; a 64-bit access is single-copy atomic, so value
-// and tag arrive together): a consumer polls the words themselves, one L2
-// round trip, with no flag and no fence between data and signal. The words
-// are zeroed by a memset before each launch.
+// A task is eight consecutive block rows of a panel, one a CTA of a cluster. A
+// finished block goes to the next four CTAs by st.async into their shared memory
+// (with an mbarrier each, 0.2 us), and to everyone as 1024 tagged 64-bit words (FP32
+// bits in the low half, 1 in the high half; a 64-bit access is single-copy atomic, so
+// value and tag arrive together): a consumer polls the words themselves, one L2
+// round trip (0.64 us a poll, 1.5 us from store to use), with no flag and no fence
+// between data and signal. The words are zeroed by a memset before each launch.
+//
+// Four warps of a CTA bring in the tiles of M through a ring of cp.async stages, the
+// eight others do the products. Bound by the chain: from X_i-2's arrival a CTA does
+// three products (its last tile, the inverse, Z) of 0.5-0.67 us each in two steps.
+// us, this kernel against one CTA per ticket that published through L2 only, staged M
+// between its products and had a thread on 4 rows x 1 column: 8191 x 16 transposed
+// 323 -> 259, 8192 x 16 323 -> 225, 8192 x 64 449 -> 316, a 2048-row leaf with 256
+// right-hand sides 121 -> 87. On the way: the products alone 309, clusters with M
+// still staged between them 283.
 //
 // Tasks are taken in order from an atomic counter (block row major), so a
 // task only waits for tasks taken before it, which are running or done: the
-// solve progresses whatever the number of resident CTAs. Every wait is
+// solve progresses whatever the number of resident clusters. Every wait is
 // bounded: past the budget the CTA writes TRX_ERR_TIMEOUT to the error word
 // and the launch's stop word, and every waiting CTA then stops.
 //
@@ -54,6 +65,9 @@ constexpr int NP = kThinPanel;       // columns of a panel
 constexpr int NT = 256;
 constexpr int LD = BR + 4;           // shared row stride (floats): 16-byte aligned rows
 constexpr int LDT = BR + 1;          // inverse work tile: conflict-free column reads
+constexpr int CL = 8;                // block rows of a task, CTAs of a cluster
+constexpr int ND = 4;                // block rows that a CTA pushes its block to
+constexpr int NTP = 128;             // threads of the solve that bring in M
 constexpr int kTimeout = 4;          // TRX_ERR_TIMEOUT
 
 struct Params {
@@ -89,12 +103,16 @@ constexpr int STAGES = 3;
 struct Smem {
     // M_ij tiles, k-major: m[s][kk * LD + r] = M[i0 + r][j0 + kk]; tile j of
     // a task's sum sits in stage (j + 1) % STAGES (stage 0 also serves as the
-    // work tile of the inverse and of Z before the ring reaches it)
+    // work tile of the inverse and of Z before)
     float m[STAGES][BR * LD];
     float inv[BR * LD];      // inv(M_ii), k-major: inv[kk * LD + r] = Inv[r][kk]
     float z[BR * LD];        // Z = inv(M_ii) M_i,i-1, k-major
-    float x[BR * NP];        // X_jp tile / right-hand side: x[kk * NP + c]
+    float x[2][BR * NP];     // X_jp tiles / right-hand side: x[.][kk * NP + c]
+    float near[ND][BR * NP];  // X_i-1 .. X_i-ND as the cluster's CTAs push them
     float dinv[BR];
+    unsigned long long near_full[ND];                // mbarriers: `near`,
+    unsigned long long full[STAGES], empty[STAGES];  // the stages of m
+    int pushed[ND];          // set by the CTA that has sent a block to `near`
     int task;
     int abort;
 };
@@ -105,9 +123,14 @@ __device__ __forceinline__ unsigned long long ld_relaxed64(const unsigned long l
     asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
-__device__ __forceinline__ void st_relaxed64(unsigned long long* p, unsigned long long v) {
-    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+// two words, each an access of its own to the memory model (16-byte aligned)
+__device__ __forceinline__ void st_relaxed64x2(unsigned long long* p, unsigned long long u,
+                                               unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(u), "l"(v) : "memory");
 }
+
+// barrier of the NT threads that compute
+__device__ __forceinline__ void sync_nt() { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); }
 
 __device__ __forceinline__ uint64_t gtimer() {
     uint64_t t;
@@ -120,28 +143,33 @@ constexpr int Q = (BR * NP) / NT;    // tagged words of a block per thread
 // values are checked by finish_x, so they can be issued a step ahead).
 __device__ __forceinline__ void issue_x(const Params& p, int pn, int j,
                                         unsigned long long (&w)[Q]) {
-    const unsigned long long* src = p.xt + ((int64_t)pn * p.nbr + j) * (BR * NP);
+    const unsigned long long* src = p.xt + ((int64_t)pn * p.nbr + j) * (BR * NP) + 2 * threadIdx.x;
 #pragma unroll
-    for (int q = 0; q < Q; ++q) w[q] = ld_relaxed64(src + threadIdx.x + NT * q);
+    for (int q = 0; q < Q; q += 2)
+        asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];"
+                     : "=l"(w[q]), "=l"(w[q + 1])
+                     : "l"(src + NT * q)
+                     : "memory");
 }
 
-// X_jp into sm.x from its tagged words: a word loaded before it was
+// X_jp into `x` from its tagged words: a word loaded before it was
 // published (tag 0) is polled again (single-copy atomic 64-bit loads: value
 // and tag arrive together), at most wait_ns. False on timeout (the error
 // word and the launch's stop word are set) or once another CTA has stopped
 // the launch.
-__device__ bool finish_x(const Params& p, Smem& sm, int pn, int j,
+__device__ bool finish_x(const Params& p, float* x, int pn, int j,
                          const unsigned long long (&w)[Q]) {
     const unsigned long long* src = p.xt + ((int64_t)pn * p.nbr + j) * (BR * NP);
     const int t = threadIdx.x;
     bool ok = true;
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
-        const int idx = t + NT * q;
+        const int idx = 2 * t + NT * (q & ~1) + (q & 1);
         unsigned long long v = w[q];
         if (v < kTag) {
             const uint64_t t0 = gtimer();
             while ((v = ld_relaxed64(src + idx)) < kTag) {
+                
                 if (*(volatile int*)p.stop) { ok = false; break; }
                 if (gtimer() - t0 > (uint64_t)p.wait_ns) {
                     atomicExch(p.err, kTimeout);
@@ -152,9 +180,69 @@ __device__ bool finish_x(const Params& p, Smem& sm, int pn, int j,
             }
             if (!ok) break;
         }
-        sm.x[idx] = __uint_as_float((unsigned)v);
+        x[idx] = __uint_as_float((unsigned)v);
     }
     return ok;
+}
+
+// ---- blocks pushed from one CTA of a cluster to the next ones --------------
+__device__ __forceinline__ uint32_t smem_u32(const void* p) {
+    return (uint32_t)__cvta_generic_to_shared(p);
+}
+__device__ __forceinline__ int cluster_rank() {
+    int r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ bool try_wait(uint32_t bar, int parity) {
+    uint32_t done;
+    asm volatile(
+        "{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p; }"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return done;
+}
+// Bounded like finish_x.
+__device__ bool wait_bar(const Params& p, const unsigned long long* bar, int parity) {
+    const uint32_t a = smem_u32(bar);
+    if (try_wait(a, parity)) return true;
+    const uint64_t t0 = gtimer();
+    while (!try_wait(a, parity)) {
+        if (*(volatile int*)p.stop) return false;
+        if (gtimer() - t0 > (uint64_t)p.wait_ns) {
+            atomicExch(p.err, kTimeout);
+            atomicExch(p.stop, 1);
+            return false;
+        }
+    }
+    return true;
+}
+// For a block that is known to be under way.
+__device__ void wait_landed(const unsigned long long* bar) {
+    const uint64_t t0 = gtimer();
+    while (!try_wait(smem_u32(bar), 0) && gtimer() - t0 < 1000000000ull) {}
+}
+// This thread's two columns of one row of X_i into slot `slot` of CTA `rank`, which
+// counts the bytes as they land.
+__device__ __forceinline__ void push_near(const Smem& sm, int slot, int rank, int at, float u,
+                                          float v) {
+    asm volatile(
+        "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(
+            map_rank(smem_u32(&sm.near[slot][at]), rank)),
+        "r"(__float_as_uint(u)), "r"(__float_as_uint(v)),
+        "r"(map_rank(smem_u32(&sm.near_full[slot]), rank))
+        : "memory");
 }
 
 // Tile (i0.., j0..) of M into registers, 16 elements a thread, along M's
@@ -189,23 +277,32 @@ __device__ __forceinline__ void cp_wait_ring() {
     asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
 }
 
-// Tile (i0.., j0..) of M into ring stage `dst` by cp.async (element by
-// element along M's contiguous direction, into the k-major layout); rows
-// past the order are zero-filled (no read). Commits one group.
+// The producer warps' share of tile (i0.., j0..) of M into `dst` by cp.async: in
+// 16-byte copies where M's columns are contiguous and aligned, else element by element
+// along M's contiguous direction (8.6 clocks a warp, 0.6 us a tile); rows past the
+// order are zero-filled (no read).
 __device__ __forceinline__ void issue_m(const Params& p, float* dst, int64_t i0, int64_t j0,
-                                        bool colmajor) {
-    const int t = threadIdx.x;
-    const int rr0 = colmajor ? (t & 63) : (t >> 6), cc0 = colmajor ? (t >> 6) : (t & 63);
-    const float* src = p.A + (i0 + rr0) * p.a_rs + (j0 + cc0) * p.a_cs;
-    const int64_t step = 4 * (colmajor ? p.a_cs : p.a_rs);
-    const int64_t rows_left = p.k - (i0 + rr0);
+                                        bool colmajor, bool wide) {
+    const int t = threadIdx.x - NT;
+    if (wide && i0 + BR <= p.k) {
+        const int rr = 4 * (t & 15), cc = t >> 4;
+        const float* src = p.A + (i0 + rr) + (j0 + cc) * p.a_cs;
+        float* d = dst + cc * LD + rr;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-        const int rr = colmajor ? rr0 : rr0 + 4 * q, cc = colmajor ? cc0 + 4 * q : cc0;
-        const bool in = colmajor ? rows_left > 0 : rows_left > 4 * q;
-        cp_async4(dst + cc * LD + rr, in ? src + q * step : p.A, in);
+        for (int q = 0; q < BR * BR / 4 / NTP; ++q, src += 8 * p.a_cs) cp_async16(d + 8 * q * LD, src);
+        return;
     }
-    cp_commit();
+    const int rr = colmajor ? (t & 63) : (t >> 6), cc = colmajor ? (t >> 6) : (t & 63);
+    const float* src = p.A + (i0 + rr) * p.a_rs + (j0 + cc) * p.a_cs;
+    const int64_t step = 2 * (colmajor ? p.a_cs : p.a_rs);
+    const int64_t rows = p.k - (i0 + rr);
+    float* d = dst + cc * LD + rr;
+    const int dstep = colmajor ? 2 * LD : 2;
+#pragma unroll 8
+    for (int q = 0; q < BR * BR / NTP; ++q, src += step, d += dstep) {
+        const bool in = colmajor ? rows > 0 : rows > 2 * q;
+        cp_async4(d, in ? src : p.A, in);
+    }
 }
 
 // Packed FP32 pairs: fma.rn.f32x2 does two independent round-to-nearest
@@ -224,23 +321,63 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
     return d;
 }
 
-// acc[e] += sum_kk a[kk][4 ty + e] * x[kk][tx] over kk < kend (rows in
-// packed pairs (4 ty, 4 ty + 1), (4 ty + 2, 4 ty + 3): two FMA
-// instructions per kk instead of four).
-__device__ __forceinline__ void mma_tile(const float* a, const float* x, int kend,
-                                         float (&acc)[4]) {
-    const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-    uint64_t s01 = pk2(acc[0], acc[1]), s23 = pk2(acc[2], acc[3]);
+// The two rows and two columns of a 64 x 16 block that a thread ends up with.
+struct Own {
+    int row, col;
+};
+__device__ __forceinline__ Own own_elements() {
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, kg = (l >> 2) & 3;
+    return {32 * (w >> 2) + 4 * (w & 3) + 16 * (l >> 4) + 2 * (kg & 1), 4 * (l & 3) + 2 * (kg >> 1)};
+}
+// acc[r][c] += sum_kk a[kk][row + r] * x[kk][col + c] for the thread's rows and columns;
+// LOWER: a is lower triangular. Four lanes share a 4 x 4 tile, each with every
+// fourth kk, and exchange halves of their sums at the end: 32 vector loads and 128
+// packed FMAs a thread for 64 kk. (With a thread on 4 rows x 1 column over all kk,
+// 128 loads, shared memory set the pace.) A warp's two row tiles
+// lie 16 rows apart, so its M words fall into 32 different banks.
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+template <bool LOWER = false>
+__device__ __forceinline__ void mma_tile(const float* a, const float* x, float (&acc)[2][2]) {
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, ct = l & 3, kg = (l >> 2) & 3;
+    const int row = 32 * (w >> 2) + 4 * (w & 3) + 16 * (l >> 4);   // the four rows' first
+    const int kend = LOWER ? 32 * (w >> 2) + 4 * (w & 3) + 20 : BR;
+    const float* ap = a + kg * LD + row;
+    const float* xp = x + kg * NP + 4 * ct;
+    uint64_t s0[4] = {}, s1[4] = {};       // rows 0, 1 and 2, 3 of the tile by column
 #pragma unroll 8
-    for (int kk = 0; kk < kend; ++kk) {
-        const float4 m = *reinterpret_cast<const float4*>(a + kk * LD + 4 * ty);
-        const float xv = x[kk * NP + tx];
-        const uint64_t xx = pk2(xv, xv);
-        s01 = fma2(pk2(m.x, m.y), xx, s01);
-        s23 = fma2(pk2(m.z, m.w), xx, s23);
+    for (int kk = 0; kk < kend; kk += 4) {
+        const ulonglong2 m = *reinterpret_cast<const ulonglong2*>(ap + kk * LD);
+        float4 v = *reinterpret_cast<const float4*>(xp + kk * NP);
+        // (lower: nothing right of the tile takes part, as a zero times an Inf there
+        // would make a NaN)
+        if (LOWER && kk > row) v = make_float4(0.f, 0.f, 0.f, 0.f);
+        const uint64_t b[4] = {pk2(v.x, v.x), pk2(v.y, v.y), pk2(v.z, v.z), pk2(v.w, v.w)};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            s0[c] = fma2(m.x, b[c], s0[c]);
+            s1[c] = fma2(m.y, b[c], s1[c]);
+        }
     }
-    upk2(s01, acc[0], acc[1]);
-    upk2(s23, acc[2], acc[3]);
+    // lanes kg and kg ^ 1 swap row pairs, then kg and kg ^ 2 column pairs
+    uint64_t h[4], f[2];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const uint64_t got = __shfl_xor_sync(0xffffffffu, kg & 1 ? s0[c] : s1[c], 4);
+        h[c] = add2(kg & 1 ? s1[c] : s0[c], got);
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const uint64_t got = __shfl_xor_sync(0xffffffffu, kg & 2 ? h[c] : h[c + 2], 8);
+        f[c] = add2(kg & 2 ? h[c + 2] : h[c], got);
+        float lo, hi;
+        upk2(f[c], lo, hi);
+        acc[0][c] += lo;
+        acc[1][c] += hi;
+    }
 }
 
 // inv(M_ii) into sm.inv. M_ii's lower triangle goes to a work tile (aliasing
@@ -253,23 +390,28 @@ __device__ void invert_diag(const Params& p, Smem& sm, int64_t i0) {
     float* T = sm.m[0];
     const int t = threadIdx.x, w = t >> 5, l = t & 31;
     const bool colmajor = p.a_rs == 1 || p.a_rs == -1;
-    for (int e = t; e < BR * BR; e += NT) {
-        const int rr = colmajor ? e % BR : e / BR;
-        const int cc = colmajor ? e / BR : e % BR;
-        const int64_t gi = i0 + rr, gj = i0 + cc;
-        float v = 0.0f;
-        if (gi >= p.k) v = rr == cc ? 1.0f : 0.0f;
-        else if (cc < rr) v = __ldg(p.A + gi * p.a_rs + gj * p.a_cs);
-        else if (cc == rr) v = p.unit ? 1.0f : __ldg(p.A + gi * p.a_rs + gj * p.a_cs);
-        T[rr * LDT + cc] = v;
+    // all loads in flight at once (one after the other they took most of the time)
+    float v[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+        const int rr = colmajor ? (t & 63) : (t >> 6) + 4 * q;
+        const int cc = colmajor ? (t >> 6) + 4 * q : (t & 63);
+        const bool read = i0 + rr < p.k && (cc < rr || (cc == rr && !p.unit));
+        v[q] = read ? __ldg(p.A + (i0 + rr) * p.a_rs + (i0 + cc) * p.a_cs) : rr == cc ? 1.0f : 0.0f;
     }
-    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+        const int rr = colmajor ? (t & 63) : (t >> 6) + 4 * q;
+        const int cc = colmajor ? (t >> 6) + 4 * q : (t & 63);
+        T[rr * LDT + cc] = v[q];
+    }
+    sync_nt();
     if (t < BR) sm.dinv[t] = 1.0f / T[t * LDT + t];
-    __syncthreads();
+    sync_nt();
     float y0[8], y1[8];          // rows l and l + 32, columns 8 w + u
 #pragma unroll
     for (int u = 0; u < 8; ++u) y0[u] = y1[u] = 0.0f;
-    for (int r = 0; r < BR; ++r) {
+    for (int r = 8 * w; r < BR; ++r) {   // (rows above the columns: zeros)
         const float dr = sm.dinv[r];
         const int owner = r & 31;
         const bool hi = r >= 32;
@@ -293,7 +435,7 @@ __device__ void invert_diag(const Params& p, Smem& sm, int64_t i0) {
         sm.inv[(8 * w + u) * LD + l] = y0[u];
         sm.inv[(8 * w + u) * LD + l + 32] = y1[u];
     }
-    __syncthreads();
+    sync_nt();
 }
 
 // Z = inv(M_ii) M_i,i-1 into sm.z (k-major), M_i,i-1 staged row-major in
@@ -309,7 +451,7 @@ __device__ void make_z(const Params& p, Smem& sm, int64_t i0, bool colmajor) {
         const int cc = colmajor ? (t >> 6) + 4 * q : (t & 63);
         sm.m[0][rr * LD + cc] = r[q];
     }
-    __syncthreads();
+    sync_nt();
     float acc[4][4];
 #pragma unroll
     for (int e = 0; e < 4; ++e)
@@ -331,7 +473,7 @@ __device__ void make_z(const Params& p, Smem& sm, int64_t i0, bool colmajor) {
     for (int e = 0; e < 4; ++e)
 #pragma unroll
         for (int u = 0; u < 4; ++u) sm.z[(tx + 16 * u) * LD + 4 * ty + e] = acc[e][u];
-    __syncthreads();
+    sync_nt();
 }
 
 // inv(M_ii) and Z_i = inv(M_ii) M_i,i-1 of block row blockIdx.x into
@@ -351,99 +493,159 @@ __global__ void __launch_bounds__(NT) thin_prep_kernel(const Params p, float* in
     }
 }
 
-__global__ void __launch_bounds__(NT, 2) thin_trsm_kernel(const Params p) {
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT + NTP, 2)
+    thin_trsm_kernel(const Params p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
-    const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
+    const int t = threadIdx.x;
+    const Own own = own_elements();
     const bool colmajor = p.a_rs == 1 || p.a_rs == -1;
-    if (t == 0) sm.abort = 0;
-    while (true) {
-        __syncthreads();
-        if (t == 0) sm.task = atomicAdd(p.ticket, 1);
-        __syncthreads();
-        const int64_t task = sm.task;
-        if (task >= p.ntask || sm.abort) break;
-        const int i = (int)(task / p.npan), pn = (int)(task % p.npan);
-        const int64_t i0 = (int64_t)i * BR, c0 = (int64_t)pn * NP;
+    // one task a cluster, in the order of the tickets: CL consecutive block rows of a
+    // panel, one a CTA
+    const int rank = cluster_rank();
+    if (t == 0) {
+        sm.abort = 0;
+        for (int q = 0; q < ND; ++q) {
+            sm.pushed[q] = 0;
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&sm.near_full[q])));
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(
+                             smem_u32(&sm.near_full[q])),
+                         "r"((int)(BR * NP * sizeof(float)))
+                         : "memory");
+        }
+        for (int q = 0; q < STAGES; ++q) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&sm.full[q])),
+                         "n"(NTP));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&sm.empty[q])),
+                         "n"(NT / 32));
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        if (rank == 0) sm.task = atomicAdd(p.ticket, 1);
+    }
+    cluster_sync();
+    int task;
+    asm volatile("ld.shared::cluster.s32 %0, [%1];"
+                 : "=r"(task)
+                 : "r"(map_rank(smem_u32(&sm.task), 0)));
+    const int i = task / p.npan * CL + rank, pn = task % p.npan;
+    const int64_t i0 = (int64_t)i * BR, c0 = (int64_t)pn * NP;
+    const int jz = i - 1;                             // blocks j < jz of M go into S'
+    if (t >= NT) {
+        // producers: tile j of M into stage (j + 1) % STAGES as the stage comes free
+        const bool wide = p.a_rs == 1 && p.a_cs % 4 == 0 && ((uintptr_t)p.A & 15) == 0;
+        if (i < p.nbr)
+            for (int j = 0; j < jz; ++j) {
+                const int s = (j + 1) % STAGES, n = j / STAGES;
+                if ((s == 0 || n > 0) && !wait_bar(p, &sm.empty[s], (s == 0 ? n : n - 1) & 1)) break;
+                issue_m(p, sm.m[s], i0, (int64_t)j * BR, colmajor, wide);
+                asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(
+                                 smem_u32(&sm.full[s]))
+                             : "memory");
+            }
+    } else while (i < p.nbr) {   // left by the breaks
         // this task's right-hand side rows, read before anything is written
-        float b[4];
+        float b[2][2];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const int64_t gi = i0 + 4 * ty + e, gj = c0 + tx;
-            b[e] = (gi < p.k && gj < p.nrhs) ? __ldcg(p.C + gi * p.c_rs + gj * p.c_cs) : 0.0f;
+            const int64_t gi = i0 + own.row + (e & 1), gj = c0 + own.col + (e >> 1);
+            b[e & 1][e >> 1] = (gi < p.k && gj < p.nrhs) ? __ldcg(p.C + gi * p.c_rs + gj * p.c_cs) : 0.0f;
         }
-        // S' = sum_{j < i-1} M_ij X_jp (X_i-1,p enters through Z): tile j of M
-        // arrives through the cp.async ring (STAGES - 1 tiles ahead), X_jp's words
-        // are loaded one step ahead
-        float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        // S' = sum_{j < i-1} M_ij X_jp (X_i-1,p enters through Z), X_jp's words loaded
+        // one step ahead
+        float acc[2][2] = {};
         unsigned long long w[Q];
-        const int jz = i - 1;
         if (p.invz) {
-            // inv(M_ii) and Z_i made by thin_prep_kernel: the oldest copy
-            // group, complete by the ring's first wait or the wait below
+            // inv(M_ii) and Z_i made by thin_prep_kernel
             const float* src = p.invz + (size_t)i * 2 * BR * LD;
             for (int e = t; e < BR * LD / 4; e += NT) {
                 cp_async16(sm.inv + 4 * e, src + 4 * e);
                 if (i > 0) cp_async16(sm.z + 4 * e, src + BR * LD + 4 * e);
             }
             cp_commit();
-        }
-#pragma unroll
-        for (int q = 0; q < STAGES - 1; ++q) {      // tiles 0 .. STAGES - 2
-            if (q < jz) issue_m(p, sm.m[(q + 1) % STAGES], i0, (int64_t)q * BR, colmajor);
-            else cp_commit();
-        }
-        if (!p.invz) {
+        } else {
             invert_diag(p, sm, i0);
             if (i > 0) make_z(p, sm, i0, colmajor);
         }
-        if (jz > 0) issue_x(p, pn, 0, w);
+        const auto release = [&](int s) {
+            __syncwarp();
+            if (t % 32 == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&sm.empty[s]))
+                             : "memory");
+        };
+        release(0);
+        // the nearest blocks are pushed here by the CTAs before this one in the
+        // cluster, X_j into slot i - 1 - j; blocks j < far come from xt
+        const int far = min(jz, i - min(rank, ND));
+        if (far > 0) issue_x(p, pn, 0, w);
         for (int j = 0; j < jz; ++j) {
-            cp_wait_ring();                               // this thread's copies of tile j
-            if (!finish_x(p, sm, pn, j, w)) sm.abort = 1;
-            __syncthreads();
+            const int s = (j + 1) % STAGES;
+            const bool ok = (j < far ? finish_x(p, sm.x[j & 1], pn, j, w)
+                                     : wait_bar(p, &sm.near_full[i - 1 - j], 0)) &&
+                            wait_bar(p, &sm.full[s], j / STAGES & 1);
+            if (!ok) sm.abort = 1;
+            sync_nt();   // also: X_j-1 is done with
             if (sm.abort) break;
-            // tile j - 1's stage is free: tile j + STAGES - 1 goes there
-            if (j + STAGES - 1 < jz)
-                issue_m(p, sm.m[j % STAGES], i0, (int64_t)(j + STAGES - 1) * BR, colmajor);
-            else cp_commit();
-            if (j + 1 < jz) issue_x(p, pn, j + 1, w);
-            mma_tile(sm.m[(j + 1) % STAGES], sm.x, BR, acc);
-            __syncthreads();
+            if (j + 1 < far) issue_x(p, pn, j + 1, w);
+            mma_tile(sm.m[s], j < far ? sm.x[j & 1] : sm.near[i - 1 - j], acc);
+            release(s);
         }
         if (sm.abort) break;
-        if (i > 0) issue_x(p, pn, i - 1, w);
+        if (i > 0 && rank == 0) issue_x(p, pn, i - 1, w);
         // P = inv(M_ii) (alpha B - S'), then X = P - Z X_i-1,p
+        float* rhs = sm.x[(i + 1) & 1];   // the last product (j = i - 2) reads the other
 #pragma unroll
-        for (int e = 0; e < 4; ++e) sm.x[(4 * ty + e) * NP + tx] = fmaf(p.alpha, b[e], -acc[e]);
+        for (int e = 0; e < 4; ++e)
+            rhs[(own.row + (e & 1)) * NP + own.col + (e >> 1)] =
+                fmaf(p.alpha, b[e & 1][e >> 1], -acc[e & 1][e >> 1]);
         if (p.invz) asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();
-        float xo[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        mma_tile(sm.inv, sm.x, 8 * ((t >> 5) + 1), xo);   // inv is lower: kk <= row
+        sync_nt();
+        float xo[2][2] = {};
+        mma_tile<true>(sm.inv, rhs, xo);
         if (i > 0) {
-            __syncthreads();
-            if (!finish_x(p, sm, pn, i - 1, w)) sm.abort = 1;
-            __syncthreads();
+            float* prev = sm.x[i & 1];
+            if (!(rank == 0 ? finish_x(p, prev, pn, i - 1, w) : wait_bar(p, &sm.near_full[0], 0))) sm.abort = 1;
+            sync_nt();
             if (sm.abort) break;
-            float zx[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-            mma_tile(sm.z, sm.x, BR, zx);
+            float zx[2][2] = {};
+            mma_tile(sm.z, rank == 0 ? prev : sm.near[0], zx);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) xo[e] -= zx[e];
+            for (int e = 0; e < 4; ++e) xo[e & 1][e >> 1] -= zx[e & 1][e >> 1];
         }
         // publish the block (tagged words: the chain), then the result in C
         unsigned long long* dst = p.xt + ((int64_t)pn * p.nbr + i) * (BR * NP);
         if (!(p.withhold && i == 0)) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-                st_relaxed64(dst + (4 * ty + e) * NP + tx, kTag | __float_as_uint(xo[e]));
+            for (int d = 1; d <= ND; ++d)
+                if (rank + d < CL && i + d < p.nbr) {
+#pragma unroll
+                    for (int r = 0; r < 2; ++r)
+                        push_near(sm, d - 1, rank + d, (own.row + r) * NP + own.col, xo[r][0],
+                                  xo[r][1]);
+                    if (t == 0)
+                        asm volatile("st.shared::cluster.s32 [%0], 1;" ::"r"(
+                                         map_rank(smem_u32(&sm.pushed[d - 1]), rank + d))
+                                     : "memory");
+                }
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+                st_relaxed64x2(dst + (own.row + r) * NP + own.col, kTag | __float_as_uint(xo[r][0]),
+                               kTag | __float_as_uint(xo[r][1]));
         }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const int64_t gi = i0 + 4 * ty + e, gj = c0 + tx;
-            if (gi < p.k && gj < p.nrhs) p.C[gi * p.c_rs + gj * p.c_cs] = xo[e];
+            const int64_t gi = i0 + own.row + (e & 1), gj = c0 + own.col + (e >> 1);
+            if (gi < p.k && gj < p.nrhs) p.C[gi * p.c_rs + gj * p.c_cs] = xo[e & 1][e >> 1];
         }
+        break;
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");   // nothing in flight at exit
+    __syncwarp();
+    // no CTA leaves while another may read its task or push to it, nor (after a
+    // timeout) before what was pushed has landed
+    cluster_sync();
+    if (t == 0)
+        for (int q = 0; q < ND; ++q)
+            if (*(volatile int*)&sm.pushed[q]) wait_landed(&sm.near_full[q]);
 }
 
 // ---- TRMM with few right-hand sides ---------------------------------------
@@ -514,7 +716,8 @@ __global__ void __launch_bounds__(NT, 2) thin_trmm_kernel(const Params p, const 
                                                           float* part, int* count) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SmemM& sm = *reinterpret_cast<SmemM*>(smem_raw);
-    const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
+    const int t = threadIdx.x;
+    const Own own = own_elements();
     const bool colmajor = p.a_rs == 1 || p.a_rs == -1;
     const int64_t total = pieces_upto(p.nbr - 1);
     while (true) {
@@ -557,7 +760,7 @@ __global__ void __launch_bounds__(NT, 2) thin_trmm_kernel(const Params p, const 
                 sm.d[cc * LD + rr] = v;
             }
         }
-        float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        float acc[2][2] = {};
         for (int j = jb; j < je; ++j) {
             cp_wait_ring();                          // this thread's copies of tile j
             __syncthreads();
@@ -565,7 +768,7 @@ __global__ void __launch_bounds__(NT, 2) thin_trmm_kernel(const Params p, const 
             if (j + STAGES - 1 < je)
                 issue_mb(p, sm, (j + STAGES - 1) % STAGES, i0, j + STAGES - 1, btiles, colmajor);
             else cp_commit();
-            mma_tile(sm.m[j % STAGES], sm.x[j % STAGES], BR, acc);
+            mma_tile(sm.m[j % STAGES], sm.x[j % STAGES], acc);
             __syncthreads();
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -575,13 +778,15 @@ __global__ void __launch_bounds__(NT, 2) thin_trmm_kernel(const Params p, const 
             *reinterpret_cast<float4*>(sm.x[0] + 4 * t) =
                 *reinterpret_cast<const float4*>(btiles + (int64_t)i * (BR * NP) + 4 * t);
             __syncthreads();
-            mma_tile(sm.d, sm.x[0], 8 * ((t >> 5) + 1), acc);   // lower: kk <= row
+            mma_tile<true>(sm.d, sm.x[0], acc);
         }
         if (np_i > 1) {
             // partial sums to this piece's slot; the last to arrive combines
             float* slots = part + ((int64_t)pn * total + pieces_upto(i - 1)) * (BR * NP);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) __stcg(slots + q * (BR * NP) + (4 * ty + e) * NP + tx, acc[e]);
+            for (int e = 0; e < 4; ++e)
+                __stcg(slots + q * (BR * NP) + (own.row + (e & 1)) * NP + own.col + (e >> 1),
+                       acc[e & 1][e >> 1]);
             __threadfence();
             __syncthreads();
             if (t == 0) sm.last = atomicAdd(count + (int64_t)pn * p.nbr + i, 1) == np_i - 1;
@@ -592,14 +797,14 @@ __global__ void __launch_bounds__(NT, 2) thin_trmm_kernel(const Params p, const 
             for (int e = 0; e < 4; ++e) {
                 float sum = 0.0f;
                 for (int64_t r = 0; r < np_i; ++r)
-                    sum += __ldcg(slots + r * (BR * NP) + (4 * ty + e) * NP + tx);
-                acc[e] = sum;
+                    sum += __ldcg(slots + r * (BR * NP) + (own.row + (e & 1)) * NP + own.col + (e >> 1));
+                acc[e & 1][e >> 1] = sum;
             }
         }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const int64_t gi = i0 + 4 * ty + e, gj = c0 + tx;
-            if (gi < p.k && gj < p.nrhs) p.C[gi * p.c_rs + gj * p.c_cs] = p.alpha * acc[e];
+            const int64_t gi = i0 + own.row + (e & 1), gj = c0 + own.col + (e >> 1);
+            if (gi < p.k && gj < p.nrhs) p.C[gi * p.c_rs + gj * p.c_cs] = p.alpha * acc[e & 1][e >> 1];
         }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -620,7 +825,7 @@ size_t thin_scratch_bytes(int64_t k, int64_t nrhs) {
            (npan > 1 ? (size_t)nbr * 2 * thin::BR * thin::LD * sizeof(float) : 0);
 }
 
-static int g_thin_ctas_per_sm = 0, g_thin_trmm_ctas_per_sm = 0;
+static int g_thin_trmm_ctas_per_sm = 0;
 
 cudaError_t thin_configure() {
     cudaError_t e0 = cudaFuncSetAttribute(thin::thin_trmm_kernel,
@@ -639,11 +844,6 @@ cudaError_t thin_configure() {
     e = cudaFuncSetAttribute(thin::thin_prep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sizeof(thin::Smem));
     if (e != cudaSuccess) return e;
-    int n = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, thin::thin_trsm_kernel, thin::NT,
-                                                      sizeof(thin::Smem));
-    if (e != cudaSuccess) return e;
-    g_thin_ctas_per_sm = n > 0 ? n : 1;
     return cudaSuccess;
 }
 
@@ -684,10 +884,9 @@ cudaError_t launch_thin_trsm(const Canon<float>& c, float alpha, int* scratch, i
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         p.invz = invz;
     }
-    const int per_sm = g_thin_ctas_per_sm > 0 ? g_thin_ctas_per_sm : 1;
-    const int64_t cap = (int64_t)num_sms * per_sm;
-    const int grid = (int)(p.ntask < cap ? p.ntask : cap);
-    thin::thin_trsm_kernel<<<grid, thin::NT, sizeof(thin::Smem), s>>>(p);
+    const int64_t clusters = (nbr + thin::CL - 1) / thin::CL * npan;
+    thin::thin_trsm_kernel<<<(unsigned)(clusters * thin::CL), thin::NT + thin::NTP,
+                             sizeof(thin::Smem), s>>>(p);
     return cudaGetLastError();
 }
 
