@@ -286,6 +286,7 @@ struct Exec {
     __nv_bfloat16* w_lo2 = nullptr;
     int* dag_flags = nullptr;      // device-scheduled TRSM: block flags + task counter
     int* thin_scratch = nullptr;   // thin TRSM: task counter, stop word, block flags
+    float* thin_invz = nullptr;    // thin leaves: all block rows' inverses and Z tiles
     // side R solved on B^T: B and its transpose in the workspace
     float *turn_b = nullptr, *turn_t = nullptr;
     int64_t turn_ldb = 0, turn_ldt = 0;
@@ -427,10 +428,19 @@ struct Exec {
                         tc.C += st.r0 * tc.c_rs;
                         tc.k = st.b;
                     }
+                    // the leaves' inverses and Z tiles: all by one pass before the first
+                    // leaf (15 us a leaf when each made its own)
+                    float* invz = nullptr;
+                    if (st.trsm && st.b > 0) {
+                        if (st.r0 == 0 &&
+                            (e = launch_thin_prep(*reinterpret_cast<const Canon<float>*>(&c),
+                                                  thin_invz, s)) != cudaSuccess)
+                            break;
+                        invz = thin_invz + thin_prep_bytes(st.r0) / sizeof(float);
+                    }
                     if (st.trsm)
-                        e = launch_thin_trsm(tc, (float)st.alpha, thin_scratch, h->d_err,
-                                             h->wait_ns, h->num_sms, s,
-                                             h->opt_test_withhold != 0);
+                        e = launch_thin_trsm(tc, (float)st.alpha, thin_scratch, invz, h->d_err,
+                                             h->wait_ns, s, h->opt_test_withhold != 0);
                     else
                         e = launch_thin_trmm(tc, (float)st.alpha, thin_scratch, h->num_sms, s);
                     if (e == cudaSuccess && st.b > 0 && st.planes && st.r0 + st.b < c.k)
@@ -595,7 +605,8 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
     plan.tc = !thin && tc_ok;
     const size_t thin_need = thin ? (trsm ? thin_scratch_bytes(k, ex.c.nrhs)
                                           : thin_trmm_scratch_bytes(k, ex.c.nrhs))
-                             : thin_leaf > 0 ? thin_scratch_bytes(thin_leaf, ex.c.nrhs)
+                             : thin_leaf > 0 ? thin_prep_bytes(k) +
+                                                   thin_scratch_bytes(thin_leaf, ex.c.nrhs)
                                              : 0;
     if (thin_need > 0 && h->thin_bytes < thin_need) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -620,6 +631,10 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
         }
     }
     ex.thin_scratch = (thin || thin_leaf > 0) ? h->thin_buf : nullptr;
+    if (thin_leaf > 0) {
+        ex.thin_invz = reinterpret_cast<float*>(h->thin_buf);
+        ex.thin_scratch += thin_prep_bytes(k) / sizeof(int);
+    }
     if (thin_leaf > 0) b = thin_leaf;
     plan.thin_leaf = thin_leaf > 0;
     // A prepared factor supplies the M planes (and its split): the workspace

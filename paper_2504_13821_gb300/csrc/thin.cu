@@ -813,16 +813,18 @@ __global__ void __launch_bounds__(NT, 2) thin_trmm_kernel(const Params p, const 
 }  // namespace thin
 
 // The thin TRSM's scratch: ticket and stop word (16 bytes), the tagged
-// words of every (block, panel), and with several panels the block rows'
-// inv / Z tiles.
+// words of every (block, panel); with several panels also the block rows' inv / Z
+// tiles.
 static size_t thin_words_bytes(int64_t nbr, int64_t npan) {
     return 16 + (size_t)(nbr * npan) * kThinBlock * kThinPanel * 8;
+}
+size_t thin_prep_bytes(int64_t k) {
+    return (size_t)((k + kThinBlock - 1) / kThinBlock) * 2 * thin::BR * thin::LD * sizeof(float);
 }
 size_t thin_scratch_bytes(int64_t k, int64_t nrhs) {
     const int64_t nbr = (k + kThinBlock - 1) / kThinBlock;
     const int64_t npan = (nrhs + kThinPanel - 1) / kThinPanel;
-    return thin_words_bytes(nbr, npan) +
-           (npan > 1 ? (size_t)nbr * 2 * thin::BR * thin::LD * sizeof(float) : 0);
+    return thin_words_bytes(nbr, npan) + (npan > 1 ? thin_prep_bytes(k) : 0);
 }
 
 static int g_thin_trmm_ctas_per_sm = 0;
@@ -847,10 +849,8 @@ cudaError_t thin_configure() {
     return cudaSuccess;
 }
 
-cudaError_t launch_thin_trsm(const Canon<float>& c, float alpha, int* scratch, int* err,
-                             long long wait_ns, int num_sms, cudaStream_t s, bool withhold) {
-    if (c.k <= 0 || c.nrhs <= 0) return cudaSuccess;
-    thin::Params p;
+static thin::Params thin_params(const Canon<float>& c, float alpha) {
+    thin::Params p{};
     p.k = c.k;
     p.nrhs = c.nrhs;
     p.A = c.A;
@@ -861,11 +861,24 @@ cudaError_t launch_thin_trsm(const Canon<float>& c, float alpha, int* scratch, i
     p.c_cs = c.c_cs;
     p.alpha = alpha;
     p.unit = c.unit ? 1 : 0;
+    p.nbr = (int)((c.k + kThinBlock - 1) / kThinBlock);
+    p.npan = (int)((c.nrhs + kThinPanel - 1) / kThinPanel);
+    return p;
+}
+
+cudaError_t launch_thin_prep(const Canon<float>& c, float* invz, cudaStream_t s) {
+    const thin::Params p = thin_params(c, 1.0f);
+    thin::thin_prep_kernel<<<(unsigned)p.nbr, thin::NT, sizeof(thin::Smem), s>>>(p, invz);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_thin_trsm(const Canon<float>& c, float alpha, int* scratch, const float* invz,
+                             int* err, long long wait_ns, cudaStream_t s, bool withhold) {
+    if (c.k <= 0 || c.nrhs <= 0) return cudaSuccess;
     const int64_t nbr = (c.k + kThinBlock - 1) / kThinBlock;
     const int64_t npan = (c.nrhs + kThinPanel - 1) / kThinPanel;
     if (nbr * npan > (int64_t)1 << 30) return cudaErrorInvalidValue;
-    p.nbr = (int)nbr;
-    p.npan = (int)npan;
+    thin::Params p = thin_params(c, alpha);
     p.ntask = nbr * npan;
     p.ticket = scratch;
     p.stop = scratch + 1;
@@ -873,17 +886,16 @@ cudaError_t launch_thin_trsm(const Canon<float>& c, float alpha, int* scratch, i
     p.err = err;
     p.wait_ns = wait_ns;
     p.withhold = withhold ? 1 : 0;
-    p.invz = nullptr;
     // the words (and ticket) are zeroed every launch; inv / Z are written
     cudaError_t e = cudaMemsetAsync(scratch, 0, thin_words_bytes(nbr, npan), s);
     if (e != cudaSuccess) return e;
-    if (npan > 1) {
-        float* invz = reinterpret_cast<float*>(reinterpret_cast<char*>(scratch) +
-                                               thin_words_bytes(nbr, npan));
-        thin::thin_prep_kernel<<<(unsigned)nbr, thin::NT, sizeof(thin::Smem), s>>>(p, invz);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        p.invz = invz;
+    if (npan > 1 && invz == nullptr) {
+        float* own = reinterpret_cast<float*>(reinterpret_cast<char*>(scratch) +
+                                              thin_words_bytes(nbr, npan));
+        if ((e = launch_thin_prep(c, own, s)) != cudaSuccess) return e;
+        invz = own;
     }
+    p.invz = invz;
     const int64_t clusters = (nbr + thin::CL - 1) / thin::CL * npan;
     thin::thin_trsm_kernel<<<(unsigned)(clusters * thin::CL), thin::NT + thin::NTP,
                              sizeof(thin::Smem), s>>>(p);
@@ -906,23 +918,11 @@ size_t thin_trmm_scratch_bytes(int64_t k, int64_t nrhs) {
 cudaError_t launch_thin_trmm(const Canon<float>& c, float alpha, int* scratch, int num_sms,
                              cudaStream_t s) {
     if (c.k <= 0 || c.nrhs <= 0) return cudaSuccess;
-    thin::Params p{};
-    p.k = c.k;
-    p.nrhs = c.nrhs;
-    p.A = c.A;
-    p.a_rs = c.a_rs;
-    p.a_cs = c.a_cs;
-    p.C = c.C;
-    p.c_rs = c.c_rs;
-    p.c_cs = c.c_cs;
-    p.alpha = alpha;
-    p.unit = c.unit ? 1 : 0;
     const int64_t nbr = (c.k + kThinBlock - 1) / kThinBlock;
     const int64_t npan = (c.nrhs + kThinPanel - 1) / kThinPanel;
     const int64_t total = thin::pieces_upto(nbr - 1);
     if (total * npan > (int64_t)1 << 30) return cudaErrorInvalidValue;
-    p.nbr = (int)nbr;
-    p.npan = (int)npan;
+    thin::Params p = thin_params(c, alpha);
     p.ntask = total * npan;
     p.ticket = scratch;
     int* count = scratch + 4;
