@@ -235,11 +235,11 @@ def auto_path_desc(k, n):
     thin_leaf_rows, the leaf kernel by right-hand-side count) run for FP32
     side-L TRSM and TRMM of order k with n right-hand sides."""
     thin_leaf = 0
-    if k >= 4096 and 64 < n <= 1024 and not (n <= 128 and k < 8192):
-        thin_leaf = 2048 if n <= 256 else 1024
+    if k >= 1024 and 64 < n <= 1536 and k * n >= 1 << 20:
+        thin_leaf = 2048 if n <= 256 else 1024 if n <= 1024 else 512
     if thin_leaf and k > thin_leaf:
         trsm = f"TRSM leaves of {thin_leaf} rows as thin solves (64-row blocks, 16-column panels)"
-    elif k > 256 and (n <= 64 or (n <= 256 and k * n <= 1 << 21)):
+    elif (k > 256 and n <= 64) or (k >= 256 and n <= min(1536, 4 * k) and k * n <= 1 << 20):
         trsm = "TRSM as one thin solve (64-row blocks, 16-column panels, one launch)"
     else:
         trsm = f"TRSM 128 ({'wide leaf' if n >= 1024 else 'lane-split leaf'})"

@@ -108,7 +108,9 @@ enum {
                               cached CUDA graph; 0: launch directly         */
     TRX_OPT_PROFILE = 4,   /* 1: time every launch with CUDA events and
                               accumulate into trx_profile_t (launches
-                              directly, no graph); 0 (default): off        */
+                              directly, no graph; FP32 TRSM keeps to the
+                              recursion where only the wider automatic rule
+                              of TRX_OPT_THIN would not); 0 (default): off */
     TRX_OPT_WAIT_LIMIT = 5,/* nanoseconds a device-side wait may spin
                               before it gives up and the launch reports
                               TRX_ERR_TIMEOUT (default 2e9, minimum 1000) */
@@ -230,11 +232,15 @@ enum {
                               TRMM: every block row's sum from a packed copy
                               of B, long rows in pieces added in a fixed
                               order, no waits; FP32 FMA, no operand split);
-                              -1 = the recursion; 0 = automatic (default:
-                              order above 256; TRSM with at most 64
-                              right-hand sides, or at most 256 while order
-                              x right-hand sides <= 2^21 and the thin
-                              leaves of TRX_OPT_THIN_LEAF do not apply;
+                              -1 = the recursion; 0 = automatic (default):
+                              TRSM of order above 256 with at most 64
+                              right-hand sides, of order 256 on with at most
+                              1536, four times the order, while order x
+                              right-hand sides <= 2^20 (where a leaf, GEMM,
+                              split, panel, DAG or profile option is set:
+                              above 256 with at most 256 while it is <=
+                              2^21), and the thin leaves of
+                              TRX_OPT_THIN_LEAF do not apply;
                               TRMM with at most 32). Its scratch lives in a
                               handle buffer grown on first use (cached
                               graphs are dropped when it grows)           */
@@ -252,9 +258,13 @@ enum {
                               rows, its result converted to the GEMM
                               operand planes for the updates after it;
                               -1 = off; 0 = automatic (default: from
-                              order 4096, leaves of 2048 rows for 65 .. 256
-                              right-hand sides (129 .. 256 below order
-                              8192), of 1024 rows for 257 .. 1024; off
+                              order 1024 and order x right-hand sides 2^20
+                              on, leaves of 2048 rows for 65 .. 256
+                              right-hand sides, of 1024 for 257 .. 1024, of
+                              512 for 1025 .. 1536; where one of the options
+                              named there is set from order 4096, for 65 ..
+                              256 (129 .. 256 below order 8192) and 257 ..
+                              1024 right-hand sides; off
                               when TRX_OPT_LEAF sets the cutoff). Where
                               this and an automatic whole-call
                               thin solve (TRX_OPT_THIN 0) both apply, the

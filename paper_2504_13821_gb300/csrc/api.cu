@@ -589,12 +589,19 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
     // in a handle buffer, grown here (never inside a stream capture: a
     // capture keeps the recursive chain with the ordinary leaves).
     const bool tc_ok = use_tc<T>(h, k, trsm, ex.c.nrhs);
+    // (a profile is of the recursion's kernel classes: it keeps the narrower rule)
+    const bool automatic = tc_ok && !ex.profile && h->opt_leaf == 0 && h->opt_gemm == 0 &&
+                           h->opt_panels == 0 &&
+                           h->opt_trsm_dag == 0 && h->opt_trsm_tc_leaf == 0 &&
+                           h->opt_thin_leaf == 0 && terms_override == 0 && slices_for(h) == 3;
     bool thin = std::is_same<T, float>::value &&
-                use_thin_mode(h->opt_thin, trsm, (int)sizeof(T), k, ex.c.nrhs);
+                use_thin_mode(h->opt_thin, trsm, (int)sizeof(T), k, ex.c.nrhs,
+                              automatic && h->opt_thin == 0);
     // (an explicit leaf size turns the automatic thin leaves off)
     const int64_t tl_opt = (h->opt_leaf != 0 && h->opt_thin_leaf == 0) ? -1 : h->opt_thin_leaf;
     int thin_leaf = std::is_same<T, float>::value
-                        ? thin_leaf_rows(tl_opt, tc_ok, trsm, (int)sizeof(T), k, ex.c.nrhs)
+                        ? thin_leaf_rows(tl_opt, tc_ok, trsm, (int)sizeof(T), k, ex.c.nrhs,
+                                         automatic && h->opt_thin == 0)
                         : 0;
     // both apply: a forced whole-call solve wins, else the thin leaves
     if (thin && thin_leaf > 0) {
@@ -655,7 +662,7 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
         }
         char* base = static_cast<char*>(h->ws);
         if constexpr (std::is_same<T, float>::value) {
-            if (upc(side) == 'R' && !dag && !plan.thin_leaf && h->opt_panels <= 1 &&
+            if (upc(side) == 'R' && !dag && h->opt_panels <= 1 &&
                 turn_applies(k, ex.c.nrhs) &&
                 h->ws_bytes >= need + turn_bytes(k, ex.c.nrhs)) {
                 ex.turn_b = B;
@@ -2393,7 +2400,8 @@ int trx_debug_plan(char op, char side, char uplo, char transa, char diag, int64_
     Plan plan;
     plan.tc = use_tc_mode(elem_bytes, gemm_mode, k, b);
     const int tl = thin_leaf_rows((leaf != 0 && thin_leaf == 0) ? -1 : thin_leaf, plan.tc,
-                                  is_trsm, elem_bytes, k, nrhs);
+                                  is_trsm, elem_bytes, k, nrhs,
+                                  leaf == 0 && gemm_mode == 0 && trsm_tc_leaf == 0);
     if (tl > 0) b = tl;
     plan.thin_leaf = tl > 0;
     plan.tc_leaf = is_trsm && elem_bytes == 4 && !plan.thin_leaf &&

@@ -385,40 +385,66 @@ inline bool use_dag_mode(int64_t opt, bool tc, bool trsm, int elem, int64_t k, i
 // 0 automatic): automatically for FP32 TRSM of order above kThinMinK with
 // at most kThinMaxNrhs right-hand sides, or up to kThinWideNrhs of them
 // while order x right-hand sides stays within kThinMaxWork, where the
-// chain's launch and leaf latency bound the recursive path (measured on
-// GB300: 1.04-4.2x faster there; at order 16384 with 256 right-hand sides
-// the chain's tensor-core updates win). Where the thin leaves below also
-// apply automatically, the call takes those instead (execute in api.cu).
+// chain's launch and leaf latency bound the recursive path. Where the thin leaves
+// below also apply automatically, the call takes those instead (execute in api.cu).
 constexpr int64_t kThinMaxNrhs = 64, kThinWideNrhs = 256;
 constexpr int64_t kThinMaxWork = (int64_t)1 << 21;
 constexpr int64_t kThinMinK = 256;
+// Where every option is automatic and the operands keep all three planes: from order
+// 256 on up to kThinAutoNrhs right-hand sides, four times the order at most, the
+// whole call while order x right-hand sides is within kThinAutoWork (the chain's
+// leaves, 16-32 us each whatever their right-hand sides, are its time there), the
+// thin leaves from there on from order 1024 on. Measured (us, order x right-hand
+// sides, side L and R; chain / whole call / leaves of 512, 1024 and 2048 rows):
+//   256 x 256     L 50 / 48                    R 66 / 47
+//   256 x 1000    L 53 / 54                    R 68 / 55
+//   512 x 512     L 83 / 57                    R 110 / 57
+//   1000 x 400    L 148 / 84 / 93              R 201 / 88 / 102
+//   1000 x 1000   L 157 / 131 / 130            R 207 / 138 / 137
+//   768 x 1500    L 128 / 139 / 133            R 174 / 146 / 144
+//   2048 x 512    L 293 / 174 / 172 / 163      R 390 / 201 / 178 / 180
+//   2048 x 1500   L 339 / 395 / 307 / 332      R 450 / 463 / 337 / 372
+//   2000 x 2000   L 345 / - / 384 / 418
+//   4096 x 256    L 615 / 276 / 326 / 269 / 260
+//   4096 x 1000   L 659 / 845 / 502 / 521 / 618
+//   8192 x 80     L - / 368 / 671 / 530 / 467
+//   8192 x 512    L 1352 / - / 804 / 766 / 843
+constexpr int64_t kThinAutoNrhs = 1536, kThinAutoK = 256, kThinAutoLeafK = 1024;
+constexpr int64_t kThinAutoWork = (int64_t)1 << 20;
 // TRMM (thin.cu's one-launch product): automatically with at most
 // kThinTrmmMaxNrhs right-hand sides above order kThinMinK (measured on
 // GB300: 1.1-2.9x the recursion's grouped product up to 32 right-hand
 // sides; from 64 on the tensor-core product is as fast or faster).
 constexpr int64_t kThinTrmmMaxNrhs = 32;
-inline bool use_thin_mode(int64_t opt, bool trsm, int elem, int64_t k, int64_t nrhs) {
+inline bool use_thin_mode(int64_t opt, bool trsm, int elem, int64_t k, int64_t nrhs,
+                          bool automatic = false) {
     if (opt < 0 || elem != 4 || k <= 0 || nrhs <= 0) return false;
     if (opt > 0) return true;
     if (!trsm) return k > kThinMinK && nrhs <= kThinTrmmMaxNrhs;
+    if (automatic && k >= kThinAutoK && nrhs <= std::min(kThinAutoNrhs, 4 * k) &&
+        k * nrhs <= kThinAutoWork)
+        return true;
     return k > kThinMinK &&
            (nrhs <= kThinMaxNrhs || (nrhs <= kThinWideNrhs && k * nrhs <= kThinMaxWork));
 }
 
 // Leaves of the recursion as thin solves (TRX_OPT_THIN_LEAF: -1 off, a row
 // count 256 .. 8192 (multiple of 128) on, 0 automatic): FP32 TRSM on the
-// tensor-core path whose order exceeds the leaf. Automatically from order
-// kThinLeafMinK: leaves of 2048 rows for 65 .. 256 right-hand sides (from
-// order 8192 when there are at most 128: below it the whole-call thin solve
-// is faster), of 1024 rows for 257 .. 1024 (measured on GB300 against the
-// chain of 128-row leaves and the whole-call thin solve: 1.57x the chain at
-// order 16384 with 256 right-hand sides, 1.56x the whole-call thin solve
-// with 128, 1.13-1.3x the chain at 512 and 1024). Returns the leaf rows, or
-// 0.
+// tensor-core path whose order exceeds the leaf. Automatically where the table above
+// says, or (some other option set) from order kThinLeafMinK: leaves of 2048 rows for
+// 65 .. 256 right-hand sides (from order 8192 when there are at most 128: below it
+// the whole-call thin solve is faster), of 1024 rows for 257 .. 1024. Returns the
+// leaf rows, or 0.
 constexpr int64_t kThinLeafMinK = 4096;
-inline int thin_leaf_rows(int64_t opt, bool tc, bool trsm, int elem, int64_t k, int64_t nrhs) {
+inline int thin_leaf_rows(int64_t opt, bool tc, bool trsm, int elem, int64_t k, int64_t nrhs,
+                          bool automatic = false) {
     if (opt < 0 || !tc || !trsm || elem != 4) return 0;
     if (opt > 0) return k > opt ? (int)opt : 0;
+    if (automatic && nrhs > kThinMaxNrhs) {
+        if (k < kThinAutoLeafK || nrhs > kThinAutoNrhs || k * nrhs < kThinAutoWork) return 0;
+        const int rows = nrhs <= kThinWideNrhs ? 2048 : nrhs <= 1024 ? 1024 : 512;
+        return k > rows ? rows : 0;
+    }
     if (k < kThinLeafMinK || nrhs <= kThinMaxNrhs || nrhs > 1024) return 0;
     if (nrhs <= 128 && k < 2 * kThinLeafMinK) return 0;
     return nrhs <= kThinWideNrhs ? 2048 : 1024;
