@@ -34,8 +34,10 @@
 // Staging: the triangle and the panel arrive by cp.async (one memory round
 // trip, no registers held); alpha is applied where the panel is first read.
 // Write-back: a lane stores 8 rows x 4 columns of the panel, each column's
-// 8 rows as 16-byte vectors of C and of every Y plane (packed BF16
-// conversions), where the addresses line up; else one element per lane.
+// 8 rows as 16-byte vectors of every Y plane (packed BF16 conversions) and of C where
+// its addresses line up, forwards or reversed; else C goes one element per lane. (With
+// the planes' vectors tied to C's: 2000 x 2000 reversed 389 us against 324, order 2001
+// 406 against 321.)
 //
 // The chunk-to-warp map is rotated by the group index, so each of the SM's
 // four warp schedulers (warp w runs on w % 4) holds one warp of every chunk,
@@ -56,7 +58,8 @@ struct Wide {
     static constexpr int NT = GROUPS * GT;
     static constexpr int NC = 32;                 // columns per panel
     static constexpr int LDC = NC + 4;            // panel row stride (16-byte rows)
-    static constexpr size_t smem = sizeof(float) * ((size_t)B * B + B + (size_t)GROUPS * B * LDC);
+    static constexpr int LDT = B + 4;             // triangle column stride (see its staging)
+    static constexpr size_t smem = sizeof(float) * ((size_t)B * LDT + B + (size_t)GROUPS * B * LDC);
 };
 
 // Packed FP32 pairs (Blackwell's f32x2 FMA: two independent
@@ -132,8 +135,8 @@ __global__ void __launch_bounds__(Wide::NT, 1) leaf_trsm_wide_kernel(LeafArgs<fl
                                                                    int64_t npanels) {
     using S = Wide;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float* sT = reinterpret_cast<float*>(smem_raw);   // M(r0+i, r0+l) at l*B + i (i > l, else 0)
-    float* sD = sT + S::B * S::B;                       // reciprocal diagonal (1: unit / ragged)
+    float* sT = reinterpret_cast<float*>(smem_raw);   // M(r0+i, r0+l) at l*LDT + i (i > l)
+    float* sD = sT + S::B * S::LDT;                      // reciprocal diagonal (1: unit / ragged)
     const int tid = threadIdx.x, g = tid / S::GT, gt = tid % S::GT;
     float* sC = sD + S::B + (size_t)g * S::B * S::LDC;  // this group's panel: row i at i*LDC
     pdl_trigger();
@@ -175,7 +178,11 @@ __global__ void __launch_bounds__(Wide::NT, 1) leaf_trsm_wide_kernel(LeafArgs<fl
     if (panel < npanels) fetch_panel(panel * S::NC);
 
     // Triangle, read along A's contiguous index; its copies are in flight
-    // together with the first panel's.
+    // together with the first panel's. Only what lies below the diagonal is read or
+    // used. Where the rows of M are contiguous a warp's words go to 32 columns: 4
+    // words of padding spread them over 8 banks (with none they all met in one: order
+    // 2000, 2000 right-hand sides, side R 442 us against 346, upper transposed 442
+    // against 329).
     {
         const bool a_row_fast = (p.a_rs == 1 || p.a_rs == -1);
         constexpr int ADV = S::NT / S::B;          // 4
@@ -188,8 +195,7 @@ __global__ void __launch_bounds__(Wide::NT, 1) leaf_trsm_wide_kernel(LeafArgs<fl
         for (int u = 0; u < TP; ++u) {
             const int w = first + u * ADV;
             const int i = a_row_fast ? fixed : w, l = a_row_fast ? w : fixed;
-            const bool in = i < bs && l < i;
-            cp_async4(sT + l * S::B + i, in ? src + (int64_t)u * ADV * st_walk : p.A, in);
+            if (i < bs && l < i) cp_async4(sT + l * S::LDT + i, src + (int64_t)u * ADV * st_walk, true);
         }
         if (tid < S::B)
             sD[tid] = (tid < bs && !p.unit) ? 1.f / p.A[(r0 + tid) * (p.a_rs + p.a_cs)] : 1.f;
@@ -206,7 +212,7 @@ __global__ void __launch_bounds__(Wide::NT, 1) leaf_trsm_wide_kernel(LeafArgs<fl
     // in place; column jj+1 of the block's M is loaded (four 16-byte
     // broadcasts) while column jj is applied.
     auto solve_block = [&](float (&v)[S::SB], int s0) {
-        const float* mcol = sT + s0 * S::B + s0;      // M(s0+q, s0+jj) at jj*B + q
+        const float* mcol = sT + s0 * S::LDT + s0;    // M(s0+q, s0+jj) at jj*LDT + q
         float4 cur[4], nxt[4];
 #pragma unroll
         for (int w = 0; w < 4; ++w) cur[w] = *reinterpret_cast<const float4*>(mcol + 4 * w);
@@ -215,7 +221,7 @@ __global__ void __launch_bounds__(Wide::NT, 1) leaf_trsm_wide_kernel(LeafArgs<fl
             if (jj + 1 < S::SB) {
 #pragma unroll
                 for (int w = 0; w < 4; ++w)
-                    nxt[w] = *reinterpret_cast<const float4*>(mcol + (jj + 1) * S::B + 4 * w);
+                    nxt[w] = *reinterpret_cast<const float4*>(mcol + (jj + 1) * S::LDT + 4 * w);
             }
             const float m[16] = {cur[0].x, cur[0].y, cur[0].z, cur[0].w,
                                  cur[1].x, cur[1].y, cur[1].z, cur[1].w,
@@ -234,9 +240,11 @@ __global__ void __launch_bounds__(Wide::NT, 1) leaf_trsm_wide_kernel(LeafArgs<fl
                        (reinterpret_cast<uintptr_t>(a.pl.y_lo) & 15) == 0 &&
                        (reinterpret_cast<uintptr_t>(a.pl.y_lo2) & 15) == 0 &&
                        (a.pl.ldy & 7) == 0 && (r0 & 7) == 0;
-    const bool c_vec = !ROWS || (p.c_rs == 1 && (reinterpret_cast<uintptr_t>(p.C) & 15) == 0 &&
-                                 (p.c_cs & 3) == 0 && (r0 & 3) == 0);
-    const bool vec_wb = y_vec && c_vec;
+    // (reversed rows: the eight lie in descending order below row i0's address)
+    const int c_vec = !ROWS || (p.c_cs & 3) != 0                                              ? 0
+                      : p.c_rs == 1 && (reinterpret_cast<uintptr_t>(p.C + r0) & 15) == 0      ? 1
+                      : p.c_rs == -1 && (reinterpret_cast<uintptr_t>(p.C - r0 - 7) & 15) == 0 ? -1
+                                                                                              : 0;
 
 #pragma unroll 1
     for (bool first = true; panel < npanels; panel += pstride, first = false) {
@@ -285,13 +293,13 @@ __global__ void __launch_bounds__(Wide::NT, 1) leaf_trsm_wide_kernel(LeafArgs<fl
                 for (int h = 0; h < S::SB / 2; ++h)
                     v2[h] = pack2(sc * sC[(t0 + 2 * h) * S::LDC + lane],
                                   sc * sC[(t0 + 2 * h + 1) * S::LDC + lane]);
-                const float* mb = sT + s0 * S::B + t0;   // M(t0+q, s0+kk) at kk*B + q
+                const float* mb = sT + s0 * S::LDT + t0; // M(t0+q, s0+kk) at kk*LDT + q
 #pragma unroll
                 for (int kk = 0; kk < S::SB; ++kk) {
-                    const float4 m0 = *reinterpret_cast<const float4*>(mb + kk * S::B);
-                    const float4 m1 = *reinterpret_cast<const float4*>(mb + kk * S::B + 4);
-                    const float4 m2 = *reinterpret_cast<const float4*>(mb + kk * S::B + 8);
-                    const float4 m3 = *reinterpret_cast<const float4*>(mb + kk * S::B + 12);
+                    const float4 m0 = *reinterpret_cast<const float4*>(mb + kk * S::LDT);
+                    const float4 m1 = *reinterpret_cast<const float4*>(mb + kk * S::LDT + 4);
+                    const float4 m2 = *reinterpret_cast<const float4*>(mb + kk * S::LDT + 8);
+                    const float4 m3 = *reinterpret_cast<const float4*>(mb + kk * S::LDT + 12);
                     const uint64_t xn = pack2(-xs[kk], -xs[kk]);
                     v2[0] = ffma2(pack2(m0.x, m0.y), xn, v2[0]);
                     v2[1] = ffma2(pack2(m0.z, m0.w), xn, v2[1]);
@@ -313,8 +321,8 @@ __global__ void __launch_bounds__(Wide::NT, 1) leaf_trsm_wide_kernel(LeafArgs<fl
                 for (int kk = 0; kk < S::SB; ++kk) {
                     const int l = s0 + kk;
                     const float4 xv = *reinterpret_cast<const float4*>(sC + l * S::LDC + 4 * cg);
-                    const float4 t0v = *reinterpret_cast<const float4*>(sT + l * S::B + 8 * rg);
-                    const float4 t1v = *reinterpret_cast<const float4*>(sT + l * S::B + 8 * rg + 4);
+                    const float4 t0v = *reinterpret_cast<const float4*>(sT + l * S::LDT + 8 * rg);
+                    const float4 t1v = *reinterpret_cast<const float4*>(sT + l * S::LDT + 8 * rg + 4);
                     const uint64_t tp[4] = {pack2(t0v.x, t0v.y), pack2(t0v.z, t0v.w),
                                             pack2(t1v.x, t1v.y), pack2(t1v.z, t1v.w)};
                     const uint64_t xb[4] = {pack2(xv.x, xv.x), pack2(xv.y, xv.y),
@@ -342,7 +350,7 @@ __global__ void __launch_bounds__(Wide::NT, 1) leaf_trsm_wide_kernel(LeafArgs<fl
         group_sync(g);   // the last block solved is visible: every row is final
 
         // Write back (and the Y planes on the tensor-core path).
-        if (vec_wb) {
+        if (y_vec) {
             // lane: rows 8ro..8ro+7 x columns 4c4..4c4+3 (a warp: 32 rows)
             const int ro = 4 * (gt >> 5) + (lane >> 3), c4 = lane & 7;
             const int i0 = 8 * ro;
@@ -361,21 +369,33 @@ __global__ void __launch_bounds__(Wide::NT, 1) leaf_trsm_wide_kernel(LeafArgs<fl
                         v[e] = cc == 0 ? w[e].x : cc == 1 ? w[e].y : cc == 2 ? w[e].z : w[e].w;
                     if (i0 + 8 <= bs) {
                         put_y8(a.pl, (j0 + c) * a.pl.ldy + r0 + i0, v);
-                        if constexpr (ROWS) {
+                        if (ROWS && c_vec > 0) {
                             float* dst = p.C + (r0 + i0) + (j0 + c) * p.c_cs;
                             *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
                             *reinterpret_cast<float4*>(dst + 4) = make_float4(v[4], v[5], v[6], v[7]);
+                        } else if (ROWS && c_vec < 0) {
+                            float* dst = p.C - (r0 + i0 + 7) + (j0 + c) * p.c_cs;
+                            *reinterpret_cast<float4*>(dst) = make_float4(v[7], v[6], v[5], v[4]);
+                            *reinterpret_cast<float4*>(dst + 4) = make_float4(v[3], v[2], v[1], v[0]);
                         }
                     } else {
 #pragma unroll 1
                         for (int e = 0; e < 8 && i0 + e < bs; ++e) {
                             put_y(a.pl, (j0 + c) * a.pl.ldy + r0 + i0 + e, v[e]);
-                            if constexpr (ROWS) p.C[(r0 + i0 + e) + (j0 + c) * p.c_cs] = v[e];
+                            if (ROWS && c_vec != 0)
+                                p.C[(r0 + i0 + e) * p.c_rs + (j0 + c) * p.c_cs] = v[e];
                         }
                     }
                 }
             }
-            if constexpr (!ROWS) {
+            if constexpr (ROWS) {
+                // unaligned columns: a lane per row
+                if (c_vec == 0 && gt < bs) {
+                    float* dst = p.C + (r0 + gt) * p.c_rs + j0 * p.c_cs;
+#pragma unroll 8
+                    for (int c = 0; c < ncols; ++c) dst[(int64_t)c * p.c_cs] = sC[gt * S::LDC + c];
+                }
+            } else {
                 const int c = gt & 31, ii = gt >> 5;
                 if (c < ncols) {
 #pragma unroll 4
