@@ -391,25 +391,28 @@ constexpr int64_t kThinMaxNrhs = 64, kThinWideNrhs = 256;
 constexpr int64_t kThinMaxWork = (int64_t)1 << 21;
 constexpr int64_t kThinMinK = 256;
 // Where every option is automatic and the operands keep all three planes: from order
-// 256 on up to kThinAutoNrhs right-hand sides, four times the order at most, the
+// 256 on up to kThinAutoWhole right-hand sides, four times the order at most, the
 // whole call while order x right-hand sides is within kThinAutoWork (the chain's
-// leaves, 16-32 us each whatever their right-hand sides, are its time there), the
-// thin leaves from there on from order 1024 on. Measured (us, order x right-hand
-// sides, side L and R; chain / whole call / leaves of 512, 1024 and 2048 rows):
+// leaves, 10-32 us each whatever their right-hand sides, are its time there); from
+// there on, and from order 1024 on, the thin leaves up to kThinAutoNrhs. Measured
+// (us, order x right-hand sides, side L and R; chain / whole call / leaves of 512,
+// 1024 and 2048 rows):
 //   256 x 256     L 50 / 48                    R 66 / 47
 //   256 x 1000    L 53 / 54                    R 68 / 55
 //   512 x 512     L 83 / 57                    R 110 / 57
 //   1000 x 400    L 148 / 84 / 93              R 201 / 88 / 102
 //   1000 x 1000   L 157 / 131 / 130            R 207 / 138 / 137
-//   768 x 1500    L 128 / 139 / 133            R 174 / 146 / 144
+//   640 x 1500    L 111 / 124                  R 114 / 132
+//   1024 x 1536   L 161 / - / 156              R 170 / - / 171
 //   2048 x 512    L 293 / 174 / 172 / 163      R 390 / 201 / 178 / 180
-//   2048 x 1500   L 339 / 395 / 307 / 332      R 450 / 463 / 337 / 372
-//   2000 x 2000   L 345 / - / 384 / 418
+//   2048 x 1536   L 332 / - / 307 / 337        R 344 / - / 337 / 386
+//   2000 x 2000   L 325 / - / 384 / 418
 //   4096 x 256    L 615 / 276 / 326 / 269 / 260
 //   4096 x 1000   L 659 / 845 / 502 / 521 / 618
 //   8192 x 80     L - / 368 / 671 / 530 / 467
 //   8192 x 512    L 1352 / - / 804 / 766 / 843
-constexpr int64_t kThinAutoNrhs = 1536, kThinAutoK = 256, kThinAutoLeafK = 1024;
+constexpr int64_t kThinAutoWhole = 1024, kThinAutoNrhs = 1536;
+constexpr int64_t kThinAutoK = 256, kThinAutoLeafK = 1024;
 constexpr int64_t kThinAutoWork = (int64_t)1 << 20;
 // TRMM (thin.cu's one-launch product): automatically with at most
 // kThinTrmmMaxNrhs right-hand sides above order kThinMinK (measured on
@@ -421,7 +424,7 @@ inline bool use_thin_mode(int64_t opt, bool trsm, int elem, int64_t k, int64_t n
     if (opt < 0 || elem != 4 || k <= 0 || nrhs <= 0) return false;
     if (opt > 0) return true;
     if (!trsm) return k > kThinMinK && nrhs <= kThinTrmmMaxNrhs;
-    if (automatic && k >= kThinAutoK && nrhs <= std::min(kThinAutoNrhs, 4 * k) &&
+    if (automatic && k >= kThinAutoK && nrhs <= std::min(kThinAutoWhole, 4 * k) &&
         k * nrhs <= kThinAutoWork)
         return true;
     return k > kThinMinK &&

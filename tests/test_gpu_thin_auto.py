@@ -1,5 +1,5 @@
 """The automatic thin solve and thin leaves around their lines (order 256 and 1024,
-1536 right-hand sides, four times the order, 2^20 elements): both sides, forward and
+1024 and 1536 right-hand sides, four times the order, 2^20 elements): both sides, forward and
 reversed, plain calls, a prepared factor and capture of a call that has not run before,
 against the FP64 oracle; an explicit option keeps the recursion."""
 import numpy as np
