@@ -294,6 +294,7 @@ struct Exec {
     void* oz_ws = nullptr;         // FP64 updates on the tensor cores: operand images
     cudaStream_t s;
     bool profile;
+    bool same_a = false;
 
     // NVTX range name of a step (TRX_OPT_NVTX): kind and its row ranges
     static void nvtx_push(const Step& st) {
@@ -432,15 +433,15 @@ struct Exec {
                     // leaf (15 us a leaf when each made its own)
                     float* invz = nullptr;
                     if (st.trsm && st.b > 0) {
-                        if (st.r0 == 0 &&
+                        if (st.r0 == 0 && !same_a &&
                             (e = launch_thin_prep(*reinterpret_cast<const Canon<float>*>(&c),
                                                   thin_invz, s)) != cudaSuccess)
                             break;
                         invz = thin_invz + thin_prep_bytes(st.r0) / sizeof(float);
                     }
                     if (st.trsm)
-                        e = launch_thin_trsm(tc, (float)st.alpha, thin_scratch, invz, h->d_err,
-                                             h->wait_ns, s, h->opt_test_withhold != 0);
+                        e = launch_thin_trsm(tc, (float)st.alpha, thin_scratch, invz, same_a,
+                                             h->d_err, h->wait_ns, s, h->opt_test_withhold != 0);
                     else
                         e = launch_thin_trmm(tc, (float)st.alpha, thin_scratch, h->num_sms, s);
                     if (e == cudaSuccess && st.b > 0 && st.planes && st.r0 + st.b < c.k)
@@ -549,10 +550,13 @@ int pair_trmm(trx_handle_t h, char side, char uplo, char transa, char diag, int6
 // element, is inside 8 k u of FP64 from here on.
 constexpr int64_t kPairMinK = 64;
 
+// same_a: a call of one operation's that repeats its solve before it, launched
+// directly: same handle, stream, A, sizes and options, and nothing in between on the
+// workspace or the thin solve's scratch, so what they hold of A is made already.
 template <typename T>
 int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char diag, int64_t m,
             int64_t n, T alpha, const T* A, int64_t lda, T* B, int64_t ldb, void* stream,
-            const trx_factor_s* f = nullptr, int terms_override = 0) {
+            const trx_factor_s* f = nullptr, int terms_override = 0, bool same_a = false) {
     const int info = check_args(side, uplo, transa, diag, m, n, A, lda, B, ldb);
     if (info) return info;
     if (!valid(h)) return TRX_ERR_HANDLE;
@@ -580,6 +584,7 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
     ex.c = canonicalize<T>(side, uplo, transa, diag, m, n, A, lda, B, ldb);
     ex.s = s;
     ex.profile = h->opt_profile != 0;
+    ex.same_a = same_a;
     const int64_t k = ex.c.k;
     int b = leaf_for(h->opt_leaf, k, trsm, (int)sizeof(T), ex.c.nrhs);
 
@@ -775,7 +780,7 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
     body.tc_leaf = plan.tc_leaf;
     body.thin_leaf = plan.thin_leaf;
     if (ex.turn_t) pre.steps.push_back(Step{kTurnIn});
-    if (plan.tc && !factor_planes) {
+    if (plan.tc && !factor_planes && !same_a) {
         Step cm{kConvM};
         cm.b = dense;
         pre.steps.push_back(cm);
@@ -1888,8 +1893,11 @@ int refine_fixed(trx_handle_t h, bool fp64_data, char side, char uplo, char tran
                                                   s);
             return le == cudaSuccess ? TRX_SUCCESS : fail_cuda(le, "refine solve");
         }
+        // (the corrections' solves find the first one's operand planes of A and block
+        // inverses: 33 us a solve at order 4096; a first one with alpha 0 made none)
         return execute<float>(h, true, 'L', uplo, transI, diag, k, nr,
-                              first ? (float)alpha : 1.0f, As, ldas, D32, k, stream);
+                              first ? (float)alpha : 1.0f, As, ldas, D32, k, stream, nullptr, 0,
+                              !first && (float)alpha != 0.0f);
     };
     // the FP32 solve, Xi := its result
     if ((rc = solve32(true)) != TRX_SUCCESS) return rc;

@@ -337,13 +337,15 @@ constexpr int kThinBlock = 64, kThinPanel = 16;
 size_t thin_scratch_bytes(int64_t k, int64_t nrhs);
 // The block rows' inverses and Z tiles of c's triangle (thin_prep_bytes(c.k)): a
 // launch with several panels makes its own in its scratch unless it is given them
-// (invz: its first block row's). The leaves of a recursion take theirs from one pass.
+// (invz: its first block row's) or they are `made`: in the same scratch by a launch
+// for the same A before it. The leaves of a recursion take theirs from one pass.
 size_t thin_prep_bytes(int64_t k);
 cudaError_t launch_thin_prep(const Canon<float>& c, float* invz, cudaStream_t s);
 // withhold: test hook, block row 0 is never published, so the bounded waits
 // of the blocks after it run out (TRX_ERR_TIMEOUT).
 cudaError_t launch_thin_trsm(const Canon<float>& c, float alpha, int* scratch, const float* invz,
-                             int* err, long long wait_ns, cudaStream_t s, bool withhold = false);
+                             bool made, int* err, long long wait_ns, cudaStream_t s,
+                             bool withhold = false);
 // The thin TRMM (thin.cu): C := alpha M C in one launch after a packing
 // pass of C's original rows (no waits); scratch: thin_trmm_scratch_bytes.
 size_t thin_trmm_scratch_bytes(int64_t k, int64_t nrhs);

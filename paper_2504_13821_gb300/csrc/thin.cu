@@ -873,7 +873,8 @@ cudaError_t launch_thin_prep(const Canon<float>& c, float* invz, cudaStream_t s)
 }
 
 cudaError_t launch_thin_trsm(const Canon<float>& c, float alpha, int* scratch, const float* invz,
-                             int* err, long long wait_ns, cudaStream_t s, bool withhold) {
+                             bool made, int* err, long long wait_ns, cudaStream_t s,
+                             bool withhold) {
     if (c.k <= 0 || c.nrhs <= 0) return cudaSuccess;
     const int64_t nbr = (c.k + kThinBlock - 1) / kThinBlock;
     const int64_t npan = (c.nrhs + kThinPanel - 1) / kThinPanel;
@@ -892,7 +893,7 @@ cudaError_t launch_thin_trsm(const Canon<float>& c, float alpha, int* scratch, c
     if (npan > 1 && invz == nullptr) {
         float* own = reinterpret_cast<float*>(reinterpret_cast<char*>(scratch) +
                                               thin_words_bytes(nbr, npan));
-        if ((e = launch_thin_prep(c, own, s)) != cudaSuccess) return e;
+        if (!made && (e = launch_thin_prep(c, own, s)) != cudaSuccess) return e;
         invz = own;
     }
     p.invz = invz;
