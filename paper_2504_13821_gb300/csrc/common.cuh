@@ -146,6 +146,13 @@ cudaError_t launch_leaf(bool trsm, const Canon<T>& p, int64_t r0, int b,
 // kMaxBlockLeaf rows (the block-leaf kernel).
 constexpr int kMaxLeaf = 128;
 constexpr int kMaxBlockLeaf = 256;
+// FP64 TRSM leaves (us, order x right-hand sides, leaves of 64 / 128 / 256 rows): 256 x 16
+// 101 / 77 / 71, 256 x 600 111 / 91 / 93, 1000 x 16 412 / 305 / 293, 1000 x 200 418 /
+// 303 / 288, 1000 x 400 447 / 369 / 377, 1000 x 1000 489 / 470 / 579, 4096 x 200 1937 /
+// 1422 / 1349, 4096 x 1000 2415 / 2312 / 2798.
+constexpr int64_t kF64TallMaxNrhs = 1024;      // 128 rows up to here,
+constexpr int64_t kF64TallestMaxNrhs = 304;    // 256 up to here
+
 
 // CUDA-core GEMM update on the canonical matrices:
 //   C[rc+i, j] = beta*C[rc+i, j] + gamma * sum_l M(rc+i, rk+l) * Y[rk+l, j]

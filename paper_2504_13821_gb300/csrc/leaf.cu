@@ -47,6 +47,8 @@ extern template cudaError_t leaf_b256_launch<double>(const LeafArgs<double>&, cu
 cudaError_t leaf_wide_configure();
 cudaError_t leaf_wide_launch(const LeafArgs<float>& a, int num_sms, cudaStream_t s);
 cudaError_t leaf64_configure();
+cudaError_t leaf256_configure();
+cudaError_t leaf256_launch(const LeafArgs<double>& a, int num_sms, cudaStream_t s);
 cudaError_t leaf64_launch(const LeafArgs<double>& a, int num_sms, cudaStream_t s);
 cudaError_t convert_configure();
 cudaError_t refine_configure();
@@ -69,6 +71,7 @@ cudaError_t leaf_configure_all() {
     if ((e = leaf_b256_configure<double>()) != cudaSuccess) return e;
     if ((e = leaf_wide_configure()) != cudaSuccess) return e;
     if ((e = leaf64_configure()) != cudaSuccess) return e;
+    if ((e = leaf256_configure()) != cudaSuccess) return e;
     if ((e = convert_configure()) != cudaSuccess) return e;
     if ((e = refine_configure()) != cudaSuccess) return e;
     if ((e = dag_configure()) != cudaSuccess) return e;
@@ -100,6 +103,11 @@ cudaError_t launch_leaf(bool trsm, const Canon<T>& p, int64_t r0, int b,
         const char* e = std::getenv("TRX_LEAF_BLOCKED");
         return !(e && e[0] == '0');
     }();
+    // FP64, one leaf of 65..256 rows, few right-hand sides.
+    if constexpr (std::is_same<T, double>::value) {
+        if (blocked_on && trsm && nleaves == 1 && b > 64 && p.nrhs <= kF64TallMaxNrhs)
+            return leaf256_launch(a, num_sms > 0 ? num_sms : 1, s);
+    }
     if (trsm && b > kMaxLeaf) return leaf_b256_launch<T>(a, s);   // block leaf, 129..256 rows
     // FP32, one leaf of 65..128 rows, many right-hand sides: the wide kernel
     // (register-resident tiles, four column groups per CTA).

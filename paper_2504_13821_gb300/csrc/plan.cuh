@@ -339,15 +339,15 @@ inline int trmm_dense_mode(int64_t opt, int64_t opt_leaf, bool tc, int64_t k) {
     return (opt_leaf == 0 && k >= kTrmmDenseMinOrder) ? kTrmmDenseRows : 0;
 }
 
-// Recursion cutoff: TRX_OPT_LEAF when set, else 128 for FP32 TRSM and 64
-// otherwise. With 256 a TRSM's leaves run as block leaves (one launch per 256
+// Recursion cutoff: TRX_OPT_LEAF when set, else 128 for FP32 TRSM, 256 or 128 for
+// FP64 TRSM with few right-hand sides (kF64TallMaxNrhs) and 64 otherwise. With 256 a TRSM's leaves run as block leaves (one launch per 256
 // rows); TRMM leaves stop at 128 rows.
 inline int leaf_for(int64_t opt_leaf, int64_t k, bool trsm, int elem, int64_t nrhs) {
     int b = kDefaultLeaf;
     if (opt_leaf > 0) b = (int)opt_leaf;
     else if (trsm && elem == 4) b = kF32TrsmLeaf;
+    else if (trsm && nrhs <= kF64TallMaxNrhs) b = nrhs <= kF64TallestMaxNrhs ? 256 : 128;
     if (!trsm && b > kMaxLeaf) b = kMaxLeaf;
-    (void)nrhs;
     return (int)std::min<int64_t>(b, std::max<int64_t>(k, 1));
 }
 
