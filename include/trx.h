@@ -93,7 +93,9 @@ enum {
     TRX_OPT_LEAF = 1,      /* leaf cutoff b (Section 3.1 "chosen threshold"):
                               16, 32, 64, 128 or 256 (256: TRSM block
                               leaves; TRMM stops at 128); 0 = automatic
-                              (default: 128 for FP32 TRSM, else 64)        */
+                              (default: 128 for FP32 TRSM; FP64 TRSM: 256
+                              with at most 304 right-hand sides, 128 with
+                              at most 1024; else 64)                      */
     TRX_OPT_GEMM = 2,      /* FP32 GEMM-update engine: 0 automatic, 1 CUDA
                               cores (FP32 FMA), 2 tensor cores (tcgen05,
                               split BF16 products of TRX_OPT_SPLIT terms,

@@ -103,9 +103,10 @@ cudaError_t launch_leaf(bool trsm, const Canon<T>& p, int64_t r0, int b,
         const char* e = std::getenv("TRX_LEAF_BLOCKED");
         return !(e && e[0] == '0');
     }();
-    // FP64, one leaf of 65..256 rows, few right-hand sides.
+    // FP64, one leaf of 33..256 rows, few right-hand sides (64 rows, a whole call, lane-split
+    // sweep / this kernel, us: 16 right-hand sides 28.1 / 26.2, 100 29.5 / 26.3, 600 27.6 / 26.1).
     if constexpr (std::is_same<T, double>::value) {
-        if (blocked_on && trsm && nleaves == 1 && b > 64 && p.nrhs <= kF64TallMaxNrhs)
+        if (blocked_on && trsm && nleaves == 1 && b > 32 && p.nrhs <= kF64TallMaxNrhs)
             return leaf256_launch(a, num_sms > 0 ? num_sms : 1, s);
     }
     if (trsm && b > kMaxLeaf) return leaf_b256_launch<T>(a, s);   // block leaf, 129..256 rows

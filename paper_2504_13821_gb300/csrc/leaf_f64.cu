@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(128) leaf64_kernel(LeafArgs<double> a) {
     }
 }
 
-// FP64 TRSM leaf of 65..256 rows with few right-hand sides, C columns a CTA, in 16-row
+// FP64 TRSM leaf of 33..256 rows with few right-hand sides, C columns a CTA, in 16-row
 // blocks: warp 0 substitutes block q (32 / C lanes a column) while warps 1-3 take block
 // q - 1's columns off the rows below it and four more warps bring M's columns of block
 // q + 1 in; then the four take block q's columns off block q + 1.

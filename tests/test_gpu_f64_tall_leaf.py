@@ -1,4 +1,4 @@
-"""FP64 TRSM leaves of 65 to 256 rows (few right-hand sides): orders at the edges of the
+"""FP64 TRSM leaves of 33 to 256 rows (few right-hand sides): orders at the edges of the
 16-row blocks and of the leaf, right-hand sides at the edges of a CTA's 2, 4 and 8
 columns and of the rule, both sides and directions; FP64 oracle. A row's Inf reaches no
 row before it and no other column."""
@@ -12,7 +12,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("k", [65, 79, 80, 81, 127, 128, 129, 200, 255, 256, 257, 300])
+@pytest.mark.parametrize("k", [33, 63, 65, 79, 80, 81, 127, 128, 129, 200, 255, 256, 257, 300])
 @pytest.mark.parametrize("variant", ["LLNN", "LUNU", "LLTN", "RLNN", "RUTU"])
 def test_edges(k, variant):
     side, uplo, trans, diag = variant
