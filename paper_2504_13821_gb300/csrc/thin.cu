@@ -40,7 +40,7 @@
 // three products (its last tile, the inverse, Z) of 0.5-0.67 us each in two steps.
 // us, this kernel against one CTA per ticket that published through L2 only, staged M
 // between its products and had a thread on 4 rows x 1 column: 8191 x 16 transposed
-// 323 -> 259, 8192 x 16 323 -> 225, 8192 x 64 449 -> 316, a 2048-row leaf with 256
+// 323 -> 230, 8192 x 16 323 -> 208, 8192 x 64 449 -> 316, a 2048-row leaf with 256
 // right-hand sides 121 -> 87. On the way: the products alone 309, clusters with M
 // still staged between them 283.
 //
@@ -67,6 +67,7 @@ constexpr int LD = BR + 4;           // shared row stride (floats): 16-byte alig
 constexpr int LDT = BR + 1;          // inverse work tile: conflict-free column reads
 constexpr int CL = 8;                // block rows of a task, CTAs of a cluster
 constexpr int ND = 4;                // block rows that a CTA pushes its block to
+constexpr size_t kAlone = 120 * 1024;   // shared memory that leaves no room for a second CTA
 constexpr int NTP = 128;             // threads of the solve that bring in M
 constexpr int kTimeout = 4;          // TRX_ERR_TIMEOUT
 
@@ -411,21 +412,26 @@ __device__ void invert_diag(const Params& p, Smem& sm, int64_t i0) {
     float y0[8], y1[8];          // rows l and l + 32, columns 8 w + u
 #pragma unroll
     for (int u = 0; u < 8; ++u) y0[u] = y1[u] = 0.0f;
-    for (int r = 8 * w; r < BR; ++r) {   // (rows above the columns: zeros)
+    // (rows above the warp's columns: zeros)
+    for (int r = 8 * w; r < 32; ++r) {           // lane r owns row r
         const float dr = sm.dinv[r];
-        const int owner = r & 31;
-        const bool hi = r >= 32;
         const float m0 = T[l * LDT + r], m1 = T[(l + 32) * LDT + r];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            const float s = hi ? y1[u] : y0[u];
-            const float v = ((r == 8 * w + u) ? 1.0f : 0.0f) - s;
-            const float yr = __shfl_sync(0xffffffffu, v * dr, owner);
-            if (l == owner) {
-                if (hi) y1[u] = yr; else y0[u] = yr;
-            }
-            if (l > r) y0[u] = fmaf(m0, yr, y0[u]);
-            if (l + 32 > r) y1[u] = fmaf(m1, yr, y1[u]);
+            const float v = (((r == 8 * w + u) ? 1.0f : 0.0f) - y0[u]) * dr;
+            const float yr = __shfl_sync(0xffffffffu, v, r);
+            y0[u] = l > r ? fmaf(m0, yr, y0[u]) : l == r ? yr : y0[u];
+            y1[u] = fmaf(m1, yr, y1[u]);
+        }
+    }
+    for (int r = w < 4 ? 32 : 8 * w; r < BR; ++r) {   // lane r - 32 owns row r
+        const float dr = sm.dinv[r];
+        const float m1 = T[(l + 32) * LDT + r];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const float v = (((r == 8 * w + u) ? 1.0f : 0.0f) - y1[u]) * dr;
+            const float yr = __shfl_sync(0xffffffffu, v, r - 32);
+            y1[u] = l + 32 > r ? fmaf(m1, yr, y1[u]) : l + 32 == r ? yr : y1[u];
         }
     }
     // s_r accumulated with +: the recurrence above keeps s = sum m y and
@@ -827,6 +833,13 @@ size_t thin_scratch_bytes(int64_t k, int64_t nrhs) {
     return thin_words_bytes(nbr, npan) + (npan > 1 ? thin_prep_bytes(k) : 0);
 }
 
+// Two clusters fit the same SMs, where each would stage M at half the rate: from
+// kSpreadRows block rows on, launches of at most kSpread CTAs (two clusters of eight SMs
+// in each part of the chip) ask for more shared memory than two have room for. us,
+// without / with: 8191 x 16 transposed 281 / 230, 8192 x 16 228 / 208, 4096 x 32 131 /
+// 117, 2048 x 64 73 / 69, 4096 x 16 115 / 114; but 1024 x 128 48 / 54, 512 x 256 36 / 46
+// (the SMs change their split of shared memory between the launches of a call).
+constexpr int64_t kSpread = 128, kSpreadRows = 32;
 static int g_thin_trmm_ctas_per_sm = 0;
 
 cudaError_t thin_configure() {
@@ -841,7 +854,7 @@ cudaError_t thin_configure() {
     g_thin_trmm_ctas_per_sm = nm > 0 ? nm : 1;
     cudaError_t e = cudaFuncSetAttribute(thin::thin_trsm_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(thin::Smem));
+                                         (int)thin::kAlone);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(thin::thin_prep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sizeof(thin::Smem));
@@ -898,8 +911,10 @@ cudaError_t launch_thin_trsm(const Canon<float>& c, float alpha, int* scratch, c
     }
     p.invz = invz;
     const int64_t clusters = (nbr + thin::CL - 1) / thin::CL * npan;
-    thin::thin_trsm_kernel<<<(unsigned)(clusters * thin::CL), thin::NT + thin::NTP,
-                             sizeof(thin::Smem), s>>>(p);
+    // a long chain on few enough CTAs for an SM each: shared memory for one
+    const size_t smem = nbr >= kSpreadRows && clusters * thin::CL <= kSpread ? thin::kAlone
+                                                                             : sizeof(thin::Smem);
+    thin::thin_trsm_kernel<<<(unsigned)(clusters * thin::CL), thin::NT + thin::NTP, smem, s>>>(p);
     return cudaGetLastError();
 }
 
