@@ -239,7 +239,7 @@ def auto_path_desc(k, n):
         thin_leaf = 2048 if n <= 256 else 1024 if n <= 1024 else 512
     if thin_leaf and k > thin_leaf:
         trsm = f"TRSM leaves of {thin_leaf} rows as thin solves (64-row blocks, 16-column panels)"
-    elif (k > 256 and n <= 64) or (k >= 256 and n <= min(1024, 4 * k) and k * n <= 1 << 20):
+    elif (k > 256 and n <= 64) or (k >= 256 and n <= min(1024, 2 * k) and k * n <= 1 << 20):
         trsm = "TRSM as one thin solve (64-row blocks, 16-column panels, one launch)"
     else:
         trsm = f"TRSM 128 ({'wide leaf' if n >= 1024 else 'lane-split leaf'})"

@@ -237,7 +237,7 @@ enum {
                               -1 = the recursion; 0 = automatic (default):
                               TRSM of order above 256 with at most 64
                               right-hand sides, of order 256 on with at most
-                              1024, four times the order, while order x
+                              1024, twice the order, while order x
                               right-hand sides <= 2^20 (where a leaf, GEMM,
                               split, panel, DAG or profile option is set:
                               above 256 with at most 256 while it is <=

@@ -391,13 +391,14 @@ constexpr int64_t kThinMaxNrhs = 64, kThinWideNrhs = 256;
 constexpr int64_t kThinMaxWork = (int64_t)1 << 21;
 constexpr int64_t kThinMinK = 256;
 // Where every option is automatic and the operands keep all three planes: from order
-// 256 on up to kThinAutoWhole right-hand sides, four times the order at most, the
+// 256 on up to kThinAutoWhole right-hand sides, twice the order at most, the
 // whole call while order x right-hand sides is within kThinAutoWork (the chain's
 // leaves, 10-32 us each whatever their right-hand sides, are its time there); from
 // there on, and from order 1024 on, the thin leaves up to kThinAutoNrhs. Measured
 // (us, order x right-hand sides, side L and R; chain / whole call / leaves of 512,
 // 1024 and 2048 rows):
 //   256 x 256     L 50 / 48                    R 66 / 47
+//   256 x 768     L 50 / 53                    R 68 / 52
 //   256 x 1000    L 53 / 54                    R 68 / 55
 //   512 x 512     L 83 / 57                    R 110 / 57
 //   1000 x 400    L 148 / 84 / 93              R 201 / 88 / 102
@@ -424,7 +425,7 @@ inline bool use_thin_mode(int64_t opt, bool trsm, int elem, int64_t k, int64_t n
     if (opt < 0 || elem != 4 || k <= 0 || nrhs <= 0) return false;
     if (opt > 0) return true;
     if (!trsm) return k > kThinMinK && nrhs <= kThinTrmmMaxNrhs;
-    if (automatic && k >= kThinAutoK && nrhs <= std::min(kThinAutoWhole, 4 * k) &&
+    if (automatic && k >= kThinAutoK && nrhs <= std::min(kThinAutoWhole, 2 * k) &&
         k * nrhs <= kThinAutoWork)
         return true;
     return k > kThinMinK &&
