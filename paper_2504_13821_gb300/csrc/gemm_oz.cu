@@ -43,6 +43,8 @@
 // 5.6e-17 (DFMA 7.7e-16).
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
@@ -153,7 +155,7 @@ __device__ void split_strip(const Operand& o, int64_t K, int nk, int64_t r0) {
             const int64_t end = o.tri ? min(k1, r0 + q) : k1;
             unsigned mx = 0;
             int cnt = 0;
-#pragma unroll 8
+#pragma unroll 16
             for (int64_t l = k0 + lane; l < end; l += 32) {
                 const unsigned long long b = __double_as_longlong((double)src[l * o.ls]) &
                                              0x7fffffffffffffffull;
@@ -171,7 +173,7 @@ __device__ void split_strip(const Operand& o, int64_t K, int nk, int64_t r0) {
     __syncthreads();
     if (r >= o.rows) return;
     const int emax = (int)(smax[rl] >> 20);
-    if (warp == 0 && kl == 0) {
+    if (warp == 0 && kl == 0 && blockIdx.z == 0) {
         const int e = emax - 1021;           // |x| 2^-e < 1/2
         const bool ok = scnt[rl] == 0 || (e >= -kMaxExp && e <= kMaxExp);
         o.info[seg * o.rows + r] = make_int2(ok ? (scnt[rl] ? e : 0) : kBadExp, scnt[rl]);
@@ -185,7 +187,8 @@ __device__ void split_strip(const Operand& o, int64_t K, int nk, int64_t r0) {
     // 16-byte loads of FP64 data along K where every row starts on 16 bytes
     const bool pairs = sizeof(TX) == 8 && o.ls == 1 && (o.rs & 1) == 0 &&
                        (reinterpret_cast<uintptr_t>(X) & 15) == 0;
-    for (int kc = 2 * seg * SEG_STEPS + warp * KL + kl; kc < kc1; kc += NW * KL) {
+    for (int kc = 2 * seg * SEG_STEPS + ((int)blockIdx.z * NW + warp) * KL + kl; kc < kc1;
+         kc += (int)gridDim.z * NW * KL) {
         const int64_t l0 = (int64_t)kc * 8;
         unsigned lo[8], hi[8];               // lower seven digits, each + 128
         int top[8];
@@ -856,8 +859,14 @@ static cudaError_t launch_split(const Operand& o0, const Operand* o1, int64_t K,
     a.nk = (int)((K + KS - 1) / KS);
     a.strips0 = (int)((o0.rows + STRIP - 1) / STRIP);
     const int64_t strips = a.strips0 + (o1 ? (o1->rows + STRIP - 1) / STRIP : 0);
-    return launch_kernel(oz_split_kernel<T0>, dim3((unsigned)strips, (unsigned)nseg(K)),
-                         dim3(SPLIT_NT), 0, s, a);
+    // few strips: several CTAs each, which all look for the exponent and share the digits
+    // (256 columns with K 4096 55 -> 18 us; TRSM 1000 x 200 290 -> 285; more than 256
+    // CTAs read more than they save: refined 4096 x 256 1351 us, with 1024 1367, 2048 1422)
+    const int64_t parts = std::max<int64_t>(
+        1, std::min({(int64_t)8, std::min<int64_t>(K, SEG) / 128, 256 / (strips * nseg(K))}));
+    return launch_kernel(oz_split_kernel<T0>,
+                         dim3((unsigned)strips, (unsigned)nseg(K), (unsigned)parts), dim3(SPLIT_NT),
+                         0, s, a);
 }
 
 // The product of two split operands (the rest of `q` set by the caller), and
