@@ -15,10 +15,13 @@ RIGHT = [v for v in inputs.VARIANTS if v[0] == "R"]
 
 
 @pytest.mark.parametrize("op", ["trsm", "trmm"])
-@pytest.mark.parametrize("m,n", [(256, 256), (257, 511), (1025, 320), (2111, 257)])
+@pytest.mark.parametrize("m,n", [(512, 512), (515, 511), (1025, 320), (2111, 257)])
 def test_turned_against_oracle(op, m, n):
     import paper_2504_13821_gb300 as trx
     turned, plain = trx.Handle(0), trx.Handle(0)
+    for h in (turned, plain):                    # the recursion at every size
+        h.set_option(trx.OPT_THIN, -1)
+        h.set_option(trx.OPT_THIN_LEAF, -1)
     need = turned.workspace_size("S" if op == "trsm" else "M", "R", m, n, 4)
     planes = turned.workspace_size("S" if op == "trsm" else "M", "L", n, m, 4)
     assert need > planes
@@ -42,7 +45,9 @@ def test_repeated_calls_on_other_arrays(op):
     another leading dimension, write that one."""
     import paper_2504_13821_gb300 as trx
     h = trx.Handle(0)
+    h.set_option(trx.OPT_THIN, -1)
+    h.set_option(trx.OPT_THIN_LEAF, -1)
     for seed, pad in ((1, 0), (2, 0), (3, 5), (1, 0)):
         for v in RIGHT[:4]:
-            run_case(op, *v, 300, 500, 0.5, np.float32, seed=seed, handle=h, ldb_pad=pad)
+            run_case(op, *v, 600, 500, 0.5, np.float32, seed=seed, handle=h, ldb_pad=pad)
     h.close()
