@@ -460,11 +460,10 @@ inline int thin_leaf_rows(int64_t opt, bool tc, bool trsm, int elem, int64_t k, 
 // past the planes, B is turned into the workspace, solved there and turned back (in
 // the canonical order, so a reversed problem's rows run forwards too). The two
 // passes cost 16 bytes an element. Measured (us, nrhs x order, in place / turned):
-// TRSM 600 x 600 148 / 123, 2000 x 2000 628 / 441, 4096 x 4096 1343 / 945, 8192 x 8192
-// 5375 / 3813; TRMM 500 x 300 30 / 36, 300 x 500 33 / 32, 400 x 400 33 / 31, 600 x 500
-// 39 / 34, 1000 x 600 41 / 36, 1000 x 1000 56 / 42, 3000 x 5000 609 / 432. Below 2^18
-// elements nothing is gained.
-constexpr int64_t kTurnMinElements = (int64_t)1 << 18;
+// TRSM 256 x 256 53 / 51, 600 x 300 58 / 52, 600 x 600 148 / 123, 2000 x 2000 628 /
+// 441, 4096 x 4096 1343 / 945, 8192 x 8192 5375 / 3813; TRMM 500 x 300 31 / 31,
+// 1000 x 1000 56 / 42, 3000 x 5000 609 / 432. Below 2^16 elements nothing is gained.
+constexpr int64_t kTurnMinElements = (int64_t)1 << 16;
 inline bool turn_applies(int64_t k, int64_t nrhs) {
     return k * nrhs >= kTurnMinElements && k <= 64 * 65535ll && nrhs <= 64 * 65535ll;
 }
