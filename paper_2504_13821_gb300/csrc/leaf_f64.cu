@@ -1,4 +1,4 @@
-// FP64 TRSM leaf (Section 3.3 base kernel) of 33..64 rows with many right-hand
+// FP64 TRSM leaves (Section 3.3 base kernel). First, 33..64 rows with many right-hand
 // sides: blocked forward substitution in 16-row blocks, C columns per CTA of 128
 // threads.
 //
@@ -14,8 +14,8 @@
 //
 // Measured, one 64-row leaf (us by right-hand sides, that kernel / this one, ncu):
 // 1024 47 / 17, 1500 48 / 21, 4096 54 / 29; four lanes per column took 20 (1024)
-// and 29 (4096), 32 columns per CTA 34 (4096). Below 1024 the lane-split leaf has as
-// short a chain and no barriers (16 us at 200 against 17).
+// and 29 (4096), 32 columns per CTA 34 (4096). Up to 1024 right-hand sides
+// leaf256_kernel below serves.
 #include "common.cuh"
 #include "leaf_impl.cuh"
 
