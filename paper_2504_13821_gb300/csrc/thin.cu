@@ -644,7 +644,8 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT + NTP, 2)
         }
         break;
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");   // nothing in flight at exit
+    // nothing in flight at exit (the producers' copies belong to no group)
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncwarp();
     // no CTA leaves while another may read its task or push to it, nor (after a
     // timeout) before what was pushed has landed
