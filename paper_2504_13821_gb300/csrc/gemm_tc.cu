@@ -75,7 +75,7 @@ constexpr int kTimeout = 4;                          // TRX_ERR_TIMEOUT
 // shared memory), tensor memory (two accumulators of BN FP32 columns) and
 // the kind::f16 instruction descriptor (FP32 accumulator, BF16 A and B, both
 // K-major, M = 128, N = BN).
-template <int BN, int S>
+template <int BN, int S, bool ONE_LANE = false>
 struct Cfg {
     static constexpr int B_TILE = BN * BK * 2;
     static constexpr int STAGE_BYTES = S * A_TILE + S * B_TILE;
@@ -86,8 +86,11 @@ struct Cfg {
     // lane needs to issue it) and the two accumulators of a chunk double buffered,
     // for which tensor memory has room. At 256 columns an MMA takes 128 clocks
     // either way and the kernel runs at the power limit; the denser issue measured
-    // 1-2 % slower there.
-    static constexpr bool WARP_ISSUE = S == 3 && BN < 256;
+    // 1-2 % slower there. Column-panel branches, where launches of several streams
+    // follow one another on an SM, keep one lane and one set (ONE_LANE): their test
+    // ended twice in a memory fault with the form for the whole warp, which single
+    // streams have never shown and reading has not explained.
+    static constexpr bool WARP_ISSUE = S == 3 && BN < 256 && !ONE_LANE;
     static constexpr int SETS = WARP_ISSUE ? 2 : 1;
     static constexpr int TMEM_COLS = 2 * BN * SETS;
     static constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + 256;
@@ -238,10 +241,10 @@ __device__ __forceinline__ Tile map_tile(const PP& p, int t) {
     return r;
 }
 
-template <int BN, int S, int MG>
+template <int BN, int S, int MG, bool ONE_LANE = false>
 __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
     gemm_tc_kernel(const __grid_constant__ ParamsT<MG> p) {
-    using C = Cfg<BN, S>;
+    using C = Cfg<BN, S, ONE_LANE>;
     constexpr bool P = Precise<S>::value;
     constexpr int STAGES = C::STAGES;
     constexpr int STAGE_BYTES = C::STAGE_BYTES;
@@ -707,6 +710,13 @@ cudaError_t tc_configure() {
     cudaError_t e;
     if ((e = tc_configure_s<1>()) != cudaSuccess) return e;
     if ((e = tc_configure_s<2>()) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(tc::gemm_tc_kernel<128, 3, tc::MAXG_SMALL, true>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  tc::Cfg<128, 3>::SMEM_BYTES)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(tc::gemm_tc_kernel<64, 3, tc::MAXG_SMALL, true>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  tc::Cfg<64, 3>::SMEM_BYTES)) != cudaSuccess)
+        return e;
     return tc_configure_s<3>();
 }
 
@@ -729,7 +739,7 @@ cudaError_t tc_make_maps(const Planes& pl, int64_t k, int64_t nrhs, void* out) {
 cudaError_t launch_gemm_tc(const Canon<float>& p, const void* maps, int slices,
                            const TcGemm* gemms, int ngemms, float beta, float gamma,
                            int* err_word, long long wait_ns, int num_sms, cudaStream_t s,
-                           bool diag_beta, const TcYOut* yout) {
+                           bool diag_beta, const TcYOut* yout, bool branches) {
     if (slices < 1 || slices > 3) return cudaErrorInvalidValue;
     using namespace tc;
     for (int g0 = 0; g0 < ngemms; g0 += MAXG) {
@@ -803,6 +813,11 @@ cudaError_t launch_gemm_tc(const Canon<float>& p, const void* maps, int slices,
         else if (slices == 2)
             e = bn == 256 ? TRX_TC_LAUNCH(256, 2) : bn == 128 ? TRX_TC_LAUNCH(128, 2)
                                                               : TRX_TC_LAUNCH(64, 2);
+        else if (branches && small && bn < 256)
+            e = bn == 128 ? launch_kernel(gemm_tc_kernel<128, 3, MAXG_SMALL, true>, dim3(grid),
+                                          dim3(NTHREADS_P), Cfg<128, 3>::SMEM_BYTES, s, prm_small)
+                          : launch_kernel(gemm_tc_kernel<64, 3, MAXG_SMALL, true>, dim3(grid),
+                                          dim3(NTHREADS_P), Cfg<64, 3>::SMEM_BYTES, s, prm_small);
         else
             e = bn == 256 ? TRX_TC_LAUNCH(256, 3) : bn == 128 ? TRX_TC_LAUNCH(128, 3)
                                                               : TRX_TC_LAUNCH(64, 3);
