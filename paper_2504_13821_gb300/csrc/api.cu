@@ -295,7 +295,6 @@ struct Exec {
     cudaStream_t s;
     bool profile;
     bool same_a = false;
-    bool branches = false;         // one of several column panels on streams of their own
 
     // NVTX range name of a step (TRX_OPT_NVTX): kind and its row ranges
     static void nvtx_push(const Step& st) {
@@ -357,7 +356,7 @@ struct Exec {
                                            st.inv ? maps_w : maps, pl.slices, st.gemms.data(),
                                            (int)st.gemms.size(), (float)st.beta, (float)st.gamma,
                                            h->d_err, h->wait_ns, h->num_sms, s, st.dense,
-                                           st.y1 > st.y0 ? &yo : nullptr, branches);
+                                           st.y1 > st.y0 ? &yo : nullptr);
                         cls = st.inv ? TRX_KERNEL_LEAF_TRSM : TRX_KERNEL_GEMM_TC;
                     } else {
                         cls = TRX_KERNEL_GEMM_SIMT;
@@ -725,7 +724,6 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
         const int64_t step = round_up((ex.c.nrhs + P - 1) / P, 256);
         P = (int)std::max<int64_t>(1, (ex.c.nrhs + step - 1) / step);
     }
-    ex.branches = P > 1;
     std::vector<Exec<T>> parts((size_t)P, ex);
     std::vector<std::vector<unsigned char>> maps((size_t)P);
     {

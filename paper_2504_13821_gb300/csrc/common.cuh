@@ -249,12 +249,11 @@ struct TcYOut {
     __nv_bfloat16* lo2 = nullptr;
     int64_t ld = 0, row0 = 0, row1 = 0;
 };
-// branches: one of several column-panel branches on streams of their own
 cudaError_t launch_gemm_tc(const Canon<float>& p, const void* maps, int slices,
                            const TcGemm* gemms, int ngemms, float beta,
                            float gamma, int* err_word, long long wait_limit,
                            int num_sms, cudaStream_t s, bool diag_beta = false,
-                           const TcYOut* yout = nullptr, bool branches = false);
+                           const TcYOut* yout = nullptr);
 // Refined TRSM helpers (refine.cu): casts, residual, correction, norms.
 cudaError_t refine_cast_f32_f64(const float* src, int64_t lds, double* dst, int64_t ldd, int64_t m,
                                 int64_t n, double scale, cudaStream_t s);

@@ -411,9 +411,9 @@ __device__ __forceinline__ int round_tile(int r) {
 // tensor cores work on the other.
 //
 // Bound by the tensor pipe: 36 x 64 columns a step (1184 clocks at BN = 64)
-// against 48 KB of operands through L2. 2048 x 4096 with K 2048: 790 us; with the
-// MMAs issued from a one-lane branch 825, and with 128-term chunks and spilled
-// sums as well 886.
+// against 48 KB of operands through L2. One lane, elect.sync's, waits, issues and
+// commits: FP64 TRSM 4096 x 4096 5205 us, TRMM 2500 x 1500 455; with lane 0 in its place
+// 5353 and 485.
 template <int BN>
 __global__ void __launch_bounds__(NT, 1) oz_gemm_kernel(const __grid_constant__ Params p) {
     using C = Cfg<BN>;
@@ -508,20 +508,14 @@ __global__ void __launch_bounds__(NT, 1) oz_gemm_kernel(const __grid_constant__ 
                 if (--stage < 0) { stage = STAGES - 1; phase ^= 1u; }
                 wait_bounded(smem_u32(&sm->full[stage]), phase, p, abort, false);
             }
-        } else if (warp == 1) {
-            // ---------------- MMA issuer (the whole warp, one lane elected) ----------------
-            const uint32_t lead = elect_lane();
+        } else if (warp == 1 && elect_lane()) {
+            // ---------------- MMA issuer ----------------
             int stage = 0;
             uint32_t phase = 0, hi_phase = 0, lo_phase = 0;
             const uint64_t a_ring = sdesc_plain(ring), b_ring = sdesc_plain(ring + C::A_BYTES);
             constexpr uint32_t ST = C::STAGE_BYTES >> 4, AP = C::A_PLANE >> 4, BP = C::B_PLANE >> 4;
             const auto wait = [&](uint64_t* bar, uint32_t ph, bool honour_abort = true) {
-                int w = mbar_try(smem_u32(bar), ph);
-                if (!__all_sync(0xffffffffu, w)) {
-                    if (lane == 0) w = wait_bounded(smem_u32(bar), ph, p, abort, honour_abort);
-                    w = __shfl_sync(0xffffffffu, w, 0);
-                    if (!w) return false;
-                }
+                if (!wait_bounded(smem_u32(bar), ph, p, abort, honour_abort)) return false;
                 tc_fence_after();
                 return true;
             };
@@ -534,12 +528,11 @@ __global__ void __launch_bounds__(NT, 1) oz_gemm_kernel(const __grid_constant__ 
                     const uint64_t a = a_ring + stage * ST, b = b_ring + stage * ST;
                     const int ns = min(S, nk - i * S);
                     for (int s = 0; s < ns; ++s)
-                        umma_elected(tmem, a + s * AP, b + s * BP, C::idesc(BN),
-                                     (i | s) != 0 ? 1u : 0u, lead);
-                    umma_commit_elected(smem_u32(&sm->empty[stage]), lead);
+                        umma(tmem, a + s * AP, b + s * BP, C::idesc(BN), (i | s) != 0 ? 1u : 0u);
+                    umma_commit(smem_u32(&sm->empty[stage]));
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
-                umma_commit_elected(smem_u32(&sm->hi_full), lead);
+                umma_commit(smem_u32(&sm->hi_full));
                 hi_phase ^= 1u;
                 for (int k0 = 0; k0 < nk; k0 += CHUNK) {
                     const int k1 = min(nk, k0 + CHUNK);
@@ -554,11 +547,11 @@ __global__ void __launch_bounds__(NT, 1) oz_gemm_kernel(const __grid_constant__ 
                             const uint32_t on = k + b > k0 ? 1u : 0u;
 #pragma unroll
                             for (int i = 1; i <= 4; ++i)     // levels i+1 .. 5: B digits 1 .. 5-i
-                                umma_elected(tmem + (uint32_t)(BN * (i - 1)), A + (i - 1) * AP, B,
-                                             C::idesc(BN * (5 - i)), i == 1 ? on : 1u, lead);
+                                umma(tmem + (uint32_t)(BN * (i - 1)), A + (i - 1) * AP, B,
+                                     C::idesc(BN * (5 - i)), i == 1 ? on : 1u);
                             if (++s1 == STAGES) { s1 = 0; ph1 ^= 1u; }
                         }
-                        if (k + nb == k1) umma_commit_elected(smem_u32(&sm->hi_full), lead);
+                        if (k + nb == k1) umma_commit(smem_u32(&sm->hi_full));
                         if (k == k0 && !wait(&sm->lo_empty, lo_phase ^ 1u)) return false;
                         for (int b = 0; b < nb; ++b) {
                             const uint64_t A = a_ring + stage * ST, B = b_ring + stage * ST;
@@ -566,16 +559,16 @@ __global__ void __launch_bounds__(NT, 1) oz_gemm_kernel(const __grid_constant__ 
 #pragma unroll
                             for (int i = 1; i <= 8; ++i) {   // levels max(6, i+1) .. 9
                                 const int j0 = i < 6 ? 6 - i : 1, j1 = 9 - i;
-                                umma_elected(tmem + (uint32_t)(BN * (i + j0 - 2)),
-                                             A + (i - 1) * AP, B + (j0 - 1) * BP,
-                                             C::idesc(BN * (j1 - j0 + 1)), i == 1 ? on : 1u, lead);
+                                umma(tmem + (uint32_t)(BN * (i + j0 - 2)), A + (i - 1) * AP,
+                                     B + (j0 - 1) * BP, C::idesc(BN * (j1 - j0 + 1)),
+                                     i == 1 ? on : 1u);
                             }
-                            umma_commit_elected(smem_u32(&sm->empty[stage]), lead);
+                            umma_commit(smem_u32(&sm->empty[stage]));
                             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                         }
                         k += nb;
                     }
-                    umma_commit_elected(smem_u32(&sm->lo_full), lead);
+                    umma_commit(smem_u32(&sm->lo_full));
                     hi_phase ^= 1u;
                     lo_phase ^= 1u;
                 }
@@ -590,7 +583,7 @@ __global__ void __launch_bounds__(NT, 1) oz_gemm_kernel(const __grid_constant__ 
                     ok = segment(min(SEG_STEPS, nk - s0));
             }
             // All MMAs issued by this CTA complete before TMEM is released.
-            umma_commit_elected(smem_u32(&sm->drain), lead);
+            umma_commit(smem_u32(&sm->drain));
             wait(&sm->drain, 0, false);
         }
     } else {

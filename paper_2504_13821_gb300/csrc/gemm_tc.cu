@@ -75,24 +75,21 @@ constexpr int kTimeout = 4;                          // TRX_ERR_TIMEOUT
 // shared memory), tensor memory (two accumulators of BN FP32 columns) and
 // the kind::f16 instruction descriptor (FP32 accumulator, BF16 A and B, both
 // K-major, M = 128, N = BN).
-template <int BN, int S, bool ONE_LANE = false>
+template <int BN, int S>
 struct Cfg {
     static constexpr int B_TILE = BN * BK * 2;
     static constexpr int STAGE_BYTES = S * A_TILE + S * B_TILE;
     static constexpr int STAGES =
         (1024 + MAX_STAGES * STAGE_BYTES + 256 <= 227 * 1024) ? MAX_STAGES : 3;
-    // The precise form's tiles below 256 columns: MMAs issued by the whole warp
-    // (umma_elected: one of 64 columns takes 48 clocks instead of the 128 that one
-    // lane needs to issue it) and the two accumulators of a chunk double buffered,
-    // for which tensor memory has room. At 256 columns an MMA takes 128 clocks
-    // either way and the kernel runs at the power limit; the denser issue measured
-    // 1-2 % slower there. Column-panel branches, where launches of several streams
-    // follow one another on an SM, keep one lane and one set (ONE_LANE): their test
-    // ended twice in a memory fault with the form for the whole warp, which single
-    // streams have never shown and reading has not explained.
-    static constexpr bool WARP_ISSUE = S == 3 && BN < 256 && !ONE_LANE;
-    static constexpr int SETS = WARP_ISSUE ? 2 : 1;
-    static constexpr int TMEM_COLS = 2 * BN * SETS;
+    // One lane waits, issues and commits, and a chunk has one set of accumulators, at
+    // every width. (A form with the whole warp in the issue loop and two sets below
+    // 256 columns is not used: runs with it ended in a memory fault that reading has
+    // not explained.) Below 256 columns the lane is elect.sync's: TRSM 2000 x 2000 side
+    // R 356 us with lane 0, 340 with the elected one; order 4096 with a factor and 256
+    // right-hand sides 232 and 226. At 256 an MMA takes the pipe 128 clocks whoever
+    // issues it, and a denser issue measured 0-2 % slower at the power limit.
+    static constexpr bool ELECT = BN < 256;
+    static constexpr int TMEM_COLS = 2 * BN;
     static constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + 256;
     static_assert(SMEM_BYTES <= 227 * 1024, "ring does not fit in shared memory");
     static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) |
@@ -170,20 +167,6 @@ __device__ bool wait_bounded(uint32_t bar, uint32_t parity, const Params& p, vol
     }
 }
 
-// The same for a whole warp (lane 0 waits where the phase is not there yet and the
-// others follow its verdict), with the fence that orders tensor-core work after it.
-__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, const Params& p,
-                                          volatile int* abort, bool honour_abort = true) {
-    int w = mbar_try(bar, parity);
-    if (!__all_sync(0xffffffffu, w)) {
-        if ((threadIdx.x & 31) == 0) w = wait_bounded(bar, parity, p, abort, honour_abort);
-        w = __shfl_sync(0xffffffffu, w, 0);
-        if (!w) return false;
-    }
-    tc_fence_after();
-    return true;
-}
-
 struct Tile {
     int g, m, n;
 };
@@ -241,10 +224,10 @@ __device__ __forceinline__ Tile map_tile(const PP& p, int t) {
     return r;
 }
 
-template <int BN, int S, int MG, bool ONE_LANE = false>
+template <int BN, int S, int MG>
 __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
     gemm_tc_kernel(const __grid_constant__ ParamsT<MG> p) {
-    using C = Cfg<BN, S, ONE_LANE>;
+    using C = Cfg<BN, S>;
     constexpr bool P = Precise<S>::value;
     constexpr int STAGES = C::STAGES;
     constexpr int STAGE_BYTES = C::STAGE_BYTES;
@@ -257,9 +240,7 @@ __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
     Smem* sm = reinterpret_cast<Smem*>(smem_raw + (ring - raw) + STAGES * STAGE_BYTES);
     volatile int* abort = &sm->abort;
 
-    const int warp = C::WARP_ISSUE ? __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0)
-                                   : (int)(threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(smem_u32(&sm->full[s]), 1);
@@ -320,49 +301,7 @@ __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
             if (--stage < 0) { stage = STAGES - 1; phase ^= 1u; }
             wait_bounded(smem_u32(&sm->full[stage]), phase, p, abort, false);
         }
-    } else if (C::WARP_ISSUE && warp == 1) {
-        // ---------------- MMA issuer, precise accumulation, whole warp ----------------
-        const uint32_t lead = elect_lane();
-        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
-        int stage = 0, set = 0;
-        uint32_t phase = 0, acc_phase = 0;
-        const uint64_t a_ring = sdesc(ring), b_ring = sdesc(ring + S * A_TILE);
-        bool ok = true;
-        for (int t = blockIdx.x; ok && t < p.total_tiles && !*abort; t = next_tile(p, t)) {
-            const int nkb = (int)(p.g[map_tile(p, t).g].klen / BK);
-            for (int kb0 = 0; kb0 < nkb && ok; kb0 += CH) {
-                ok = warp_wait(smem_u32(&sm->acc_empty[set]), acc_phase ^ 1u, p, abort);
-                const uint32_t dbig = tm + (uint32_t)(set * 2 * BN), dsmall = dbig + BN;
-                const int kb1 = min(nkb, kb0 + CH);
-                for (int kb = kb0; kb < kb1 && ok; ++kb) {
-                    if (!(ok = warp_wait(smem_u32(&sm->full[stage]), phase, p, abort))) break;
-                    const uint64_t A = a_ring + (uint32_t)stage * (STAGE_BYTES >> 4);
-                    const uint64_t B = b_ring + (uint32_t)stage * (STAGE_BYTES >> 4);
-                    const uint32_t on = kb == kb0 ? 0u : 1u;
-#pragma unroll
-                    for (int kk = 0; kk < BK / 16; ++kk) {
-                        const uint64_t a0 = A + kk * 2, b0 = B + kk * 2;
-                        const uint64_t a1 = a0 + (A_TILE >> 4), b1 = b0 + (B_TILE >> 4);
-                        const uint64_t a2 = a1 + (A_TILE >> 4), b2 = b1 + (B_TILE >> 4);
-                        const uint32_t acc_on = kk == 0 ? on : 1u;
-                        umma_elected(dbig, a0, b0, C::IDESC, acc_on, lead);
-                        umma_elected(dsmall, a0, b1, C::IDESC, acc_on, lead);
-                        umma_elected(dsmall, a1, b0, C::IDESC, 1u, lead);
-                        umma_elected(dsmall, a0, b2, C::IDESC, 1u, lead);
-                        umma_elected(dsmall, a1, b1, C::IDESC, 1u, lead);
-                        umma_elected(dsmall, a2, b0, C::IDESC, 1u, lead);
-                    }
-                    umma_commit_elected(smem_u32(&sm->empty[stage]), lead);
-                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
-                }
-                if (!ok) break;
-                umma_commit_elected(smem_u32(&sm->acc_full[set]), lead);
-                if (++set == C::SETS) { set = 0; acc_phase ^= 1u; }
-            }
-        }
-        umma_commit_elected(smem_u32(&sm->drain), lead);
-        warp_wait(smem_u32(&sm->drain), 0, p, abort, false);
-    } else if (P && !C::WARP_ISSUE && warp == 1 && lane == 0) {
+    } else if (P && warp == 1 && (C::ELECT ? elect_lane() : lane == 0)) {
         // ---------------- MMA issuer, precise accumulation ----------------
         int stage = 0;
         uint32_t phase = 0, acc_phase = 0;
@@ -422,7 +361,6 @@ __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
         // warp w: TMEM lanes 32 (w % 4) .., columns [half * HC, half * HC + HC)
         constexpr int HC = BN / 2;
         const int q = warp & 3, half = (warp - 2) >> 2;
-        int set = 0;
         uint32_t acc_phase = 0;
         for (int t = blockIdx.x; t < p.total_tiles; t = next_tile(p, t)) {
             const Tile ti = map_tile(p, t);
@@ -442,14 +380,14 @@ __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
             bool ok = true;
             for (int kb0 = 0; kb0 < nkb; kb0 += CH) {
                 int w = 1;
-                if (lane == 0) w = wait_bounded(smem_u32(&sm->acc_full[set]), acc_phase, p, abort);
+                if (lane == 0) w = wait_bounded(smem_u32(&sm->acc_full[0]), acc_phase, p, abort);
                 w = __shfl_sync(0xffffffffu, w, 0);
                 if (!w) { ok = false; break; }
                 tc_fence_after();
 #pragma unroll
                 for (int cc = 0; cc < HC / 16; ++cc) {
                     float v[16];
-                    const uint32_t ta = tmem + (uint32_t)(set * 2 * BN + half * HC + cc * 16) +
+                    const uint32_t ta = tmem + (uint32_t)(half * HC + cc * 16) +
                                         ((uint32_t)(q * 32) << 16);
                     tmem_ld16(ta, v);
 #pragma unroll
@@ -462,8 +400,8 @@ __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&sm->acc_empty[set]));
-                if (++set == C::SETS) { set = 0; acc_phase ^= 1u; }
+                if (lane == 0) mbar_arrive(smem_u32(&sm->acc_empty[0]));
+                acc_phase ^= 1u;
             }
             if (!ok) break;
             // C := beta C + gamma sum over this thread's row and columns
@@ -710,13 +648,6 @@ cudaError_t tc_configure() {
     cudaError_t e;
     if ((e = tc_configure_s<1>()) != cudaSuccess) return e;
     if ((e = tc_configure_s<2>()) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(tc::gemm_tc_kernel<128, 3, tc::MAXG_SMALL, true>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  tc::Cfg<128, 3>::SMEM_BYTES)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(tc::gemm_tc_kernel<64, 3, tc::MAXG_SMALL, true>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  tc::Cfg<64, 3>::SMEM_BYTES)) != cudaSuccess)
-        return e;
     return tc_configure_s<3>();
 }
 
@@ -739,7 +670,7 @@ cudaError_t tc_make_maps(const Planes& pl, int64_t k, int64_t nrhs, void* out) {
 cudaError_t launch_gemm_tc(const Canon<float>& p, const void* maps, int slices,
                            const TcGemm* gemms, int ngemms, float beta, float gamma,
                            int* err_word, long long wait_ns, int num_sms, cudaStream_t s,
-                           bool diag_beta, const TcYOut* yout, bool branches) {
+                           bool diag_beta, const TcYOut* yout) {
     if (slices < 1 || slices > 3) return cudaErrorInvalidValue;
     using namespace tc;
     for (int g0 = 0; g0 < ngemms; g0 += MAXG) {
@@ -813,11 +744,6 @@ cudaError_t launch_gemm_tc(const Canon<float>& p, const void* maps, int slices,
         else if (slices == 2)
             e = bn == 256 ? TRX_TC_LAUNCH(256, 2) : bn == 128 ? TRX_TC_LAUNCH(128, 2)
                                                               : TRX_TC_LAUNCH(64, 2);
-        else if (branches && small && bn < 256)
-            e = bn == 128 ? launch_kernel(gemm_tc_kernel<128, 3, MAXG_SMALL, true>, dim3(grid),
-                                          dim3(NTHREADS_P), Cfg<128, 3>::SMEM_BYTES, s, prm_small)
-                          : launch_kernel(gemm_tc_kernel<64, 3, MAXG_SMALL, true>, dim3(grid),
-                                          dim3(NTHREADS_P), Cfg<64, 3>::SMEM_BYTES, s, prm_small);
         else
             e = bn == 256 ? TRX_TC_LAUNCH(256, 3) : bn == 128 ? TRX_TC_LAUNCH(128, 3)
                                                               : TRX_TC_LAUNCH(64, 3);

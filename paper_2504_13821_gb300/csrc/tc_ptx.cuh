@@ -63,35 +63,15 @@ __device__ __forceinline__ void umma(uint32_t d, uint64_t a, uint64_t b, uint32_
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
         "l"(a), "l"(b), "r"(idesc), "r"(accum));
 }
-// tcgen05.mma issued by a whole warp through one elected lane (`lead` from
-// elect_lane(), the same for a warp's life). With every lane in the code the
-// descriptors stay in uniform registers: one MMA issues in about 40 clocks, against
-// 128 from a branch that only one lane takes (measured with back-to-back
-// 128 x 64 x 16 MMAs, 48 against 128 clocks each; 128 x 256 x 16 take 128 either
-// way).
-__device__ __forceinline__ uint32_t elect_lane() {
+// True in one lane of a converged warp, which then waits, issues and commits alone. MMAs
+// of fewer than 256 columns issue faster in a branch on this than in one on lane == 0
+// (gemm_tc.cu and gemm_oz.cu have both times).
+__device__ __forceinline__ bool elect_lane() {
     uint32_t r;
     asm volatile(
         "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
         : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void umma_elected(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
-                                             uint32_t accum, uint32_t lead) {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.b32 q, %5, 0;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc), "r"(accum), "r"(lead));
-}
-__device__ __forceinline__ void umma_commit_elected(uint32_t bar, uint32_t lead) {
-    asm volatile(
-        "{\n\t.reg .pred q;\n\t"
-        "setp.ne.b32 q, %1, 0;\n\t"
-        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n"
-        ::"r"(bar), "r"(lead)
-        : "memory");
+    return r != 0;
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile(
