@@ -115,7 +115,6 @@ struct Smem {
     unsigned long long full[STAGES], empty[STAGES];  // the stages of m
     int pushed[ND];          // set by the CTA that has sent a block to `near`
     int task;
-    int abort;
 };
 constexpr unsigned long long kTag = 1ull << 32;
 
@@ -132,6 +131,20 @@ __device__ __forceinline__ void st_relaxed64x2(unsigned long long* p, unsigned l
 
 // barrier of the NT threads that compute
 __device__ __forceinline__ void sync_nt() { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); }
+// The same, and whether any of them passed true: the verdict comes with the barrier, so
+// that all leave a step together (a flag in shared memory could be set for the next
+// step by a fast warp before a slow one has read it for this one).
+__device__ __forceinline__ bool sync_nt_any(bool v) {
+    uint32_t r;
+    asm volatile(
+        "{ .reg .pred p, q; setp.ne.u32 q, %1, 0;\n"
+        "bar.red.or.pred p, 1, %2, q;\n"
+        "selp.u32 %0, 1, 0, p; }"
+        : "=r"(r)
+        : "r"((uint32_t)v), "n"(NT)
+        : "memory");
+    return r != 0;
+}
 
 __device__ __forceinline__ uint64_t gtimer() {
     uint64_t t;
@@ -510,7 +523,6 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT + NTP, 2)
     // panel, one a CTA
     const int rank = cluster_rank();
     if (t == 0) {
-        sm.abort = 0;
         for (int q = 0; q < ND; ++q) {
             sm.pushed[q] = 0;
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&sm.near_full[q])));
@@ -583,19 +595,18 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT + NTP, 2)
         // cluster, X_j into slot i - 1 - j; blocks j < far come from xt
         const int far = min(jz, i - min(rank, ND));
         if (far > 0) issue_x(p, pn, 0, w);
+        bool stop = false;
         for (int j = 0; j < jz; ++j) {
             const int s = (j + 1) % STAGES;
             const bool ok = (j < far ? finish_x(p, sm.x[j & 1], pn, j, w)
                                      : wait_bar(p, &sm.near_full[i - 1 - j], 0)) &&
                             wait_bar(p, &sm.full[s], j / STAGES & 1);
-            if (!ok) sm.abort = 1;
-            sync_nt();   // also: X_j-1 is done with
-            if (sm.abort) break;
+            if ((stop = sync_nt_any(!ok))) break;   // also: X_j-1 is done with
             if (j + 1 < far) issue_x(p, pn, j + 1, w);
             mma_tile(sm.m[s], j < far ? sm.x[j & 1] : sm.near[i - 1 - j], acc);
             release(s);
         }
-        if (sm.abort) break;
+        if (stop) break;
         if (i > 0 && rank == 0) issue_x(p, pn, i - 1, w);
         // P = inv(M_ii) (alpha B - S'), then X = P - Z X_i-1,p
         float* rhs = sm.x[(i + 1) & 1];   // the last product (j = i - 2) reads the other
@@ -609,9 +620,9 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT + NTP, 2)
         mma_tile<true>(sm.inv, rhs, xo);
         if (i > 0) {
             float* prev = sm.x[i & 1];
-            if (!(rank == 0 ? finish_x(p, prev, pn, i - 1, w) : wait_bar(p, &sm.near_full[0], 0))) sm.abort = 1;
-            sync_nt();
-            if (sm.abort) break;
+            const bool ok = rank == 0 ? finish_x(p, prev, pn, i - 1, w)
+                                      : wait_bar(p, &sm.near_full[0], 0);
+            if (sync_nt_any(!ok)) break;
             float zx[2][2] = {};
             mma_tile(sm.z, rank == 0 ? prev : sm.near[0], zx);
 #pragma unroll
