@@ -18,6 +18,8 @@
 // CTAs: the FP64 pipe is about 1/64 of the FP32 one per SM on this part, so
 // a small FP64 update on a few SMs was the FP64 path's bottleneck at small
 // orders.
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace trx {
@@ -203,18 +205,26 @@ __global__ void __launch_bounds__(NT, 2) gemm_pieces_kernel(PieceArgs<TA> g) {
         for (int64_t l0 = k0; l0 < k1; l0 += BK) {
             const bool more = l0 + BK < k1;
             if (more) load(l0 + BK);
+            // a triangle's steps at its diagonal: a row takes part only in the products
+            // left of it (a zero in A's place times an Inf or NaN of Y would be a NaN)
+            const auto products = [&](auto edge) {
 #pragma unroll
-            for (int l = 0; l < BK; ++l) {
-                double a[TM], b[TM];
+                for (int l = 0; l < BK; ++l) {
+                    double a[TM], b[TM];
 #pragma unroll
-                for (int u = 0; u < TM; ++u) a[u] = sA[buf][l][tx + 16 * u];
+                    for (int u = 0; u < TM; ++u) a[u] = sA[buf][l][tx + 16 * u];
 #pragma unroll
-                for (int v = 0; v < TM; ++v) b[v] = sB[buf][l][ty + 16 * v];
+                    for (int v = 0; v < TM; ++v) b[v] = sB[buf][l][ty + 16 * v];
 #pragma unroll
-                for (int u = 0; u < TM; ++u)
+                    for (int u = 0; u < TM; ++u) {
+                        if (decltype(edge)::value && l0 + l >= i0 + tx + 16 * u) continue;
 #pragma unroll
-                    for (int v = 0; v < TM; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
-            }
+                        for (int v = 0; v < TM; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
+                    }
+                }
+            };
+            if (g.pc.tri && l0 + BK > i0) products(std::true_type{});
+            else products(std::false_type{});
             if (more) {
                 store(buf ^ 1);
                 __syncthreads();
