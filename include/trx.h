@@ -319,8 +319,9 @@ int trx_set_workspace(trx_handle_t handle, void* ptr, size_t bytes);
  * tensor-core trx_sgemm_update, with m = M + K and n = N (side 'L').
  * Depends on the handle's options (the CUDA-core path needs none; FP64 TRSM
  * on the mixed engine, TRX_OPT_FP64_TRSM, needs the FP32 solve's). For side R
- * on the FP32 tensor-core path it includes room for B's transpose, without which
- * the call still runs, more slowly. For the recursive FP64 calls it is what their updates on the tensor cores use; with
+ * on the FP32 tensor-core path it includes room for B's transpose, and for TRMM
+ * there a word per 128 rows and right-hand side for the Infs and NaNs of B, without
+ * which the call still runs, more slowly. For the recursive FP64 calls it is what their updates on the tensor cores use; with
  * less the call runs all its updates on the CUDA cores instead.
  * Returns 0 and sets *bytes, or an argument code as for the compute calls. */
 int trx_workspace_size(trx_handle_t handle, char op, char side, int64_t m,

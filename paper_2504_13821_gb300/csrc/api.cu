@@ -154,6 +154,12 @@ size_t turn_bytes(int64_t k, int64_t nrhs) {
     return align256((size_t)nrhs * turn_ld(k) * 4);
 }
 
+// Bytes of the marks of a TRMM's right-hand side (rows gathered into one launch), after
+// the planes: YMarks' any, columns and words.
+size_t marks_bytes(int64_t k, int64_t nrhs) {
+    return 256 + align256((size_t)((k + 127) / 128 + 1) * nrhs * 4);
+}
+
 // Extra workspace of the device-scheduled TRSM after the planes: the
 // diagonal blocks' inverses as `slices` compact k x 128 planes, then the
 // block flags and the task counter.
@@ -222,6 +228,7 @@ struct trx_handle_s {
     // batched substitution block height per [element type][order bucket]
     // [right-hand-side bucket] (trx_batched_autotune); 8 until tuned
     int tune_sb[2][TRX_TUNE_K_BUCKETS][TRX_TUNE_N_BUCKETS] = {};
+    uint32_t mark_stamp = 0;       // of the last call with marks (YMarks)
     // column-panel branches of a TRSM: streams and fork/join events
     int64_t opt_panels = 0;
     int64_t opt_trmm_dense = 0;
@@ -290,6 +297,7 @@ struct Exec {
     // side R solved on B^T: B and its transpose in the workspace
     float *turn_b = nullptr, *turn_t = nullptr;
     int64_t turn_ldb = 0, turn_ldt = 0;
+    YMarks marks;                  // TRMM by rows: Inf and NaN of the right-hand side
     bool turn_flip = false;
     void* oz_ws = nullptr;         // FP64 updates on the tensor cores: operand images
     cudaStream_t s;
@@ -350,13 +358,14 @@ struct Exec {
                         yo.lo = pl.y_lo;
                         yo.lo2 = pl.y_lo2;
                         yo.ld = pl.ldy;
+                        const TcMarks mk{marks, {pl.y_hi, pl.y_lo, pl.y_lo2}, pl.ldy};
                         yo.row0 = st.y0;
                         yo.row1 = st.y1;
                         e = launch_gemm_tc(*reinterpret_cast<const Canon<float>*>(&c),
                                            st.inv ? maps_w : maps, pl.slices, st.gemms.data(),
                                            (int)st.gemms.size(), (float)st.beta, (float)st.gamma,
                                            h->d_err, h->wait_ns, h->num_sms, s, st.dense,
-                                           st.y1 > st.y0 ? &yo : nullptr);
+                                           st.y1 > st.y0 ? &yo : nullptr, marks.words ? &mk : nullptr);
                         cls = st.inv ? TRX_KERNEL_LEAF_TRSM : TRX_KERNEL_GEMM_TC;
                     } else {
                         cls = TRX_KERNEL_GEMM_SIMT;
@@ -397,7 +406,7 @@ struct Exec {
                     bytes = 8.0 * c.k * (c.k - 1) / 2;
                     break;
                 case kConvY:
-                    e = launch_convert_y(*reinterpret_cast<const Canon<float>*>(&c), pl, s);
+                    e = launch_convert_y(*reinterpret_cast<const Canon<float>*>(&c), pl, s, marks);
                     cls = TRX_KERNEL_CONVERT;
                     bytes = 8.0 * c.k * c.nrhs;
                     break;
@@ -656,16 +665,31 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
                        : terms_override ? slices_of_terms(terms_override) : slices_for(h);
     const bool dag = std::is_same<T, float>::value &&
                      use_dag_mode(h->opt_trsm_dag, plan.tc, trsm, (int)sizeof(T), k, ex.c.nrhs);
+    // TRMM on the tensor cores with both sizes left automatic: the recursion's
+    // updates gathered by row into one launch (six-term split: its long K ranges
+    // are summed in FP32 by chunks; with fewer terms they would add up in TMEM),
+    // where the workspace also holds the right-hand side's marks
+    bool rows = false;
     if (plan.tc) {
         const WsLayout w = ws_layout(k, ex.c.nrhs, slices);
         const size_t planes = factor_planes ? (size_t)slices * w.y_bytes : w.total;
-        const size_t need = planes + (dag ? dag_extra_bytes(k, ex.c.nrhs, slices) : 0);
+        size_t need = planes + (dag ? dag_extra_bytes(k, ex.c.nrhs, slices) : 0);
         if (h->ws == nullptr || h->ws_bytes < need) {
             snprintf(g_detail, sizeof(g_detail), "workspace of %zu bytes needed, %zu set",
                      need, h->ws_bytes);
             return TRX_ERR_WORKSPACE;
         }
         char* base = static_cast<char*>(h->ws);
+        rows = !trsm && slices == 3 && h->opt_trmm_dense == 0 && h->opt_leaf == 0 &&
+               h->ws_bytes >= need + marks_bytes(k, ex.c.nrhs);
+        if (rows) {
+            ex.marks.any = reinterpret_cast<uint32_t*>(base + need);
+            ex.marks.columns = ex.marks.any + 64;
+            ex.marks.words = ex.marks.columns + ex.c.nrhs;
+            ex.marks.stamp = ++h->mark_stamp;
+            ex.marks.per_column = (k + 127) / 128;
+            need += marks_bytes(k, ex.c.nrhs);
+        }
         if constexpr (std::is_same<T, float>::value) {
             if (upc(side) == 'R' && !dag && h->opt_panels <= 1 &&
                 turn_applies(k, ex.c.nrhs) &&
@@ -767,11 +791,6 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
                   fits(oz_trmm_bytes(k, ex.c.nrhs));
         if (oz_trmm || fits(oz_workspace(h->opt_gemm, k, ex.c.nrhs, b))) parts[0].oz_ws = h->ws;
     }
-    // TRMM on the tensor cores with both sizes left automatic: the recursion's
-    // updates gathered by row into one launch (six-term split: its long K ranges
-    // are summed in FP32 by chunks; with fewer terms they would add up in TMEM)
-    const bool rows = !trsm && plan.tc && slices == 3 && h->opt_trmm_dense == 0 &&
-                      h->opt_leaf == 0;
     const int dense = trsm   ? 0
                       : rows ? kTrmmRowsDiag
                              : trmm_dense_mode(h->opt_trmm_dense, h->opt_leaf, plan.tc, k);
@@ -1503,6 +1522,7 @@ int trx_workspace_size(trx_handle_t h, char op, char side, int64_t m, int64_t n,
         *bytes = (tc && k > 0 && nrhs > 0) ? (size_t)sl * ws_layout(k, nrhs, sl).y_bytes : 0;
         if (tc_s && k > 0 && nrhs > 0 && use_dag_mode(h->opt_trsm_dag, true, true, 4, k, nrhs))
             *bytes += dag_extra_bytes(k, nrhs, sl);
+        if (*bytes && use_tc<float>(h, k, false, nrhs)) *bytes += marks_bytes(k, nrhs);
         if (*bytes && upc(side) == 'R' && turn_applies(k, nrhs))
             *bytes += turn_bytes(k, nrhs);
         return TRX_SUCCESS;
@@ -1524,6 +1544,7 @@ int trx_workspace_size(trx_handle_t h, char op, char side, int64_t m, int64_t n,
                                     leaf_for(h->opt_leaf, k, o == 'S', 8, nrhs));
     if (*bytes && (elem_bytes == 4 || mixed64) && o == 'S' && use_dag_mode(h->opt_trsm_dag, true, true, 4, k, nrhs))
         *bytes += dag_extra_bytes(k, nrhs, slices_for(h));
+    if (*bytes && elem_bytes == 4 && o == 'M') *bytes += marks_bytes(k, nrhs);
     if (*bytes && elem_bytes == 4 && (o == 'S' || o == 'M') && upc(side) == 'R' &&
         turn_applies(k, nrhs))
         *bytes += turn_bytes(k, nrhs);

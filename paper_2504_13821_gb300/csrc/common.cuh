@@ -103,6 +103,22 @@ struct Planes {
     int slices = 2;
 };
 
+// Where Y planes carry marks (split_slices_marked): words[j * per_column + l / 128]
+// is the call's stamp where rows [l, l + 128) of right-hand side j have an Inf or NaN,
+// columns[j] where any of its rows has one and *any where there is one at all. Nothing
+// else writes them and nothing clears them: a word that holds the stamp from before, as
+// in a replay of the same launches, costs a look at planes without a mark.
+struct YMarks {
+    uint32_t* any = nullptr;
+    uint32_t* columns = nullptr;
+    uint32_t* words = nullptr;
+    int64_t per_column = 0;
+    uint32_t stamp = 0;
+};
+__device__ __forceinline__ void put_mark(const YMarks& m, int64_t l, int64_t j) {
+    *m.any = m.columns[j] = m.words[j * m.per_column + l / 128] = m.stamp;
+}
+
 // Product terms of a split (1, 3, 6) <-> slices per operand (1, 2, 3).
 inline int slices_of_terms(int terms) { return terms == 1 ? 1 : terms == 6 ? 3 : 2; }
 inline int terms_of_slices(int slices) { return slices == 1 ? 1 : slices == 3 ? 6 : 3; }
@@ -125,6 +141,35 @@ __device__ __forceinline__ void split_slices(float x, int slices, __nv_bfloat16 
     const float r = x - __bfloat162float(v[0]);
     v[1] = slices > 1 ? __float2bfloat16_rn(r) : __float2bfloat16_rn(0.f);
     v[2] = slices > 2 ? __float2bfloat16_rn(r - __bfloat162float(v[1])) : __float2bfloat16_rn(0.f);
+}
+// The same for an element that a product's zeros may meet: an Inf or NaN gets slices of
+// value zero, with signs of zero that no finite x has (x >= 0 has no -0 after a first
+// slice of +0, and only x = -0 has a +0 after a first slice of -0, with a third of +0),
+// and the function is true. A finite x that rounds to Inf keeps the largest BF16 there.
+__device__ __forceinline__ bool split_slices_marked(float x, __nv_bfloat16 (&v)[3]) {
+    const uint32_t b = __float_as_uint(x), mag = b & 0x7fffffffu;
+    const auto bf = [](uint32_t u) { return __ushort_as_bfloat16((unsigned short)u); };
+    if (mag >= 0x7f800000u) {
+        const bool nan = mag > 0x7f800000u;
+        v[0] = bf(nan ? 0x8000u : 0u);
+        v[1] = bf(nan ? 0u : 0x8000u);
+        v[2] = bf(nan || (b >> 31) ? 0x8000u : 0u);
+        return true;
+    }
+    v[0] = mag >= 0x7f7f8000u ? bf(b >> 31 << 15 | 0x7f7fu) : __float2bfloat16_rn(x);
+    const float r = x - __bfloat162float(v[0]);
+    v[1] = __float2bfloat16_rn(r);
+    v[2] = __float2bfloat16_rn(r - __bfloat162float(v[1]));
+    return false;
+}
+// Whether three slices are such a mark, and of which value.
+__device__ __forceinline__ bool marked_value(__nv_bfloat16 s0, __nv_bfloat16 s1, __nv_bfloat16 s2,
+                                             float& x) {
+    const uint32_t a = __bfloat16_as_ushort(s0), b = __bfloat16_as_ushort(s1),
+                   c = __bfloat16_as_ushort(s2);
+    const bool inf = a == 0u && b == 0x8000u, nan = a == 0x8000u && b == 0u && c == 0x8000u;
+    x = __uint_as_float(nan ? 0x7fffffffu : c == 0x8000u ? 0xff800000u : 0x7f800000u);
+    return inf || nan;
 }
 // Y-plane element o of the result x (solved rows, TRMM originals).
 __device__ __forceinline__ void put_y(const Planes& pl, int64_t o, float x) {
@@ -213,7 +258,8 @@ cudaError_t launch_turn(const float* src, int64_t lds, float* dst, int64_t ldd, 
 cudaError_t launch_convert_m(const Canon<float>& p, const Planes& pl, int diag_block,
                              cudaStream_t s);
 // Split-BF16 planes of C rows [0,k), all columns (TRMM's original values).
-cudaError_t launch_convert_y(const Canon<float>& p, const Planes& pl, cudaStream_t s);
+cudaError_t launch_convert_y(const Canon<float>& p, const Planes& pl, cudaStream_t s,
+                             const YMarks& marks = {});
 // Y planes of C's rows [r0, r0 + rows) (r0 a multiple of 4).
 cudaError_t launch_convert_y_rows(const Canon<float>& p, const Planes& pl, int64_t r0,
                                   int64_t rows, cudaStream_t s);
@@ -243,6 +289,12 @@ cudaError_t tc_make_maps(const Planes& pl, int64_t k, int64_t nrhs, void* maps_o
 // Optional second output of a tensor-core GEMM: the split BF16 planes (as
 // many slices as the operand planes) of result rows [row0, row1) (canonical rows), element (i, j) at
 // j * ld + i, as the Y planes are laid out.
+// Marked Y planes of an update whose M planes hold zeros.
+struct TcMarks {
+    YMarks at;
+    const __nv_bfloat16* y[3] = {};
+    int64_t ldy = 0;
+};
 struct TcYOut {
     __nv_bfloat16* hi = nullptr;
     __nv_bfloat16* lo = nullptr;
@@ -253,7 +305,7 @@ cudaError_t launch_gemm_tc(const Canon<float>& p, const void* maps, int slices,
                            const TcGemm* gemms, int ngemms, float beta,
                            float gamma, int* err_word, long long wait_limit,
                            int num_sms, cudaStream_t s, bool diag_beta = false,
-                           const TcYOut* yout = nullptr);
+                           const TcYOut* yout = nullptr, const TcMarks* marks = nullptr);
 // Refined TRSM helpers (refine.cu): casts, residual, correction, norms.
 cudaError_t refine_cast_f32_f64(const float* src, int64_t lds, double* dst, int64_t ldd, int64_t m,
                                 int64_t n, double scale, cudaStream_t s);

@@ -134,20 +134,37 @@ __global__ void __launch_bounds__(256) turn_kernel(const float* src, int64_t lds
 }
 
 // Y planes when C's rows are contiguous (side L): no transpose, four
-// consecutive rows per thread, 8-byte stores.
-__global__ void __launch_bounds__(256) convert_y_contig_kernel(Canon<float> p, Planes pl) {
+// consecutive rows per thread, 8-byte stores. MARK: Inf and NaN marked (three slices).
+template <bool MARK>
+__global__ void __launch_bounds__(256) convert_y_contig_kernel(Canon<float> p, Planes pl,
+                                                               YMarks marks) {
     pdl_trigger();
     pdl_wait();
     const int64_t l = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4;
-    if (l >= p.k) return;
+    if (!MARK && l >= p.k) return;
     for (int64_t j = blockIdx.y; j < p.nrhs; j += gridDim.y) {
         const float* src = p.C + j * p.c_cs;
         float v[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) v[q] = (l + q < p.k) ? src[(l + q) * p.c_rs] : 0.f;
         __nv_bfloat16 sl[4][3];
+        if constexpr (MARK) {
+            bool plain = true;            // none that rounds to Inf in BF16, nor a NaN
 #pragma unroll
-        for (int q = 0; q < 4; ++q) split_slices(v[q], pl.slices, sl[q]);
+            for (int q = 0; q < 4; ++q) plain &= fabsf(v[q]) < 0x1.ffp127f;
+            if (__all_sync(0xffffffffu, plain)) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) split_slices(v[q], 3, sl[q]);
+            } else {
+                bool odd = false;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) odd |= split_slices_marked(v[q], sl[q]);
+                if (odd) put_mark(marks, l, j);
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) split_slices(v[q], pl.slices, sl[q]);
+        }
         const int64_t off = j * pl.ldy + l;
         if (l + 3 < p.k) {
             for (int s = 0; s < pl.slices; ++s) {
@@ -162,8 +179,11 @@ __global__ void __launch_bounds__(256) convert_y_contig_kernel(Canon<float> p, P
     }
 }
 
-// Y planes when C's columns are contiguous (side R): 32x32 transpose tiles.
-__global__ void __launch_bounds__(256) convert_y_kernel(Canon<float> p, Planes pl) {
+// Y planes when C's columns are contiguous (side R): 32x32 transpose tiles. MARK: as
+// above.
+template <bool MARK>
+__global__ void __launch_bounds__(256) convert_y_kernel(Canon<float> p, Planes pl,
+                                                        YMarks marks) {
     pdl_trigger();
     pdl_wait();
     __shared__ float tile[32][33];              // tile[jj][ll]
@@ -180,7 +200,15 @@ __global__ void __launch_bounds__(256) convert_y_kernel(Canon<float> p, Planes p
     __syncthreads();
     for (int r = threadIdx.y; r < 32; r += 8) {
         const int64_t j = j0 + r, l = l0 + threadIdx.x;
-        if (l < p.k && j < p.nrhs) put_y(pl, j * pl.ldy + l, tile[r][threadIdx.x]);
+        if constexpr (MARK) {
+            __nv_bfloat16 sl[3];
+            const bool odd = split_slices_marked(tile[r][threadIdx.x], sl);   // (0 outside C)
+            if (l >= p.k || j >= p.nrhs) continue;
+            for (int s = 0; s < 3; ++s) y_plane(pl, s)[j * pl.ldy + l] = sl[s];
+            if (odd) put_mark(marks, l, j);
+        } else if (l < p.k && j < p.nrhs) {
+            put_y(pl, j * pl.ldy + l, tile[r][threadIdx.x]);
+        }
     }
 }
 
@@ -289,18 +317,21 @@ cudaError_t launch_convert_m(const Canon<float>& p, const Planes& pl, int diag_b
                          diag_block / 64);
 }
 
-cudaError_t launch_convert_y(const Canon<float>& p, const Planes& pl, cudaStream_t s) {
+cudaError_t launch_convert_y(const Canon<float>& p, const Planes& pl, cudaStream_t s,
+                             const YMarks& marks) {
     if (p.k <= 0 || p.nrhs <= 0) return cudaSuccess;
+    if (marks.words && pl.slices != 3) return cudaErrorInvalidValue;
     if (p.c_rs == 1 || p.c_rs == -1) {
         const int64_t gx = (p.k + 1023) / 1024;
         const int64_t gy = p.nrhs < 65535 ? p.nrhs : 65535;
-        return launch_kernel(convert_y_contig_kernel, dim3((unsigned)gx, (unsigned)gy), dim3(256),
-                             0, s, p, pl);
+        return launch_kernel(
+            marks.words ? convert_y_contig_kernel<true> : convert_y_contig_kernel<false>,
+            dim3((unsigned)gx, (unsigned)gy), dim3(256), 0, s, p, pl, marks);
     }
     const int64_t tl = (p.k + 31) / 32, tj = (p.nrhs + 31) / 32;
     if (tj > 65535) return cudaErrorInvalidValue;
-    return launch_kernel(convert_y_kernel, dim3((unsigned)tl, (unsigned)tj), dim3(32, 8), 0, s, p,
-                         pl);
+    return launch_kernel(marks.words ? convert_y_kernel<true> : convert_y_kernel<false>,
+                         dim3((unsigned)tl, (unsigned)tj), dim3(32, 8), 0, s, p, pl, marks);
 }
 
 cudaError_t launch_invert_diag(const Canon<float>& p, int b, __nv_bfloat16* w_hi,

@@ -116,6 +116,8 @@ struct Params {
     int diag_beta, unit;
     const float* dA;
     int64_t d_step;
+    int64_t a_rs;                   // M(i, l) = dA[i * a_rs + l * (d_step - a_rs)]
+    TcMarks marks;                  // of the Y planes, or none
     // optional second output: the split BF16 planes of result rows
     // [y_row0, y_row1) (canonical rows), element (i, j) at y[j * ldy + i]
     __nv_bfloat16* y_hi;
@@ -222,6 +224,39 @@ __device__ __forceinline__ Tile map_tile(const PP& p, int t) {
     r.m = first + idx % gm;
     r.n = idx / gm;
     return r;
+}
+
+// The products of row i (a warp's lanes: 32 rows from a multiple of 32 on; `in`: inside
+// C) with the marked elements of right-hand sides j0 .. j0 + cols - 1, which count as
+// zeros in the planes, onto C: Inf or NaN from there on.
+__device__ __noinline__ void add_marked(const Params& p, int64_t i, bool in, int64_t j0, int cols) {
+    const TcMarks& y = p.marks;
+    const int lane = threadIdx.x & 31;
+    const int64_t a_cs = p.d_step - p.a_rs;
+    // the stamped ones of n words, from the first to the last
+    const auto each = [&](const uint32_t* words, int64_t n, auto&& f) {
+        for (int64_t w = 0; w < n; w += 32) {
+            uint32_t hits = __ballot_sync(
+                0xffffffffu, w + lane < n && __ldg(words + w + lane) == y.at.stamp);
+            for (; hits; hits &= hits - 1) f(w + __ffs(hits) - 1);
+        }
+    };
+    each(y.at.columns + j0, min((int64_t)cols, p.nrhs - j0), [&](int64_t c) {
+        const int64_t j = j0 + c;
+        float sum = 0.f;
+        bool any = false;
+        each(y.at.words + j * y.at.per_column, (i - lane) / 128 + 1, [&](int64_t t) {
+            for (int64_t l = 128 * t; in && l < i && l < 128 * (t + 1); ++l) {
+                const int64_t o = j * y.ldy + l;
+                float v;
+                if (!marked_value(y.y[0][o], y.y[1][o], y.y[2][o], v)) continue;
+                sum = fmaf(p.dA[i * p.a_rs + l * a_cs], v, sum);
+                any = true;
+            }
+        });
+        float* dst = p.C + i * p.c_rs + j * p.c_cs;
+        if (any) *dst = fmaf(p.gamma, sum, *dst);
+    });
 }
 
 template <int BN, int S, int MG>
@@ -404,6 +439,8 @@ __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
                 acc_phase ^= 1u;
             }
             if (!ok) break;
+            const bool marked = ParamsT<MG>::LONG && p.marks.at.words &&
+                                __ldcg(p.marks.at.any) == p.marks.at.stamp;
             // C := beta C + gamma sum over this thread's row and columns
 #pragma unroll
             for (int cc = 0; cc < HC / 16; ++cc) {
@@ -432,6 +469,7 @@ __global__ void __launch_bounds__(Precise<S>::value ? NTHREADS_P : NTHREADS, 1)
                     }
                 }
             }
+            if (marked) add_marked(p, grow, row_ok, jbase, HC);
         }
     } else if (!P && warp == 1 && lane == 0) {
         // ---------------- MMA issuer ----------------
@@ -670,8 +708,9 @@ cudaError_t tc_make_maps(const Planes& pl, int64_t k, int64_t nrhs, void* out) {
 cudaError_t launch_gemm_tc(const Canon<float>& p, const void* maps, int slices,
                            const TcGemm* gemms, int ngemms, float beta, float gamma,
                            int* err_word, long long wait_ns, int num_sms, cudaStream_t s,
-                           bool diag_beta, const TcYOut* yout) {
+                           bool diag_beta, const TcYOut* yout, const TcMarks* marks) {
     if (slices < 1 || slices > 3) return cudaErrorInvalidValue;
+    if (marks && (slices != 3 || !diag_beta)) return cudaErrorInvalidValue;
     using namespace tc;
     for (int g0 = 0; g0 < ngemms; g0 += MAXG) {
         const int ng = (ngemms - g0) < MAXG ? (ngemms - g0) : MAXG;
@@ -696,6 +735,8 @@ cudaError_t launch_gemm_tc(const Canon<float>& p, const void* maps, int slices,
         prm.unit = p.unit;
         prm.dA = p.A;
         prm.d_step = p.a_rs + p.a_cs;
+        prm.a_rs = p.a_rs;
+        prm.marks = marks ? *marks : TcMarks{};
         prm.y_hi = yout ? yout->hi : nullptr;
         prm.y_lo = yout ? yout->lo : nullptr;
         prm.y_lo2 = yout ? yout->lo2 : nullptr;

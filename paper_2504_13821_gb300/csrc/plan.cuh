@@ -192,8 +192,11 @@ inline void plan_trmm_levels(Plan& pl, int64_t k, int b, double alpha, bool dens
 // runs over the same terms in 256-term chunks added in FP32, as inside one
 // update. Measured against the leaves and levels (us, order x right-hand
 // sides): 500 x 300 50 -> 33, 1000 x 100 57 -> 34, 1024 x 1024 equal, 4096 x 4096
-// 467 -> 353, 8192 x 40 239 -> 216, 16384 x 16384 17037 -> 16314; side R
-// 5000 x 3000 1059 -> 608; the error is 0.27-0.99 of theirs.
+// 467 -> 357, 8192 x 40 239 -> 216, 16384 x 16384 17037 -> 16314; side R
+// 5000 x 3000 1059 -> 608; the error is 0.27-0.99 of theirs. A tile's K range ends in
+// its own diagonal block, whose planes hold zeros right of each row: an Inf or NaN of
+// the right-hand side counts as zero there too (a mark in the Y planes), and the
+// epilogue adds its products to the rows below it (gemm_tc.cu, add_marked).
 inline void plan_trmm_rows(Plan& pl, int64_t k, double alpha) {
     pl.steps.push_back(Step{kConvY});
     Step d{kGemm};

@@ -173,6 +173,8 @@ size_t cost_bytes(const trx_server_s* s, const Req& r) {
     if (tc_call && fp32_solve) b += 6 * (size_t)f.k * (size_t)(f.k + nrhs);
     if (tc_call && f.elem == 4 && r.op != 'R' && upc(r.side) == 'R')
         b += 4 * (size_t)f.k * (size_t)nrhs;           // B's transpose
+    if (tc_call && f.elem == 4 && upc(r.op) == 'M')
+        b += ((size_t)(f.k + 127) / 128 + 1) * 4 * (size_t)nrhs;   // B's marks
     return b;
 }
 

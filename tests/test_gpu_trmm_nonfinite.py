@@ -1,7 +1,7 @@
 """TRMM with an Inf or NaN in the right-hand side: rows that do not depend on it are
-those of the call without it, its own row and the rows below are the CUDA cores'
-results (FP64) or not finite where those are not (FP32). Positions inside and at the edges of
-the kernels' row tiles (4, 16, 32, 64, 128), orders of one and of several tiles."""
+those of the call without it, its own row and the rows below are Inf and NaN where the
+CUDA cores' are. Positions inside and at the edges of the kernels' row tiles (4, 16, 32,
+64, 128), orders of one and of several tiles, every tile width."""
 import numpy as np
 import pytest
 
@@ -69,3 +69,50 @@ def test_f64(variant, k):
         assert np.all(fine[:r, c]) and not fine[r, c]
         assert np.abs(out[:r, c] - clean[:r, c]).max(initial=0.0) <= tol
     assert np.abs(out - ref)[fine].max() <= tol
+
+
+@pytest.mark.parametrize("factor", [False, True], ids=["call", "factor"])
+@pytest.mark.parametrize("variant", VARIANTS, ids="".join)
+@pytest.mark.parametrize("k,n", [(256, 45), (300, 70), (700, 100), (1100, 45), (1100, 2200),
+                                 (1100, 4400)])
+def test_f32_by_rows(variant, k, n, factor):
+    import paper_2504_13821_gb300 as trx
+    m_, n_ = (k, n) if variant[0] == "L" else (n, k)
+    A, B = inputs.problem(variant[0], variant[1], m_, n_, seed=k, dtype=np.float32,
+                          poison_diag=variant[3] == "U")
+    where = places(k)
+    B1 = spoilt(B, *variant[:3], where)
+    if factor:
+        At, got = to_dev(A, "cuda:0"), []
+        f = trx.Factor(*variant, At)
+        for z in (B, B1):
+            Bt = to_dev(z, "cuda:0")
+            f.trmm(0.5, Bt)
+            got.append(canonical(Bt.cpu().numpy(), *variant[:3]))
+        f.close()
+        clean, out = got
+    else:
+        clean, out = product(variant, A, B), product(variant, A, B1)
+    ref = product(variant, A, B1, 1)
+    assert np.array_equal(np.isnan(out), np.isnan(ref))
+    assert np.array_equal(np.isposinf(out), np.isposinf(ref))
+    assert np.array_equal(np.isneginf(out), np.isneginf(ref))
+    for r, c, _ in where:
+        assert np.array_equal(out[:r, c], clean[:r, c]) and not np.isfinite(out[r, c])
+    rest = np.setdiff1d(np.arange(n), [c for _, c, _ in where])
+    assert np.array_equal(out[:, rest], clean[:, rest])
+
+
+@pytest.mark.parametrize("variant", VARIANTS[::3], ids="".join)
+def test_f32_largest_finite_values(variant):
+    """Entries that round to Inf in BF16 are no Inf: a row's sum has three roundings a term
+    at most in the split form and k in the CUDA cores' chain, of |m||c| below 4e38 / k."""
+    k, n = 400, 45
+    m_, n_ = (k, n) if variant[0] == "L" else (n, k)
+    A, B = inputs.problem(variant[0], variant[1], m_, n_, seed=4, dtype=np.float32)
+    where = [(r, c, (-1) ** c * np.float32(3.4e38)) for c, r in enumerate(range(0, 400, 37))]
+    B1 = spoilt(B, *variant[:3], where)
+    out, ref = product(variant, A, B1), product(variant, A, B1, 1)
+    fine = np.isfinite(ref)     # (not where diagonal times entry overflows before alpha)
+    assert np.isfinite(out[fine]).all()
+    assert np.abs(out.astype(float) - ref)[fine].max() <= 8 * k * 2.0 ** -24 * 3.4e38
