@@ -358,22 +358,46 @@ template <bool LOWER = false>
 __device__ __forceinline__ void mma_tile(const float* a, const float* x, float (&acc)[2][2]) {
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31, ct = l & 3, kg = (l >> 2) & 3;
     const int row = 32 * (w >> 2) + 4 * (w & 3) + 16 * (l >> 4);   // the four rows' first
-    const int kend = LOWER ? 32 * (w >> 2) + 4 * (w & 3) + 20 : BR;
+    const int kend = LOWER ? 32 * (w >> 2) + 4 * (w & 3) : BR;
     const float* ap = a + kg * LD + row;
     const float* xp = x + kg * NP + 4 * ct;
     uint64_t s0[4] = {}, s1[4] = {};       // rows 0, 1 and 2, 3 of the tile by column
 #pragma unroll 8
     for (int kk = 0; kk < kend; kk += 4) {
         const ulonglong2 m = *reinterpret_cast<const ulonglong2*>(ap + kk * LD);
-        float4 v = *reinterpret_cast<const float4*>(xp + kk * NP);
-        // (lower: nothing right of the tile takes part, as a zero times an Inf there
-        // would make a NaN)
-        if (LOWER && kk > row) v = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 v = *reinterpret_cast<const float4*>(xp + kk * NP);
         const uint64_t b[4] = {pk2(v.x, v.x), pk2(v.y, v.y), pk2(v.z, v.z), pk2(v.w, v.w)};
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             s0[c] = fma2(m.x, b[c], s0[c]);
             s1[c] = fma2(m.y, b[c], s1[c]);
+        }
+    }
+    if constexpr (LOWER) {
+        // the warp's two tiles of rows: nothing right of a row takes part (a zero times
+        // an Inf there would make a NaN)
+        float s[4][4];                     // row, column
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            upk2(s0[c], s[0][c], s[1][c]);
+            upk2(s1[c], s[2][c], s[3][c]);
+        }
+#pragma unroll
+        for (int u = 0; u < 5; ++u) {
+            const int kk = kend + 4 * u, left = row - kk - kg;   // rows below: r + left >= 0
+            const float4 m = *reinterpret_cast<const float4*>(ap + kk * LD);
+            const float4 v = *reinterpret_cast<const float4*>(xp + kk * NP);
+            const float a[4] = {m.x, m.y, m.z, m.w}, b[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (r + left >= 0) s[r][c] = fmaf(a[r], b[c], s[r][c]);
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            s0[c] = pk2(s[0][c], s[1][c]);
+            s1[c] = pk2(s[2][c], s[3][c]);
         }
     }
     // lanes kg and kg ^ 1 swap row pairs, then kg and kg ^ 2 column pairs
