@@ -112,15 +112,11 @@ __global__ void __launch_bounds__(128) leaf64_kernel(LeafArgs<double> a) {
 #pragma unroll
         for (int u = 0; u < S::RU; ++u) sC[(s0 + sg + S::L * u) * S::LDC + sc] = x[u];
         __syncthreads();
-        // rank-16 update of the rows below
+        // rank-16 update of the rows below: the 16 products are summed before they meet
+        // the row, whose roundings stay as few as an update's between leaves
         constexpr int UMAX = S::B / S::SB - 1;
         const int nu = UMAX - s0 / S::SB;                  // compile-time after unrolling
-        double acc[UMAX][S::CW];
-#pragma unroll
-        for (int u = 0; u < UMAX; ++u)
-#pragma unroll
-            for (int w = 0; w < S::CW; ++w)
-                if (u < nu) acc[u][w] = sC[(s0 + S::SB * (u + 1) + rg) * S::LDC + cg * S::CW + w];
+        double acc[UMAX][S::CW] = {};
 #pragma unroll
         for (int kk = 0; kk < S::SB; ++kk) {
             double xv[S::CW];
@@ -138,7 +134,7 @@ __global__ void __launch_bounds__(128) leaf64_kernel(LeafArgs<double> a) {
         for (int u = 0; u < UMAX; ++u)
 #pragma unroll
             for (int w = 0; w < S::CW; ++w)
-                if (u < nu) sC[(s0 + S::SB * (u + 1) + rg) * S::LDC + cg * S::CW + w] = acc[u][w];
+                if (u < nu) sC[(s0 + S::SB * (u + 1) + rg) * S::LDC + cg * S::CW + w] += acc[u][w];
         __syncthreads();
     }
 #pragma unroll
