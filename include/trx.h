@@ -104,7 +104,7 @@ enum {
                               the larger ones to the tensor cores where the
                               workspace allows (64-bit fixed-point rows in
                               eight BF16 digits, exact integer sums: error
-                              below 4 u |op(A)||B| per element, elements
+                              below 8 u |op(A)||B| per element, elements
                               that cannot hold it computed by DFMA)        */
     TRX_OPT_GRAPH = 3,     /* 1 (default): replay the launch chain as a
                               cached CUDA graph; 0: launch directly         */

@@ -23,14 +23,15 @@
 // only where nearly all digits are near 128 (P is then above K' / 40). Chunks are
 // added up exactly in 64-bit integers (levels 2-6) and in FP32 values of two
 // digits (levels 7-8, level 9 rounded to 2^-64). Left out: the digit products of
-// weight below 2^-72. In units of the scaled operands a segment's
+// i + j >= 10, below 0.88 2^-63 a term; the rounding of the operands adds 0.25 2^-63 and
+// that of level 9 as much a chunk. In units of the scaled operands a segment's
 // error is below K' 2^-62, K' the smaller count of non-zeros of the two rows.
 //
 // When it applies. That error is relative to the rows' largest entries, not
 // to sum |m||c| as an FMA chain's is. So the kernel also forms P = |M||C| (one
 // BF16 product of the rounded-down magnitudes, 3 % more work) and keeps the
 // sum of a 32-row x BN/2-column piece only where P >= K' 2^-12 for every
-// element, i.e. where its error is below 4 u sum |m||c| (u = 2^-53; the bound
+// element, i.e. where its error is below 8 u sum |m||c| (u = 2^-53; the bound
 // of a K-term FMA chain is K u sum |m||c|). The sums of pieces that fail, or that
 // hold an Inf, a NaN or a row outside 2^+-300, are not added but flagged, and
 // the DFMA kernel (gemm_simt.cu), launched after this one over the flagged
