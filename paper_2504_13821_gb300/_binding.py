@@ -183,8 +183,19 @@ def _char(x: str) -> bytes:
     return x.encode()
 
 
+def _torch_stream(stream, device):
+    """The torch stream of a call's stream argument (None: the current one)."""
+    import torch
+    if stream is None or hasattr(stream, "cuda_stream"):
+        return stream
+    return (torch.cuda.ExternalStream(int(stream), device=device) if int(stream)
+            else torch.cuda.default_stream(device))
+
+
 class Handle:
     """A trx handle on one CUDA device, with a torch-allocated workspace."""
+
+    RETRY = 64                   # offer_workspace
 
     def __init__(self, device=None):
         import torch
@@ -195,6 +206,7 @@ class Handle:
         _check(lib.trx_create(ctypes.byref(self._h), self.device.index, 0), "trx_create")
         self._ws = None
         self._ws_bytes = 0
+        self._declined, self._declined_calls = float("inf"), 0
 
     @property
     def ptr(self):
@@ -237,18 +249,35 @@ class Handle:
                "trx_set_workspace")
         self._ws, self._ws_bytes = ws, nbytes
 
-    def offer_workspace(self, nbytes: int):
-        """Grow the workspace to nbytes where that is possible: an FP64 call
-        uses it for its tensor-core updates and runs without it on the CUDA
-        cores (no growth under a stream capture, which cannot synchronise,
-        nor past the device's memory)."""
+    def offer_workspace(self, nbytes: int, stream=None):
+        """Grow the workspace to nbytes where that leaves the caller room: an
+        FP64 call uses it for its tensor-core updates and runs without it on
+        the CUDA cores. Not under a capture of the call's stream, which cannot
+        synchronise, and not for more than a quarter of the memory that is
+        free on the device or in torch's cache. A size that was declined is
+        not looked at again for the next RETRY calls that ask for as much (an
+        allocation that fails empties torch's cache)."""
         import torch
-        if torch.cuda.is_current_stream_capturing():
+        if nbytes <= self._ws_bytes:
             return
-        try:
-            self.ensure_workspace(nbytes)
-        except torch.cuda.OutOfMemoryError:
-            pass
+        if nbytes >= self._declined and self._declined_calls < self.RETRY:
+            self._declined_calls += 1
+            return
+        with torch.cuda.device(self.device), torch.cuda.stream(_torch_stream(stream, self.device)):
+            if torch.cuda.is_current_stream_capturing():
+                return
+            free = torch.cuda.mem_get_info(self.device)[0]
+            if nbytes > free // 4:
+                free += (torch.cuda.memory_reserved(self.device)
+                         - torch.cuda.memory_allocated(self.device))
+            try:
+                if nbytes <= free // 4:
+                    self.ensure_workspace(nbytes)
+                    self._declined = float("inf")
+                    return
+            except torch.cuda.OutOfMemoryError:
+                pass
+        self._declined, self._declined_calls = nbytes, 0
 
     def profile(self, reset: bool = False) -> dict:
         p = _Profile()
@@ -319,7 +348,7 @@ def _call(op: str, side, uplo, trans, diag, alpha, A, B, handle=None, stream=Non
         if elem == 4 or op == "trsm" and h.get_option(OPT_FP64_TRSM) > 0:
             h.ensure_workspace(need)
         else:
-            h.offer_workspace(need)
+            h.offer_workspace(need, stream)
     if stream is None:
         stream = torch.cuda.current_stream(B.device)
     s_ptr = stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
