@@ -1073,11 +1073,22 @@ int batch_descs(trx_handle_t h, int elem_bytes, int64_t count, const trx_problem
             out.push_back(piece);
         }
     }
-    // largest first; FP32: a chunk's steps cost about as much as 16 columns more
+    // largest first, in the problems' order where equal; FP32: a chunk's steps cost about as
+    // much as 16 columns more. Sorted as one word each (the size's bits, the index), a
+    // descriptor moves once: 4504 of them 415 -> 305 us.
     const double extra = elem_bytes == 4 ? 16 : 0;
-    std::stable_sort(out.begin(), out.end(), [extra](const BatchDesc& x, const BatchDesc& y) {
-        return (double)x.k * x.k * (x.nrhs + extra) > (double)y.k * y.k * (y.nrhs + extra);
-    });
+    std::vector<uint64_t> order(out.size());
+    for (size_t i = 0; i < out.size(); ++i) {
+        const float size = (float)((double)out[i].k * out[i].k * (out[i].nrhs + extra));
+        uint32_t bits;
+        std::memcpy(&bits, &size, sizeof(bits));           // (positive: ordered as it is)
+        order[i] = (uint64_t)~bits << 32 | (uint32_t)i;
+    }
+    std::sort(order.begin(), order.end());
+    std::vector<BatchDesc> sorted;
+    sorted.reserve(out.size());
+    for (const uint64_t o : order) sorted.push_back(out[(uint32_t)o]);
+    out.swap(sorted);
     return TRX_SUCCESS;
 }
 
