@@ -51,7 +51,10 @@
 // and the launch's stop word, and every waiting CTA then stops.
 //
 // Arithmetic: FP32 FMA throughout (no operand split), partial sums in a
-// fixed order, so results are bitwise repeatable.
+// fixed order, so results are bitwise repeatable. A product with the inverted block
+// leaves a residual of the size of |M_ii| |inv(M_ii)| |right-hand side|, which an
+// ill-conditioned block makes larger than substitution's; such blocks (kMaxGrowth) keep
+// M_ii and M_i,i-1 in place of the inverse and Z, and are solved by substitution.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -70,6 +73,12 @@ constexpr int ND = 4;                // block rows that a CTA pushes its block t
 constexpr size_t kAlone = 120 * 1024;   // shared memory that leaves no room for a second CTA
 constexpr int NTP = 128;             // threads of the solve that bring in M
 constexpr int kTimeout = 4;          // TRX_ERR_TIMEOUT
+// Largest |inv(M_ii)| |M_ii| 1 (over rows, in parts of eight columns) of a block that is
+// solved by its inverse. Right-hand sides M x of random 64 x 64 triangles, entries below
+// the diagonal up to s (diagonal 1 + |N(0,1)|): the componentwise backward error of
+// substitution / of the inverse is 4.1e-7 / 1.0e-7 at s = 1/16 (growth 3), 1.9e-7 /
+// 2.2e-7 at 1/2 (29), 1.6e-7 / 1.2e-6 at 1 (370).
+constexpr float kMaxGrowth = 32.0f;
 
 struct Params {
     int64_t k, nrhs;
@@ -106,8 +115,10 @@ struct Smem {
     // a task's sum sits in stage (j + 1) % STAGES (stage 0 also serves as the
     // work tile of the inverse and of Z before)
     float m[STAGES][BR * LD];
-    float inv[BR * LD];      // inv(M_ii), k-major: inv[kk * LD + r] = Inv[r][kk]
-    float z[BR * LD];        // Z = inv(M_ii) M_i,i-1, k-major
+    // inv(M_ii), k-major: inv[kk * LD + r] = Inv[r][kk], and Z = inv(M_ii) M_i,i-1; with
+    // inv[BR] != 0 M_ii with its diagonal's reciprocals, and M_i,i-1
+    float inv[BR * LD];
+    float z[BR * LD];
     float x[2][BR * NP];     // X_jp tiles / right-hand side: x[.][kk * NP + c]
     float near[ND][BR * NP];  // X_i-1 .. X_i-ND as the cluster's CTAs push them
     float dinv[BR];
@@ -423,9 +434,12 @@ __device__ __forceinline__ void mma_tile(const float* a, const float* x, float (
 // M y = e_c for columns c = 8w .. 8w + 7, lane l holding rows l and l + 32:
 // at step r the lane owning row r finishes y_r = (delta_rc - s_r) / m_rr
 // (reciprocal of m_rr made once), broadcasts it, and every lane adds
-// m_row,r y_r into the partial sums of its later rows.
-__device__ void invert_diag(const Params& p, Smem& sm, int64_t i0) {
+// m_row,r y_r into the partial sums of its later rows. Returns whether the block is to be
+// solved by substitution (then M_ii itself is in sm.inv).
+__device__ bool invert_diag(const Params& p, Smem& sm, int64_t i0) {
     float* T = sm.m[0];
+    float* V = sm.x[0];                                    // |M_ii| 1
+    unsigned* growth = reinterpret_cast<unsigned*>(sm.x[1]);
     const int t = threadIdx.x, w = t >> 5, l = t & 31;
     const bool colmajor = p.a_rs == 1 || p.a_rs == -1;
     // all loads in flight at once (one after the other they took most of the time)
@@ -444,7 +458,15 @@ __device__ void invert_diag(const Params& p, Smem& sm, int64_t i0) {
         T[rr * LDT + cc] = v[q];
     }
     sync_nt();
-    if (t < BR) sm.dinv[t] = 1.0f / T[t * LDT + t];
+    if (t < BR) {
+        sm.dinv[t] = 1.0f / T[t * LDT + t];
+        float sum = 0.0f;
+#pragma unroll 16
+        for (int c = 0; c < BR; ++c) sum += fabsf(T[t * LDT + c]);
+        V[t] = sum;
+    } else if (t == BR) {
+        *growth = 0u;
+    }
     sync_nt();
     float y0[8], y1[8];          // rows l and l + 32, columns 8 w + u
 #pragma unroll
@@ -473,21 +495,47 @@ __device__ void invert_diag(const Params& p, Smem& sm, int64_t i0) {
     }
     // s_r accumulated with +: the recurrence above keeps s = sum m y and
     // y_r = (delta - s) / m_rr
+    float g0 = 0.0f, g1 = 0.0f;
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
         sm.inv[(8 * w + u) * LD + l] = y0[u];
         sm.inv[(8 * w + u) * LD + l + 32] = y1[u];
+        g0 = fmaf(fabsf(y0[u]), V[8 * w + u], g0);
+        g1 = fmaf(fabsf(y1[u]), V[8 * w + u], g1);
     }
+    // (bits of numbers that are not negative, or of a NaN: ordered as they are)
+    const unsigned g = __reduce_max_sync(0xffffffffu, max(__float_as_uint(g0), __float_as_uint(g1)));
+    if (l == 0) atomicMax(growth, g);
     sync_nt();
+    const bool subst = *growth > __float_as_uint(kMaxGrowth);
+    if (subst)
+        for (int e = t; e < BR * BR; e += NT) {
+            const int kk = e / BR, r = e % BR;
+            sm.inv[kk * LD + r] = r > kk ? T[r * LDT + kk] : r == kk ? sm.dinv[r] : 0.0f;
+        }
+    if (t == 0) sm.inv[BR] = subst ? 1.0f : 0.0f;
+    sync_nt();
+    return subst;
 }
 
 // Z = inv(M_ii) M_i,i-1 into sm.z (k-major), M_i,i-1 staged row-major in
 // sm.m; thread (ty, tx) forms rows 4 ty .. 4 ty + 3, columns tx + 16 u
-// (inv is lower: terms q < 8 (warp + 1) only).
-__device__ void make_z(const Params& p, Smem& sm, int64_t i0, bool colmajor) {
+// (inv is lower: terms q < 8 (warp + 1) only). For a block solved by substitution
+// M_i,i-1 itself.
+__device__ void make_z(const Params& p, Smem& sm, int64_t i0, bool colmajor, bool subst) {
     float r[16];
     load_m(p, i0, i0 - BR, colmajor, r);
     const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
+    if (subst) {
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            const int rr = colmajor ? (t & 63) : (t >> 6) + 4 * q;
+            const int cc = colmajor ? (t >> 6) + 4 * q : (t & 63);
+            sm.z[cc * LD + rr] = r[q];
+        }
+        sync_nt();
+        return;
+    }
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
         const int rr = colmajor ? (t & 63) : (t >> 6) + 4 * q;
@@ -519,6 +567,42 @@ __device__ void make_z(const Params& p, Smem& sm, int64_t i0, bool colmajor) {
     sync_nt();
 }
 
+// rhs := inv(M_ii) rhs by substitution, M_ii in sm.inv as above; a warp two columns, a
+// lane rows l and l + 32.
+__device__ __noinline__ void substitute(const Smem& sm, float* rhs) {
+    const int l = threadIdx.x & 31, c0 = 2 * (threadIdx.x >> 5);
+    float v0[2], v1[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        v0[c] = rhs[l * NP + c0 + c];
+        v1[c] = rhs[(l + 32) * NP + c0 + c];
+    }
+#pragma unroll 4
+    for (int r = 0; r < 32; ++r) {
+        const float d = sm.inv[r * LD + r], m0 = sm.inv[r * LD + l], m1 = sm.inv[r * LD + l + 32];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const float x = __shfl_sync(0xffffffffu, v0[c], r) * d;
+            v0[c] = l > r ? fmaf(-m0, x, v0[c]) : l == r ? x : v0[c];
+            v1[c] = fmaf(-m1, x, v1[c]);
+        }
+    }
+#pragma unroll 4
+    for (int r = 32; r < BR; ++r) {
+        const float d = sm.inv[r * LD + r], m1 = sm.inv[r * LD + l + 32];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const float x = __shfl_sync(0xffffffffu, v1[c], r - 32) * d;
+            v1[c] = l + 32 > r ? fmaf(-m1, x, v1[c]) : l + 32 == r ? x : v1[c];
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        rhs[l * NP + c0 + c] = v0[c];
+        rhs[(l + 32) * NP + c0 + c] = v1[c];
+    }
+}
+
 // inv(M_ii) and Z_i = inv(M_ii) M_i,i-1 of block row blockIdx.x into
 // p.invz, by the same code (so the same values) as a task of the solve
 // makes them; with several panels every task of a block row would repeat it.
@@ -527,8 +611,8 @@ __global__ void __launch_bounds__(NT) thin_prep_kernel(const Params p, float* in
     Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
     const int i = blockIdx.x;
     const int64_t i0 = (int64_t)i * BR;
-    invert_diag(p, sm, i0);
-    if (i > 0) make_z(p, sm, i0, p.a_rs == 1 || p.a_rs == -1);
+    const bool subst = invert_diag(p, sm, i0);
+    if (i > 0) make_z(p, sm, i0, p.a_rs == 1 || p.a_rs == -1, subst);
     float4* dst = reinterpret_cast<float4*>(invz + (size_t)i * 2 * BR * LD);
     for (int e = threadIdx.x; e < BR * LD / 4; e += NT) {
         dst[e] = reinterpret_cast<const float4*>(sm.inv)[e];
@@ -605,8 +689,8 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT + NTP, 2)
             }
             cp_commit();
         } else {
-            invert_diag(p, sm, i0);
-            if (i > 0) make_z(p, sm, i0, colmajor);
+            const bool subst = invert_diag(p, sm, i0);
+            if (i > 0) make_z(p, sm, i0, colmajor, subst);
         }
         const auto release = [&](int s) {
             __syncwarp();
@@ -640,8 +724,9 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT + NTP, 2)
                 fmaf(p.alpha, b[e & 1][e >> 1], -acc[e & 1][e >> 1]);
         if (p.invz) asm volatile("cp.async.wait_group 0;" ::: "memory");
         sync_nt();
+        const bool subst = sm.inv[BR] != 0.0f;
         float xo[2][2] = {};
-        mma_tile<true>(sm.inv, rhs, xo);
+        if (!subst) mma_tile<true>(sm.inv, rhs, xo);
         if (i > 0) {
             float* prev = sm.x[i & 1];
             const bool ok = rank == 0 ? finish_x(p, prev, pn, i - 1, w)
@@ -650,7 +735,18 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT + NTP, 2)
             float zx[2][2] = {};
             mma_tile(sm.z, rank == 0 ? prev : sm.near[0], zx);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) xo[e & 1][e >> 1] -= zx[e & 1][e >> 1];
+            for (int e = 0; e < 4; ++e) {
+                if (subst) rhs[(own.row + (e & 1)) * NP + own.col + (e >> 1)] -= zx[e & 1][e >> 1];
+                else xo[e & 1][e >> 1] -= zx[e & 1][e >> 1];
+            }
+        }
+        if (subst) {
+            sync_nt();
+            substitute(sm, rhs);
+            sync_nt();
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                xo[e & 1][e >> 1] = rhs[(own.row + (e & 1)) * NP + own.col + (e >> 1)];
         }
         // publish the block (tagged words: the chain), then the result in C
         unsigned long long* dst = p.xt + ((int64_t)pn * p.nbr + i) * (BR * NP);
