@@ -539,7 +539,8 @@ int trx_batch_destroy(trx_batch_t batch);
  * {"dtype", "buckets": [{"kmax", "nrhs_max", "problems", "sb", "ms": {"4",
  * "8", "16"}}, ...]} in order-major bucket order. The problems' B arrays are
  * overwritten (the batch runs several times): tune on representative
- * scratch data. Synchronises the stream. */
+ * scratch data. Synchronises the stream. FP32: times each bucket and leaves
+ * the table as it is. */
 int trx_batched_autotune(trx_handle_t handle, int elem_bytes, int64_t count,
                          const trx_problem_t* problems, void* stream,
                          char* json, size_t json_len);

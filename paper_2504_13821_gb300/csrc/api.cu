@@ -1337,7 +1337,12 @@ int trx_batched_autotune(trx_handle_t h, int elem_bytes, int64_t count,
     }
     cudaEvent_t e0 = get_event(h), e1 = get_event(h);
     for (int bkt = 0; bkt < NB; ++bkt) {
+        // (the FP32 kernel has one height: timed once, its table stays as it is)
         for (int v = 0; v < 3; ++v) {
+            if (elem_bytes == 4 && v > 0) {
+                all_ms[bkt][v] = all_ms[bkt][0];
+                continue;
+            }
             int ov[NB];
             for (int b = 0; b < NB; ++b) ov[b] = sbs[v];
             std::vector<BatchDesc> all, mine;
@@ -1361,7 +1366,7 @@ int trx_batched_autotune(trx_handle_t h, int elem_bytes, int64_t count,
                 if (rep > 0) ms_sum += ms;   // first run warms up
             }
             all_ms[bkt][v] = ms_sum / 3.0;
-            if (all_ms[bkt][v] < best_ms[bkt]) {
+            if (elem_bytes == 8 && all_ms[bkt][v] < best_ms[bkt]) {
                 best_ms[bkt] = all_ms[bkt][v];
                 best[bkt] = sbs[v];
             }
