@@ -450,7 +450,8 @@ struct Exec {
                     }
                     if (st.trsm)
                         e = launch_thin_trsm(tc, (float)st.alpha, thin_scratch, invz, same_a,
-                                             h->d_err, h->wait_ns, s, h->opt_test_withhold != 0);
+                                             h->d_err, h->wait_ns, h->num_sms, s,
+                                             h->opt_test_withhold != 0);
                     else
                         e = launch_thin_trmm(tc, (float)st.alpha, thin_scratch, h->num_sms, s);
                     if (e == cudaSuccess && st.b > 0 && st.planes && st.r0 + st.b < c.k)

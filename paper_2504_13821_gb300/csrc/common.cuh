@@ -403,8 +403,8 @@ cudaError_t launch_thin_prep(const Canon<float>& c, float* invz, cudaStream_t s)
 // withhold: test hook, block row 0 is never published, so the bounded waits
 // of the blocks after it run out (TRX_ERR_TIMEOUT).
 cudaError_t launch_thin_trsm(const Canon<float>& c, float alpha, int* scratch, const float* invz,
-                             bool made, int* err, long long wait_ns, cudaStream_t s,
-                             bool withhold = false);
+                             bool made, int* err, long long wait_ns, int num_sms,
+                             cudaStream_t s, bool withhold = false);
 // The thin TRMM (thin.cu): C := alpha M C in one launch after a packing
 // pass of C's original rows (no waits); scratch: thin_trmm_scratch_bytes.
 size_t thin_trmm_scratch_bytes(int64_t k, int64_t nrhs);

@@ -966,12 +966,13 @@ size_t thin_scratch_bytes(int64_t k, int64_t nrhs) {
 }
 
 // Two clusters fit the same SMs, where each would stage M at half the rate: from
-// kSpreadRows block rows on, launches of at most kSpread CTAs (two clusters of eight SMs
-// in each part of the chip) ask for more shared memory than two have room for. us,
+// kSpreadRows block rows on, launches that leave a few SMs over (16 of 19 taken: 128 CTAs
+// on 152 SMs, whose parts do not divide into clusters of eight evenly) ask for more shared
+// memory than two have room for. us,
 // without / with: 8191 x 16 transposed 281 / 230, 8192 x 16 228 / 208, 4096 x 32 131 /
 // 117, 2048 x 64 73 / 69, 4096 x 16 115 / 114; but 1024 x 128 48 / 54, 512 x 256 36 / 46
 // (the SMs change their split of shared memory between the launches of a call).
-constexpr int64_t kSpread = 128, kSpreadRows = 32;
+constexpr int64_t kSpreadRows = 32;
 static int g_thin_trmm_ctas_per_sm = 0;
 
 cudaError_t thin_configure() {
@@ -1018,8 +1019,8 @@ cudaError_t launch_thin_prep(const Canon<float>& c, float* invz, cudaStream_t s)
 }
 
 cudaError_t launch_thin_trsm(const Canon<float>& c, float alpha, int* scratch, const float* invz,
-                             bool made, int* err, long long wait_ns, cudaStream_t s,
-                             bool withhold) {
+                             bool made, int* err, long long wait_ns, int num_sms,
+                             cudaStream_t s, bool withhold) {
     if (c.k <= 0 || c.nrhs <= 0) return cudaSuccess;
     const int64_t nbr = (c.k + kThinBlock - 1) / kThinBlock;
     const int64_t npan = (c.nrhs + kThinPanel - 1) / kThinPanel;
@@ -1044,8 +1045,8 @@ cudaError_t launch_thin_trsm(const Canon<float>& c, float alpha, int* scratch, c
     p.invz = invz;
     const int64_t clusters = (nbr + thin::CL - 1) / thin::CL * npan;
     // a long chain on few enough CTAs for an SM each: shared memory for one
-    const size_t smem = nbr >= kSpreadRows && clusters * thin::CL <= kSpread ? thin::kAlone
-                                                                             : sizeof(thin::Smem);
+    const bool spread = nbr >= kSpreadRows && clusters * thin::CL * 19 <= (int64_t)num_sms * 16;
+    const size_t smem = spread ? thin::kAlone : sizeof(thin::Smem);
     thin::thin_trsm_kernel<<<(unsigned)(clusters * thin::CL), thin::NT + thin::NTP, smem, s>>>(p);
     return cudaGetLastError();
 }
