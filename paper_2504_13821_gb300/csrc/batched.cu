@@ -35,7 +35,8 @@ cudaError_t launch_batched_f32(const BatchDesc* descs, int64_t count, int* count
 
 namespace {
 
-template <typename T>
+using T = double;
+
 struct BShape {
     static constexpr int NT = 256;
     static constexpr int NC = kBatchF64Chunk;              // columns per chunk
@@ -48,15 +49,14 @@ struct BShape {
         sizeof(T) * ((size_t)kBatchOrder * LDC + kBatchOrder + 2 * SBMAX * SBMAX);
 };
 
-template <typename T>
 __device__ __forceinline__ T ldA(const T* A, int64_t i, int64_t l, int64_t rs, int64_t cs) {
     return __ldg(A + i * rs + l * cs);
 }
 
-template <typename T, int SB>
+template <int SB>
 __device__ __forceinline__ void trsm_chunk(const BatchDesc& d, T* sC, const T* sD, T* sTile,
                                            int k) {
-    using S = BShape<T>;
+    using S = BShape;
     static_assert(SB <= S::SBMAX, "substitution block above the staged tile size");
     const int tid = threadIdx.x;
     const T* A = static_cast<const T*>(d.A);
@@ -140,10 +140,9 @@ __device__ __forceinline__ void trsm_chunk(const BatchDesc& d, T* sC, const T* s
 // TRMM out of place: the chunk's original columns stay in shared memory and
 // every row's new value alpha * sum_{l <= i} M(i,l) C(l,:) goes straight to
 // global memory, each thread a tile of 4 rows x 4 columns.
-template <typename T>
 __device__ __forceinline__ void trmm_chunk(const BatchDesc& d, const T* sC, const T* sD, int k, T alpha,
                            T* C, int64_t c0, int ncols) {
-    using S = BShape<T>;
+    using S = BShape;
     const int tid = threadIdx.x;
     const T* A = static_cast<const T*>(d.A);
     const int cg = tid % S::CG, rg = tid / S::CG;
@@ -184,10 +183,9 @@ __device__ __forceinline__ void trmm_chunk(const BatchDesc& d, const T* sC, cons
     }
 }
 
-template <typename T>
 __global__ void __launch_bounds__(256, 3) batched_kernel(const BatchDesc* descs, int64_t count,
                                                       int* counter) {
-    using S = BShape<T>;
+    using S = BShape;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* sC = reinterpret_cast<T*>(smem_raw);         // panel: row i, column c at i*LDC + c
     T* sD = sC + (size_t)kBatchOrder * S::LDC;         // reciprocal (TRSM) or plain (TRMM) diagonal
@@ -244,15 +242,15 @@ __global__ void __launch_bounds__(256, 3) batched_kernel(const BatchDesc* descs,
             }
             __syncthreads();
             if (d.trsm) {
-                if (d.sb == 4) trsm_chunk<T, 4>(d, sC, sD, sTile, k);
-                else if (d.sb == 8) trsm_chunk<T, 8>(d, sC, sD, sTile, k);
-                else trsm_chunk<T, 16>(d, sC, sD, sTile, k);
+                if (d.sb == 4) trsm_chunk<4>(d, sC, sD, sTile, k);
+                else if (d.sb == 8) trsm_chunk<8>(d, sC, sD, sTile, k);
+                else trsm_chunk<16>(d, sC, sD, sTile, k);
                 for (int e = tid; e < k * S::NC; e += S::NT) {
                     const int i = row_fast ? e % k : e / S::NC, c = row_fast ? e / k : e % S::NC;
                     if (c < ncols) C[i * d.c_rs + (c0 + c) * d.c_cs] = sC[i * S::LDC + c];
                 }
             } else {
-                trmm_chunk<T>(d, sC, sD, k, (T)d.alpha, C, c0, ncols);
+                trmm_chunk(d, sC, sD, k, (T)d.alpha, C, c0, ncols);
             }
             __syncthreads();
         }
@@ -264,8 +262,8 @@ __global__ void __launch_bounds__(256, 3) batched_kernel(const BatchDesc* descs,
 cudaError_t batched_configure() {
     cudaError_t e = batched_f32_configure();
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(batched_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)BShape<double>::smem);
+    return cudaFuncSetAttribute(batched_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)BShape::smem);
 }
 
 // Resident CTAs per SM of the batched kernel (occupancy query, at least 1).
@@ -273,7 +271,7 @@ int batched_ctas_per_sm(int elem_bytes) {
     if (elem_bytes == 4) return batched_f32_ctas_per_sm();
     int n = 0;
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &n, batched_kernel<double>, BShape<double>::NT, BShape<double>::smem);
+        &n, batched_kernel, BShape::NT, BShape::smem);
     return (e == cudaSuccess && n > 0) ? n : 1;
 }
 
@@ -287,7 +285,7 @@ cudaError_t launch_batched(int elem_bytes, const BatchDesc* descs, int64_t count
     const int grid = (int)std::min<int64_t>(grid_ctas, count);
     if (elem_bytes == 4)
         return launch_batched_f32(descs, count, counter, grid, s);
-    return launch_kernel(batched_kernel<double>, dim3(grid), dim3(256), BShape<double>::smem, s,
+    return launch_kernel(batched_kernel, dim3(grid), dim3(256), BShape::smem, s,
                          descs, count, counter);
 }
 

@@ -205,23 +205,28 @@ __global__ void __launch_bounds__(256, B == 64 ? 2 : 1) leaf_trsm_blocked_kernel
 
 template <typename T>
 cudaError_t leaf_blocked_configure() {
-    cudaError_t e = cudaFuncSetAttribute(leaf_trsm_blocked_kernel<T, 64>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)BlkShape<T, 64>::smem);
-    if (e != cudaSuccess) return e;
+    if constexpr (sizeof(T) == 4) {
+        cudaError_t e = cudaFuncSetAttribute(leaf_trsm_blocked_kernel<T, 64>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)BlkShape<T, 64>::smem);
+        if (e != cudaSuccess) return e;
+    }
     return cudaFuncSetAttribute(leaf_trsm_blocked_kernel<T, 128>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)BlkShape<T, 128>::smem);
 }
 
-// One leaf (a.r0, a.b rows, a.b <= 128), persistent CTAs over the panels.
+// One leaf (a.r0, a.b rows, a.b <= 128; FP64 above 64, leaf_f64.cu has the shorter
+// ones), persistent CTAs over the panels.
 template <typename T>
 cudaError_t leaf_blocked_launch(const LeafArgs<T>& a, int64_t max_ctas, cudaStream_t s) {
     const int64_t npanels = (a.p.nrhs + 63) / 64;
     const int64_t nx = npanels < max_ctas ? npanels : max_ctas;
-    if (a.b <= 64)
-        return launch_kernel(leaf_trsm_blocked_kernel<T, 64>, dim3((unsigned)nx), dim3(256),
-                             BlkShape<T, 64>::smem, s, a);
+    if constexpr (sizeof(T) == 4) {
+        if (a.b <= 64)
+            return launch_kernel(leaf_trsm_blocked_kernel<T, 64>, dim3((unsigned)nx), dim3(256),
+                                 BlkShape<T, 64>::smem, s, a);
+    }
     return launch_kernel(leaf_trsm_blocked_kernel<T, 128>, dim3((unsigned)nx), dim3(256),
                          BlkShape<T, 128>::smem, s, a);
 }

@@ -89,7 +89,7 @@ struct Params {
     float alpha;
     int unit;
     int nbr, npan;
-    int64_t ntask;
+    int64_t ntask;   // TRMM: tasks in all
     int* ticket;     // next task
     int* stop;       // set by a CTA whose wait ran out: the others stop waiting
     // published blocks: X_ip as 64 x 16 tagged words (FP32 bits, tag 1 in
@@ -1026,7 +1026,6 @@ cudaError_t launch_thin_trsm(const Canon<float>& c, float alpha, int* scratch, c
     const int64_t npan = (c.nrhs + kThinPanel - 1) / kThinPanel;
     if (nbr * npan > (int64_t)1 << 30) return cudaErrorInvalidValue;
     thin::Params p = thin_params(c, alpha);
-    p.ntask = nbr * npan;
     p.ticket = scratch;
     p.stop = scratch + 1;
     p.xt = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(scratch) + 16);
