@@ -224,8 +224,8 @@ def run_reference(args):
 
 
 # automatic cutoffs of the library for this workload (FP32, 16384 right-hand
-# sides): TRSM 128-row leaves (wide leaf kernel), TRMM 1024-row diagonal blocks
-# on the tensor cores; --leaf overrides both
+# sides): TRSM 128-row leaves (wide leaf kernel), TRMM in one launch by 128-row
+# tiles on the tensor cores; --leaf overrides both
 # (FP64: 64-row leaves)
 LEAF_USED = None
 
@@ -246,7 +246,9 @@ def auto_path_desc(k, n):
     if k > 256 and n <= 32:
         trmm = "TRMM as one thin product"
     else:
-        trmm = "TRMM 1024-row diagonal blocks on the tensor cores" if k >= 1024 else "TRMM 64"
+        trmm = ("TRMM 64" if k < 256 else
+                "TRMM in one launch by 128-row tiles on the tensor cores" if SPLIT_TERMS == 6 else
+                "TRMM 1024-row diagonal blocks on the tensor cores" if k >= 1024 else "TRMM 64")
     return f"{trsm}, {trmm}"
 
 
@@ -309,7 +311,8 @@ def run_gpu(args):
     if args.tc_leaf:
         h.set_option(trx.OPT_TRSM_TC_LEAF, 1)
         LEAF_USED = (f"TRSM {args.leaf or 128} as inverse GEMMs on the tensor cores, "
-                     "TRMM 1024-row diagonal blocks on the tensor cores")
+                     + ("TRMM 64" if args.leaf else
+                        "TRMM in one launch by 128-row tiles on the tensor cores"))
     stream = torch.cuda.current_stream(dev)
     # FP32: the factor's operand planes are made once per step (update), then
     # the TRSM and the TRMM both use them. FP64 has no planes: plain calls.

@@ -15,7 +15,7 @@
 // What bounds it: the chain of a chunk's blocks (one of order 512 and 32 columns alone
 // on the GPU takes 2.2 us per block: 0.9 for the columns of M to arrive, 0.6 for the
 // substitution, 1.2 for the update, in part at once), which two CTAs per SM hide in
-// part; FMA issue is at 30 %. 4096 problems of order 16..512 with 1..64 right-hand
+// part; the FMA pipe is 27 % active. 4096 problems of order 16..512 with 1..64 right-hand
 // sides: 955 us with the kernel before it (M read four scalar loads to 16 FMAs through
 // L1, 32 columns only, a CTA a problem, FMA pipe 20 % active), 491 with this one
 // (1000 problems: 673 -> 164, 200: 361 -> 84).

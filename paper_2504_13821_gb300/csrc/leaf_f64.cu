@@ -13,7 +13,7 @@
 // at 4096 right-hand sides.
 //
 // Measured, one 64-row leaf (us by right-hand sides, that kernel / this one, ncu):
-// 1024 47 / 17, 1500 48 / 21, 4096 54 / 29; four lanes per column took 20 (1024)
+// 1024 47 / 17, 1500 48 / 21, 4096 54 / 29 (30 with the products summed first); four lanes per column took 20 (1024)
 // and 29 (4096), 32 columns per CTA 34 (4096). Up to 1024 right-hand sides
 // leaf256_kernel below serves.
 #include "common.cuh"

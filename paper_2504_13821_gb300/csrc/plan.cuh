@@ -464,8 +464,9 @@ inline int thin_leaf_rows(int64_t opt, bool tc, bool trsm, int elem, int64_t k, 
 // the canonical order, so a reversed problem's rows run forwards too). The two
 // passes cost 16 bytes an element. Measured (us, nrhs x order, in place / turned):
 // TRSM 256 x 256 53 / 51, 600 x 300 58 / 52, 600 x 600 148 / 123, 2000 x 2000 628 /
-// 441, 4096 x 4096 1343 / 945, 8192 x 8192 5375 / 3813; TRMM 500 x 300 31 / 31,
-// 1000 x 1000 56 / 42, 3000 x 5000 609 / 432. Below 2^16 elements nothing is gained.
+// 441, 4096 x 4096 1343 / 945, 8192 x 8192 5375 / 3813; TRMM 500 x 300 29-33 either
+// way (six processes each, which differ more than that from day to day), 1000 x 1000
+// 56 / 42, 3000 x 5000 609 / 432. Below 2^16 elements nothing is gained.
 constexpr int64_t kTurnMinElements = (int64_t)1 << 16;
 inline bool turn_applies(int64_t k, int64_t nrhs) {
     return k * nrhs >= kTurnMinElements && k <= 64 * 65535ll && nrhs <= 64 * 65535ll;
@@ -502,8 +503,10 @@ inline size_t oz_workspace(int64_t gemm_mode, int64_t k, int64_t nrhs, int b) {
 // the recursion's leaves and updates: from two leaves on (one leaf is one launch).
 // Measured (us, order x right-hand sides, recursion with DFMA / one product): 100 x
 // 100 43 / 43 (both the recursion), 128 x 16 42 / 31, 256 x 200 90 / 32, 1000 x 16
-// 396 / 69, 1000 x 200 495 / 79, 8192 x 100 10437 / 722, 4096 x 4096 59618 / 1985;
-// side R 1500 x 2500 6308 / 392.
+// 396 / 69, 1000 x 200 495 / 79, 8192 x 100 10437 / 722, 4096 x 4096 59618 / 2050;
+// side R 1500 x 2500 6308 / 445-485 (data with pieces left to DFMA). Where DFMA takes
+// all pieces (columns graded over e^40) the attempt costs up to 3 %: 1024 x 1024 1203 /
+// 1239, 4096 x 4096 59672 / 59936, but 1000 x 200 497 / 318.
 inline bool oz_trmm_applies(int64_t gemm_mode, int64_t k, int64_t nrhs) {
     return gemm_mode != 1 && k >= 128 && nrhs >= 1;
 }

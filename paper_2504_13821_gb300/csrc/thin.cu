@@ -23,7 +23,7 @@
 // panel, the dominant traffic) overlap the chain of diagonal blocks; the
 // chain itself is one 64 x 64 x 16 product per block.
 //
-// The same launch also serves as the recursion's leaf for 65 .. 1024
+// The same launch also serves as the recursion's leaf for 65 .. 1536
 // right-hand sides (the thin leaves): on a leaf's rows, its columns of M
 // and its rows of C, with the tensor-core updates between leaves.
 //
@@ -40,7 +40,7 @@
 // three products (its last tile, the inverse, Z) of 0.5-0.67 us each in two steps.
 // us, this kernel against one CTA per ticket that published through L2 only, staged M
 // between its products and had a thread on 4 rows x 1 column: 8191 x 16 transposed
-// 323 -> 230, 8192 x 16 323 -> 208, 8192 x 64 449 -> 316, a 2048-row leaf with 256
+// 323 -> 225, 8192 x 16 323 -> 208, 8192 x 64 449 -> 316, a 2048-row leaf with 256
 // right-hand sides 121 -> 87. On the way: the products alone 309, clusters with M
 // still staged between them 283.
 //
