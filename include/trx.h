@@ -102,7 +102,8 @@ enum {
                               FP32 accumulation). FP64 updates: 1 keeps all
                               of them on the CUDA cores (DFMA); 0 and 2 take
                               the larger ones to the tensor cores where the
-                              workspace allows (64-bit fixed-point rows in
+                              workspace allows and the call is not captured
+                              into a caller's graph (64-bit fixed-point rows in
                               eight BF16 digits, exact integer sums: error
                               below 8 u |op(A)||B| per element, elements
                               that cannot hold it computed by DFMA)        */
@@ -321,8 +322,9 @@ int trx_set_workspace(trx_handle_t handle, void* ptr, size_t bytes);
  * on the mixed engine, TRX_OPT_FP64_TRSM, needs the FP32 solve's). For side R
  * on the FP32 tensor-core path it includes room for B's transpose, and for TRMM
  * there a word per 128 rows and right-hand side for the Infs and NaNs of B, without
- * which the call still runs, more slowly. For the recursive FP64 calls it is what their updates on the tensor cores use; with
- * less the call runs all its updates on the CUDA cores instead.
+ * which the call still runs, more slowly. For the recursive FP64 calls it is what
+ * their updates on the tensor cores use; with less, or under a stream capture, the
+ * call runs all its updates on the CUDA cores instead.
  * Returns 0 and sets *bytes, or an argument code as for the compute calls. */
 int trx_workspace_size(trx_handle_t handle, char op, char side, int64_t m,
                        int64_t n, int elem_bytes, size_t* bytes);

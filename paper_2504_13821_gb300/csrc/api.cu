@@ -242,6 +242,8 @@ struct trx_handle_s {
     int64_t opt_thin_leaf = 0;       // TRSM leaves as thin solves (TRX_OPT_THIN_LEAF)
     int64_t opt_test_withhold = 0;   // test hook (TRX_OPT_TEST_WITHHOLD)
     int* thin_buf = nullptr;
+    bool thin_captured = false;    // a captured call uses thin_buf: kept when it grows
+    std::vector<int*> thin_kept;
     size_t thin_bytes = 0;
     cudaStream_t aux[kMaxPanels] = {};
     cudaEvent_t fork_ev = nullptr, join_ev[kMaxPanels] = {};
@@ -630,11 +632,11 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
                              : thin_leaf > 0 ? thin_prep_bytes(k) +
                                                    thin_scratch_bytes(thin_leaf, ex.c.nrhs)
                                              : 0;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    e = cudaStreamIsCapturing(s, &cap);
+    if (e != cudaSuccess) return fail_cuda(e, "cudaStreamIsCapturing");
     if (thin_need > 0 && h->thin_bytes < thin_need) {
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        e = cudaStreamIsCapturing(s, &cs);
-        if (e != cudaSuccess) return fail_cuda(e, "cudaStreamIsCapturing");
-        if (cs != cudaStreamCaptureStatusNone) {
+        if (cap != cudaStreamCaptureStatusNone) {
             thin = false;
             thin_leaf = 0;
             plan.tc = tc_ok;
@@ -642,7 +644,10 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
             const size_t want = std::max<size_t>(2 * thin_need, 1 << 16);
             // cached graphs hold the old buffer's address: dropped with it
             drop_graphs(h);
-            if (h->thin_buf) cudaFree(h->thin_buf);        // waits for its last use
+            // (cudaFree waits for its last use; a captured call's graph has no last one)
+            if (h->thin_captured) h->thin_kept.push_back(h->thin_buf);
+            else if (h->thin_buf) cudaFree(h->thin_buf);
+            h->thin_captured = false;
             h->thin_buf = nullptr;
             h->thin_bytes = 0;
             if ((e = cudaMalloc(&h->thin_buf, want)) != cudaSuccess) {
@@ -653,6 +658,7 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
         }
     }
     ex.thin_scratch = (thin || thin_leaf > 0) ? h->thin_buf : nullptr;
+    if (ex.thin_scratch && cap != cudaStreamCaptureStatusNone) h->thin_captured = true;
     if (thin_leaf > 0) {
         ex.thin_invz = reinterpret_cast<float*>(h->thin_buf);
         ex.thin_scratch += thin_prep_bytes(k) / sizeof(int);
@@ -781,9 +787,10 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
     }
     // FP64: the larger updates on the tensor cores, where the handle's workspace
     // holds their operand images (else the DFMA updates, which need none) and
-    // the call is one chain (column-panel branches would share the images)
+    // the call is one chain (column-panel branches would share the images). Not under a
+    // capture: its graph may run when the workspace has been replaced.
     bool oz_trmm = false;
-    if (std::is_same<T, double>::value && P == 1) {
+    if (std::is_same<T, double>::value && P == 1 && cap == cudaStreamCaptureStatusNone) {
         const auto fits = [&](size_t need) {
             return need > 0 && h->ws != nullptr && h->ws_bytes >= need;
         };
@@ -864,9 +871,6 @@ int execute(trx_handle_t h, bool trsm, char side, char uplo, char transa, char d
         return TRX_SUCCESS;
     };
 
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    e = cudaStreamIsCapturing(s, &cap);
-    if (e != cudaSuccess) return fail_cuda(e, "cudaStreamIsCapturing");
     if (ex.profile || !h->opt_graph || cap != cudaStreamCaptureStatusNone) return run_all(s);
 
     GraphKey key;
@@ -1495,6 +1499,7 @@ int trx_destroy(trx_handle_t h) {
         cudaDeviceSynchronize();
     }
     if (h->thin_buf) cudaFree(h->thin_buf);
+    for (int* p : h->thin_kept) cudaFree(p);
     free_owned_ws(h);
     if (h->d_err) cudaFree(h->d_err);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
