@@ -82,12 +82,13 @@ struct Cfg {
     static constexpr int STAGES =
         (1024 + MAX_STAGES * STAGE_BYTES + 256 <= 227 * 1024) ? MAX_STAGES : 3;
     // One lane waits, issues and commits, and a chunk has one set of accumulators, at
-    // every width. (A form with the whole warp in the issue loop and two sets below
-    // 256 columns is not used: runs with it ended in a memory fault that reading has
-    // not explained.) Below 256 columns the lane is elect.sync's: TRSM 2000 x 2000 side
-    // R 356 us with lane 0, 340 with the elected one; order 4096 with a factor and 256
-    // right-hand sides 232 and 226. At 256 an MMA takes the pipe 128 clocks whoever
-    // issues it, and a denser issue measured 0-2 % slower at the power limit.
+    // every width. (A form with the whole warp in the issue loop and two sets below 256
+    // columns, TRMM 1024 x 1024 32 us against 35 and 2048 x 300 45 against 47.5, is not
+    // used: runs with it ended in a memory fault that reading has not explained.) Below
+    // 256 columns the lane is elect.sync's: TRSM 2000 x 2000 side R 356 us with lane 0,
+    // 340 with the elected one; order 4096 with a factor and 256 right-hand sides 232 and
+    // 226. At 256 an MMA takes the pipe 128 clocks whoever issues it, and a denser issue
+    // measured 0-2 % slower at the power limit.
     static constexpr bool ELECT = BN < 256;
     static constexpr int TMEM_COLS = 2 * BN;
     static constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + 256;
